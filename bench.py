@@ -506,27 +506,21 @@ KERNEL_SOURCES = {
     "grid_rows_dft": [("paper_0812_3669_gb300/csrc/moff_image_kernels.cuh", "struct ColShape"),
                       "paper_0812_3669_gb300/csrc/moff_dft.cuh"],
     "cols_dft": [("paper_0812_3669_gb300/csrc/moff_dft_kernels.cu", "struct ColDftShape",
-                  "template <int N, int P>\nstruct RowDftShape"), "paper_0812_3669_gb300/csrc/moff_dft.cuh"],
-    "rows_dft": [("paper_0812_3669_gb300/csrc/moff_dft_kernels.cu", "template <int N, int P>\nstruct RowDftShape",
-                  "template <int N, int P>\ncudaError_t launch_rows_dft_t"), "paper_0812_3669_gb300/csrc/moff_dft.cuh"],
-    "rows_dft8": [("paper_0812_3669_gb300/csrc/moff_dft_kernels.cu", "template <int P>\nstruct RowDft8Shape",
+                  "cudaError_t launch_cols_dft_t"), "paper_0812_3669_gb300/csrc/moff_dft.cuh"],
+    "rows_dft8": [("paper_0812_3669_gb300/csrc/moff_dft_kernels.cu", "struct RowDft8Shape",
                    "}  // namespace"), "paper_0812_3669_gb300/csrc/moff_dft.cuh"],
     "grid_tc": ["paper_0812_3669_gb300/csrc/moff_gridtc.cu", "paper_0812_3669_gb300/csrc/moff_tc.cuh"],
     "volt_prep": ["paper_0812_3669_gb300/csrc/moff_tc_kernels.cu"],
 }
 # kernel kind (moff_timing) -> its name in KERNEL_SOURCES, per route
 ROUTE_KERNELS = {"fp16_dft": {"grid_rows": "grid_rows_dft", "cols_integrate": "cols_dft"},
-                 "fp16_tcgrid": {"grid_rows": "grid_tc", "row_transform": "rows_dft", "cols_integrate": "cols_dft",
+                 "fp16_tcgrid": {"grid_rows": "grid_tc", "row_transform": "rows_dft8", "cols_integrate": "cols_dft",
                                  "volt_prep": "volt_prep"}}
 
 
 def route_kernel(route, kind, N):
-    """Name (in KERNEL_SOURCES) of the kernel behind a timing kind on a route: the tensor-core
-    gridding route's row transform is the 8 x 64 kernel on the 512 grid (unless MOFF_ROWS8=0)."""
-    k = ROUTE_KERNELS.get(route, {}).get(kind, kind)
-    if k == "rows_dft" and N == 512 and os.environ.get("MOFF_ROWS8", "1") != "0":
-        return "rows_dft8"
-    return k
+    """Name (in KERNEL_SOURCES) of the kernel behind a timing kind on a route."""
+    return ROUTE_KERNELS.get(route, {}).get(kind, kind)
 
 
 def traffic_for(kernel_key, src, units_per_launch=None):

@@ -27,6 +27,7 @@
 #include <cuda_fp16.h>
 
 #include "moff_fft.cuh"
+#include "moff_internal.h"
 #include "moff_tc.cuh"
 
 namespace moff {
@@ -35,6 +36,13 @@ namespace moff {
 __device__ __forceinline__ void cp_async16(void *smem_dst, const void *gmem_src) {
     const unsigned d = (unsigned)__cvta_generic_to_shared(smem_dst);
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(gmem_src) : "memory");
+}
+// The same where `on` is set (shared-memory address given).
+__device__ __forceinline__ void cp_async16_if(uint32_t on, uint32_t smem_dst, const void *gmem_src) {
+    asm volatile(
+        "{\n.reg .pred p;\nsetp.ne.b32 p, %2, 0;\n@p cp.async.cg.shared.global [%0], [%1], 16;\n}\n" ::"r"(smem_dst),
+        "l"(gmem_src), "r"(on)
+        : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 template <int NPEND>
@@ -117,8 +125,8 @@ __device__ __forceinline__ void load_table(unsigned char *dst, const unsigned ch
 
 // Row transform of the F gridded rows of one gridding pass (FP32 in shared
 // memory, row f at src + f * LDR, element e at pad16(e)) on the tensor cores;
-// the FP16 result goes, row f as [re N][im N], to rowout(f) (nullptr: not
-// stored), through a staging copy in `stage` (may alias src: src is read
+// the FP16 result goes to the field (field_offset, moff_internal.h), the row's first
+// piece at rowout(f) (nullptr: not stored), through a staging copy in `stage` (may alias src: src is read
 // first).  All kBlock threads call it; thread 0 issues the MMAs.  sG: the
 // FP16 scale of the field.  `region`: dft_row_region_bytes(N, F) bytes
 // (16-byte aligned) whose table image is already loaded; `mbar` initialised
@@ -247,12 +255,12 @@ __device__ __forceinline__ bool rows_dft(const float2 *src, float sG, unsigned c
     }
     tc::fence_before_sync();
     __syncthreads();
-    // (4) staging -> global rows, 16-byte pieces
+    // (4) staging -> the field, 16-byte pieces (8 columns of one row and part)
     constexpr int PR = N / 8;
     for (int i = tid; i < F * 2 * PR; i += NTHREADS) {
         const int rr = i / PR, pc = i - rr * PR;
         __half *o = rowout(rr >> 1);
-        if (o) *reinterpret_cast<uint4 *>(o + (rr & 1) * N + 8 * pc) =
+        if (o) *reinterpret_cast<uint4 *>(o + field_offset(N, 0, rr & 1, pc)) =
                    *reinterpret_cast<const uint4 *>(stage + rr * SLD + 8 * pc);
     }
     return true;

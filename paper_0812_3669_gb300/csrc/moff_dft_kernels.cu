@@ -49,7 +49,7 @@ struct ColDftShape {
     static constexpr int H = W / 8;                    // 16-byte pieces per (pol, row, re/im) of the strip
     static constexpr int M1 = W * N2;                  // stage-1 rows per pol: m = W b + x
     static constexpr int T1 = M1 / 128;
-    static constexpr int LBO1 = (M1 / 8) * 128;        // stage-1 A: K-direction core-matrix stride
+    static constexpr int MH = S::K1 * 128;             // stage-1 A: bytes of 64 rows m (128-byte swizzled)
     static constexpr int A1P = M1 * S::K1 * 2;         // bytes of one pol's stage-1 A
     static constexpr int M2 = 16 * W;                  // stage-2 rows per pol: m2 = 8 W c_hi + 8 x + c_lo
     static constexpr int T2 = M2 / 128;
@@ -100,27 +100,25 @@ __global__ void __launch_bounds__(kBlock, ColDftShape<N, P, W>::MINB) k_cols_dft
         tc::tmem_alloc(tslot, CS::TCOLS);
         tc::tmem_relinquish();
     }
-    // Piece i = k kBlock + tid of a sample: pol p, row ry, re/im ri, column piece h (i = ((p N + ry) 2
-    // + ri) H + h).  With kBlock a divisor of 2 H N, k fixes p and ry's multiple of ROWS_K (PK, RYK
-    // below, compile-time) and the thread fixes ry mod ROWS_K = r0, ri and h: every offset is a thread
-    // constant plus a compile-time one.  In the stage-1 operand the piece is the 8 rows m = W b + 8 h
-    // + (0..7) at k = 2 a + ri (ry = N2 a + b).  Rows no kernel reaches are zero: cleared once in both
+    // Piece i = k kBlock + tid of a sample: pol p, row ry, re/im ri, column piece h (16 bytes = 8 columns).  With
+    // kBlock a divisor of 2 H N, k fixes p and ry's multiple of ROWS_K (PK, RYK below, compile-time) and the
+    // thread fixes ry mod ROWS_K = r0, ri and h, consecutive lanes consecutive rows.  In the stage-1 operand (128-byte swizzle) the piece is the 8 rows
+    // m = W b + 8 h + (0..7) at k = 2 a + ri (ry = N2 a + b): eight consecutive b share 128 bytes, so the copies'
+    // shared-memory writes meet no bank conflict either.  Rows no kernel reaches are zero: cleared once in both
     // buffers and never loaded.
-    const int h0 = tid % H, ri0 = (tid / H) & 1, r0 = tid / (2 * H);
+    const int r0 = tid % CS::ROWS_K, ri0 = (tid / CS::ROWS_K) & 1, h0 = tid / (2 * CS::ROWS_K);
     const int a0 = r0 / N2, b0 = r0 - a0 * N2, kt = 2 * a0 + ri0;
-    // 2 a = 2 (RYK / N2) + 2 a0: the compile-time part is a multiple of 8 when ROWS_K is one of 4 N2,
-    // else (16 columns at N = 512) kt and the compile-time part share one core-matrix row group
-    constexpr bool KSPLIT8 = CS::ROWS_K % (4 * N2) == 0;
-    const uint32_t dst_t = (uint32_t)((H * b0 + h0) * 128) +
-                           (KSPLIT8 ? (uint32_t)((kt >> 3) * CS::LBO1 + (kt & 7) * 16) : (uint32_t)(kt * 16));
-    const long long src_t = (long long)(2 * r0 + ri0) * N + x0 + 8 * h0;
+    const int cg0 = (H * b0 + h0) & 7, mh0 = (H * b0 + h0) >> 3;
+    const uint32_t dst_t = (uint32_t)(mh0 * CS::MH + kt * 128 + ((cg0 ^ (kt & 7)) << 4));
+    const int src_t = field_offset(N, r0, ri0, blockIdx.x * H + h0);
     auto piece_dst = [&](int k) -> uint32_t {      // k compile-time after unrolling
         const int PK = (k * kBlock) / (2 * H * N), RYK = ((k * kBlock) % (2 * H * N)) / (2 * H), AK = RYK / N2;
-        return (uint32_t)(PK * CS::A1P + ((2 * AK) >> 3) * CS::LBO1 + ((2 * AK) & 7) * 16) + dst_t;
+        // 2 AK is a multiple of 8 but for 16 columns at N = 512, where it flips bit 2 of the swizzle (kt < 4 there)
+        return (uint32_t)(PK * CS::A1P + 2 * AK * 128) + (dst_t ^ (uint32_t)(((2 * AK) & 4) << 4));
     };
     auto piece_src = [&](int k) -> long long {
         const int PK = (k * kBlock) / (2 * H * N), RYK = ((k * kBlock) % (2 * H * N)) / (2 * H);
-        return (long long)(PK * N + RYK) * 2 * N + src_t;
+        return (long long)PK * N * 2 * N + RYK * 2 * N + src_t;
     };
     uint32_t act = 0;
 #pragma unroll
@@ -158,7 +156,7 @@ __global__ void __launch_bounds__(kBlock, ColDftShape<N, P, W>::MINB) k_cols_dft
 #pragma unroll
                 for (int ks = 0; ks < 2; ++ks)
                     tc::mma_f16(tbase + (uint32_t)((p * CS::T1 + j) * S::C1),
-                                tc::smem_desc(a0 + p * CS::A1P + j * 2048 + ks * 2 * CS::LBO1, CS::LBO1, 128),
+                                tc::smem_desc_sw128(a0 + p * CS::A1P + j * 2 * CS::MH + ks * 2048, CS::MH, 1024),
                                 tc::smem_desc(b0 + ks * 256, 128, 512), id1, ks > 0);
         tc::mma_commit(&mbar[0]);
     };
@@ -308,244 +306,361 @@ __global__ void __launch_bounds__(kBlock, ColDftShape<N, P, W>::MINB) k_cols_dft
 }
 
 // ---------------------------------------------------------------------------------------------
-// Row transform of a gridded field that is already in global memory (FP16 rows [re N][im N],
-// written by the tensor-core gridding): one CTA = a stripe of RS grid rows (both pols) of one
-// channel walking a chunk of samples.  Per sample the F = P RS rows land by 16-byte cp.async
-// pieces as the stage-1 A operand, MN-major (row m = f N2 + b, k = 2 a + re/im: each piece is 8
-// consecutive b of one (f, a, re/im)); pieces of cells no tile reaches are zero, cleared once.
-// Stage 1, twiddle, stage 2 and the FP16 store of the row-transformed rows as in the gridding
-// kernel's row transform; loads of sample t + 1 and stage 1 of sample t overlap the epilogue of
-// sample t - 1.
-template <int N, int P>
-struct RowDftShape {
+// The column kernel as a pipeline of roles (one CTA per SM).  k_cols_dft's per-sample chain -- stage 1,
+// twiddle, barrier, stage 2, square and sum, barrier -- left the SM waiting for MMA and TMEM latencies (issue 32 %,
+// DRAM 26 % with two such CTAs per SM).  Here each step has warps of its own and hands over through
+// mbarriers, every accumulator and operand double-buffered (all 512 TMEM columns for two pols), so the steps of
+// neighbouring samples overlap:
+//   warps 0-7    twiddle stage 1's result (their 16 twiddles stay in registers: a thread keeps its b for every
+//                sample) and write the stage-2 operand
+//   warps 8-15   square and sum stage 2's result in registers; at the end fold into the FP64 accumulators
+//   warps 16, 19 cp.async of the strip into a ring of kCpStages samples (32 rows x 16 bytes per instruction; the
+//                swizzled operand's writes are conflict-free)
+//   warps 17, 18 issue the MMAs of stage 1 and of stage 2 (one elected lane each)
+// The arithmetic and the order of each pixel's sums are k_cols_dft's, so the images are bit-identical.
+// Measured (two pols; k_cols_dft with 8 columns -> this): 512 grid, 24 channels x 250 samples of 16384 antennas 3599 ->
+// 2660 us; 256 grid, 96 x 333 of 4096 antennas 4796 -> 3521 us.  About 1600 cycles per sample and SM, against 2660
+// before; no role waits long on one other: shared-memory traffic (about 1100 of them) binds next.
+// Every wait is bounded (shared abort flag); the status word is set and every role unwinds.
+constexpr int kCpThreads = 20 * 32;   // whole warpgroups (register shares below); 
+constexpr int kCpStages = 4;
+
+// Register shares of the warpgroups (launched with 96 a thread, 640 threads: 61,440): 2 x 128 threads squaring at
+// 128, 2 x 128 twiddling at 88, 128 at 40 = 60,416, so every increase is covered by the decreases.
+constexpr int kCpRegsSquare = 128, kCpRegsTwiddle = 88, kCpRegsIssue = 40;
+static_assert(256 * kCpRegsSquare + 256 * kCpRegsTwiddle + 128 * kCpRegsIssue <= kCpThreads * 96, "register shares");
+template <int R>
+__device__ __forceinline__ void regs_dec() { asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;\n" ::"n"(R)); }
+template <int R>
+__device__ __forceinline__ void regs_inc() { asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;\n" ::"n"(R)); }
+
+// *a += s v, with s a power of two, without the FP64 pipe (two operations a cycle and SM): the product's bits are put
+// together from v's and the addition is left to L2 (a reduction without return; one owner per element, so the sum
+// is that of a load, add and store).  Values whose product is subnormal, infinite or NaN take the plain path.
+__device__ __forceinline__ void red_scaled(double *a, float v, int scale_exp, double s) {
+    const uint32_t u = __float_as_uint(v);
+    const int e = (int)((u >> 23) & 255u);
+    double d;
+    if (e != 0 && e != 255) {
+        const uint32_t m = u & 0x7FFFFFu;
+        d = __hiloint2double((int)((u & 0x80000000u) | ((uint32_t)(e + 896 + scale_exp) << 20) | (m >> 3)), (int)(m << 29));
+    } else if ((u << 1) == 0u) {
+        return;                                                  // adding zero
+    } else {
+        d = (double)v * s;
+    }
+    atomicAdd(a, d);
+}
+
+template <int N, int P, int W>
+struct ColPipeShape {
     using S = DftShape<N>;
-    static constexpr int RS = 8 / P;                    // grid rows per stripe (8 transform rows, inside one tile band)
-    static constexpr int F = P * RS;                    // transform rows per sample, f = p RS + rl
-    static constexpr int N2 = S::N2;
-    static constexpr int M1 = F * N2, T1 = M1 / 128;    // stage-1 rows (f, b)
-    static constexpr int LBO1 = (M1 / 8) * 128;
-    static constexpr int A1B = M1 * S::K1 * 2;
-    static constexpr int M2 = 16 * F, T2 = M2 / 128;    // stage-2 rows (f, c)
-    static constexpr int LBO2 = (M2 / 8) * 128;
-    static constexpr int A2B = M2 * S::K2 * 2;
-    static constexpr int D1 = T1 * S::C1, D2 = T2 * S::C2;
-    static constexpr int TC_ = D1 + D2;
-    static constexpr int TCOLS = TC_ <= 32 ? 32 : (TC_ <= 64 ? 64 : (TC_ <= 128 ? 128 : (TC_ <= 256 ? 256 : 512)));
-    static constexpr int NPIECE = F * 16 * 2 * (N2 / 8);   // (f, a, re/im, b8)
-    static constexpr int ITER = NPIECE / kBlock;
-    static constexpr size_t SMEM = 16 + 2 * (size_t)A1B + A2B + S::TAB_BYTES + 32;
-    static_assert(M1 % 128 == 0 && M2 % 128 == 0 && NPIECE % kBlock == 0 && ITER <= 32, "row-transform shape");
+    using CS = ColDftShape<N, P, W>;
+    static constexpr int D1 = P * CS::T1 * S::C1, D2 = P * CS::T2 * S::C2;   // TMEM columns of one buffer
+    static constexpr int TC_ = 2 * (D1 + D2);
+    static constexpr int TCOLS = TC_ <= 128 ? 128 : (TC_ <= 256 ? 256 : 512);
+    static constexpr int A1 = P * CS::A1P, A2 = P * CS::A2P;                  // operand bytes of one sample
+    static constexpr int TAB = S::B1_BYTES + S::B2_BYTES;                     // twiddles go to registers
+    static constexpr int NBAR = 2 * kCpStages + 12;
+    static constexpr size_t SMEM = 1024 + (size_t)kCpStages * A1 + 2 * (size_t)A2 + TAB + NBAR * 8 + 16;
+    static_assert(TC_ <= 512 && SMEM <= 227 * 1024 && CS::T1 <= 2, "column pipeline shape");
 };
 
-template <int N, int P>
-__global__ void __launch_bounds__(kBlock) k_rows_dft(const RowDftArgs a) {
+template <int N, int P, int W>
+__global__ void __launch_bounds__(kCpThreads, 1) k_cols_pipe(const ColDftArgs a) {
     using S = DftShape<N>;
-    using RD = RowDftShape<N, P>;
-    constexpr int N2 = S::N2, K2 = S::K2, C2 = S::C2, F = RD::F, RS = RD::RS;
-    const int s = blockIdx.x, cl = blockIdx.y, c = a.c0 + cl;
+    using CS = ColDftShape<N, P, W>;
+    using CP = ColPipeShape<N, P, W>;
+    constexpr int N2 = S::N2, K2 = S::K2, C2 = S::C2, H = CS::H, ND = CS::ND;
+    constexpr int NPROD = P == 1 ? 1 : 4;
+    const int x0 = blockIdx.x * W, cl = blockIdx.y, c = a.c0 + cl;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, q = warp & 3;
-    const int ry0 = s * RS;
-    {   // stripes no kernel reaches carry no field: nothing to transform or store
-        bool any = false;
-        for (int rl = 0; rl < RS; ++rl) any |= ((a.row_nz[(ry0 + rl) >> 5] >> ((ry0 + rl) & 31)) & 1u) != 0;
-        if (!any) return;
-    }
-    (void)c;
-    extern __shared__ __align__(16) unsigned char smem[];
-    unsigned char *sA1 = smem;                                   // [2][A1B]
-    unsigned char *sA2 = sA1 + 2 * RD::A1B;
-    unsigned char *sTab = sA2 + RD::A2B;
-    const unsigned char *sB1 = sTab, *sB2 = sTab + S::B1_BYTES;
-    const float2 *sTw = reinterpret_cast<const float2 *>(sB2 + S::B2_BYTES);
-    uint64_t *mbar = reinterpret_cast<uint64_t *>(sTab + S::TAB_BYTES);
-    uint32_t *tslot = reinterpret_cast<uint32_t *>(mbar + 2);
 
-    dftc::load_table(sTab, a.dft_tab, S::TAB_BYTES);
+    extern __shared__ __align__(1024) unsigned char smem_raw[];
+    unsigned char *smem = smem_raw + ((1024u - (tc::smem_u32(smem_raw) & 1023u)) & 1023u);
+    unsigned char *sA1 = smem;                                   // [kCpStages][P][A1P]
+    unsigned char *sA2 = sA1 + kCpStages * CP::A1;               // [2][P][A2P]
+    unsigned char *sB1 = sA2 + 2 * CP::A2, *sB2 = sB1 + S::B1_BYTES;
+    uint64_t *bars = reinterpret_cast<uint64_t *>(sB1 + CP::TAB);
+    uint64_t *full = bars, *empty = full + kCpStages;            // strip ring
+    uint64_t *d1_full = empty + kCpStages, *d1_empty = d1_full + 2, *a2_full = d1_full + 4, *a2_empty = d1_full + 6,
+             *d2_full = d1_full + 8, *d2_empty = d1_full + 10;
+    uint32_t *tslot = reinterpret_cast<uint32_t *>(bars + CP::NBAR);
+    volatile int *abort_flag = reinterpret_cast<volatile int *>(tslot + 1);
+
+    dftc::load_table(sB1, a.dft_tab, CP::TAB);
     if (tid == 0) {
-        tc::mbar_init(&mbar[0], 1);
-        tc::mbar_init(&mbar[1], 1);
+        for (int s = 0; s < kCpStages; ++s) {
+            tc::mbar_init(&full[s], 2);          // the two producer warps
+            tc::mbar_init(&empty[s], 1);
+        }
+        for (int b = 0; b < 2; ++b) {
+            tc::mbar_init(&d1_full[b], 1);
+            tc::mbar_init(&d1_empty[b], 8);
+            tc::mbar_init(&a2_full[b], 8);
+            tc::mbar_init(&a2_empty[b], 1);
+            tc::mbar_init(&d2_full[b], 1);
+            tc::mbar_init(&d2_empty[b], 8);
+        }
+        *abort_flag = 0;
     }
     if (warp == 0) {
-        tc::tmem_alloc(tslot, RD::TCOLS);
+        tc::tmem_alloc(tslot, CP::TCOLS);
         tc::tmem_relinquish();
     }
-    // Piece i = k kBlock + tid = ((f 16 + aa) 2 + ri) (N2/8) + b8: with 32 (N2/8) a divisor of
-    // kBlock, k fixes f's high part (FK, compile-time) and the thread fixes (f mod FPK, aa, ri, b8).
-    constexpr int B8N = N2 / 8, FPK = kBlock / (32 * B8N);   // rows f per k step
-    static_assert(kBlock % (32 * B8N) == 0, "piece enumeration");
-    const int b8_0 = tid % B8N, ri_0 = (tid / B8N) & 1, aa_0 = (tid / (2 * B8N)) & 15, f_0 = tid / (32 * B8N);
-    auto piece = [&](int k, int &f, int &aa, int &ri, int &b8) {
-        f = k * FPK + f_0;
-        aa = aa_0;
-        ri = ri_0;
-        b8 = b8_0;
-    };
-    auto piece_dst = [&](int f, int aa, int ri, int b8) -> uint32_t {
-        const int k = 2 * aa + ri;
-        return (uint32_t)((f * (N2 / 8) + b8) * 128 + (k >> 3) * RD::LBO1 + (k & 7) * 16);
-    };
-    const int ty = ry0 >> 3, nty = N / 8;   // the stripe lies in one tile row (RS <= 8, aligned)
-    uint32_t act = 0;
-#pragma unroll
-    for (int k = 0; k < RD::ITER; ++k) {
-        int f, aa, ri, b8;
-        piece(k, f, aa, ri, b8);
-        const int tx = (N2 * aa + 8 * b8) >> 3;
-        if (a.active[ty * nty + tx]) {
-            act |= 1u << k;
-        } else {
-            const uint32_t d = piece_dst(f, aa, ri, b8);
-            *reinterpret_cast<uint4 *>(sA1 + d) = make_uint4(0u, 0u, 0u, 0u);
-            *reinterpret_cast<uint4 *>(sA1 + RD::A1B + d) = make_uint4(0u, 0u, 0u, 0u);
-        }
-    }
+    tc::fence_async_smem();   // the tables, written by generic stores, read by the tensor core
     tc::fence_before_sync();
     __syncthreads();
     tc::fence_after_sync();
     const uint32_t tbase = *tslot;
-    const float sc = 1.0f / (float)N2;
 
-    // output row f of sample tt: [re N][im N] halves
-    auto row_base = [&](int tt, int f) -> long long {
-        const int p = f / RS, rl = f - p * RS;
-        return (((long long)tt * a.slab_t + (long long)cl * a.slab_c) * P + p) * N * 2 * N +
-               (long long)(ry0 + rl) * 2 * N;
-    };
-    // input piece: the tile-major field, [channel][pol][tile row][tile col][sample][cy][re/im][cx]
-    const long long tstride = (long long)a.Tb * 128;
-    auto load = [&](int tt, int buf) {
-        unsigned char *dst = sA1 + buf * RD::A1B;
+    if (warp < 8) {
+        // ---------------- twiddle: row m = 128 j + 32 q + lane of tile j (b = m / W, x = m % W) of each pol
+        if constexpr (P == 2) regs_dec<kCpRegsTwiddle>();
+        constexpr int PW = CS::T1 == 2 ? 1 : 2;                  // warp groups per (tile, set of pols)
+        const int g = warp >> 2, j = CS::T1 == 2 ? g : 0, p0 = CS::T1 == 2 ? 0 : g;
+        const int m = 128 * j + 32 * q + lane, b = m / W, x = m % W;
+        const float4 *gtw = reinterpret_cast<const float4 *>(a.dft_tab + CP::TAB);   // [c pair][b]
+        float4 tw[8];
 #pragma unroll
-        for (int k = 0; k < RD::ITER; ++k) {
-            if ((act >> k) & 1u) {
-                int f, aa, ri, b8;
-                piece(k, f, aa, ri, b8);
-                const int p = f / RS, ry = ry0 + (f - p * RS), tx = (N2 * aa + 8 * b8) >> 3;
-                const __half *src = a.G + ((((long long)cl * P + p) * nty + ty) * nty + tx) * tstride +
-                                    (long long)tt * 128 + ((ry & 7) * 2 + ri) * 8;
-                cp_async16(dst + piece_dst(f, aa, ri, b8), src);
-            }
-        }
-        cp_async_commit();
-    };
-    auto issue_s1 = [&](int buf) {
-        tc::fence_after_sync();
-        const uint32_t id1 = tc::idesc_f16(128, S::C1, true, false);
-        const uint32_t a0 = tc::smem_u32(sA1 + buf * RD::A1B), b0 = tc::smem_u32(sB1);
-#pragma unroll
-        for (int j = 0; j < RD::T1; ++j)
-#pragma unroll
-            for (int ks = 0; ks < 2; ++ks)
-                tc::mma_f16(tbase + (uint32_t)(j * S::C1),
-                            tc::smem_desc(a0 + j * 2048 + ks * 2 * RD::LBO1, RD::LBO1, 128),
-                            tc::smem_desc(b0 + ks * 256, 128, 512), id1, ks > 0);
-        tc::mma_commit(&mbar[0]);
-    };
-    auto issue_s2 = [&]() {
-        tc::fence_after_sync();
-        const uint32_t id2 = tc::idesc_f16(128, C2, true, false);
-        const uint32_t a0 = tc::smem_u32(sA2), b0 = tc::smem_u32(sB2);
-        constexpr uint32_t SBOB = (K2 / 8) * 128;
-#pragma unroll
-        for (int j = 0; j < RD::T2; ++j)
-#pragma unroll
-            for (int ks = 0; ks < K2 / 16; ++ks)
-                tc::mma_f16(tbase + (uint32_t)(RD::D1 + j * C2),
-                            tc::smem_desc(a0 + j * 2048 + ks * 2 * RD::LBO2, RD::LBO2, 128),
-                            tc::smem_desc(b0 + ks * 256, 128, SBOB), id2, ks > 0);
-        tc::mma_commit(&mbar[1]);
-    };
-    // twiddle, then stage-2 A: thread (f, b) writes 8 consecutive c at k = b (re) and N2 + b (im)
-    auto epi1 = [&]() {
-        for (int u = warp >> 2; u < RD::T1; u += kBlock / 128) {
-            const int m = 128 * u + 32 * q + lane;
-            const int f = m / N2, b = m - f * N2;
-            float v[32];
-            tc::tmem_ld32(tbase + ((uint32_t)(32 * q) << 16) + (uint32_t)(32 * u), v);
-            uint32_t re[8], im[8];
-#pragma unroll
-            for (int cc = 0; cc < 16; cc += 2) {
-                const float2 t0 = sTw[cc * N2 + b], t1 = sTw[(cc + 1) * N2 + b];
-                re[cc >> 1] = dftc::pack_hh(v[2 * cc] * t0.x - v[2 * cc + 1] * t0.y,
-                                            v[2 * cc + 2] * t1.x - v[2 * cc + 3] * t1.y);
-                im[cc >> 1] = dftc::pack_hh(v[2 * cc] * t0.y + v[2 * cc + 1] * t0.x,
-                                            v[2 * cc + 2] * t1.y + v[2 * cc + 3] * t1.x);
-            }
-#pragma unroll
-            for (int ch = 0; ch < 2; ++ch) {
-                const int mg = 2 * f + ch, kr = b, ki = N2 + b;
-                *reinterpret_cast<uint4 *>(sA2 + mg * 128 + (kr >> 3) * RD::LBO2 + (kr & 7) * 16) =
-                    make_uint4(re[4 * ch], re[4 * ch + 1], re[4 * ch + 2], re[4 * ch + 3]);
-                *reinterpret_cast<uint4 *>(sA2 + mg * 128 + (ki >> 3) * RD::LBO2 + (ki & 7) * 16) =
-                    make_uint4(im[4 * ch], im[4 * ch + 1], im[4 * ch + 2], im[4 * ch + 3]);
-            }
-        }
-    };
-    // stage-2 accumulators -> FP16 (x 1/N2) rows: lane (f, c) holds k = c + 16 d; even lanes store
-    // the real parts of (c, c + 1), odd lanes the imaginary parts (pairs swapped by one shuffle)
-    auto epi2 = [&](int tt) {
-        constexpr int NCB = C2 / 32;
-        for (int u = warp >> 2; u < RD::T2 * NCB; u += kBlock / 128) {
-            const int j = u / NCB, cb2 = u - j * NCB;
-            const int m2 = 128 * j + 32 * q + lane;
-            const int f = m2 >> 4, cc = m2 & 15, odd = cc & 1;
-            float v[32];
-            tc::tmem_ld32(tbase + ((uint32_t)(32 * q) << 16) + (uint32_t)(RD::D1 + j * C2 + 32 * cb2), v);
-            __half *row = a.H + row_base(tt, f) + (odd ? N : 0) + (cc & ~1) + 16 * 16 * cb2;
-#pragma unroll
-            for (int i = 0; i < 16; ++i) {
-                const float re = v[2 * i] * sc, im = v[2 * i + 1] * sc;
-                const float re_o = __shfl_xor_sync(0xffffffffu, re, 1), im_o = __shfl_xor_sync(0xffffffffu, im, 1);
-                *reinterpret_cast<__half2 *>(row + 16 * i) = odd ? __floats2half2_rn(im_o, im) : __floats2half2_rn(re, re_o);
-            }
-        }
-    };
-
-    bool ok = true;
-    if (a.nt > 0) load(0, 0);
-    for (int t = 0; t < a.nt; ++t) {
-        const int buf = t & 1;
-        cp_async_wait<0>();
-        tc::fence_async_smem();
-        tc::fence_before_sync();
-        ok = __syncthreads_and(ok);
-        if (!ok) break;
-        if (tid == 0) issue_s1(buf);
-        if (t + 1 < a.nt) load(t + 1, buf ^ 1);
-        if (t > 0) {
-            ok &= tc::mbar_wait_bounded(&mbar[1], (uint32_t)((t - 1) & 1), dftc::kWaitCycles);
+        for (int i = 0; i < 8; ++i) tw[i] = __ldg(gtw + i * N2 + b);
+        // piece (c group ch, k) at a2_t + ch * (8 W / 64) * K2 * 128 + k * 128, k = b and N2 + b (same k mod 8)
+        const int cgx = W == 8 ? x : (x & 7);
+        const uint32_t a2_t = (uint32_t)((W == 16 ? (x >> 3) * K2 * 128 : 0) + b * 128 + ((cgx ^ (b & 7)) << 4));
+        for (int t = 0; t < a.nt; ++t) {
+            const int buf = t & 1;
+            const uint32_t ph = (uint32_t)((t >> 1) & 1);
+            if (!tc::mbar_wait_abortable(&d1_full[buf], ph, dftc::kWaitCycles, abort_flag)) break;
             tc::fence_after_sync();
-            epi2(t - 1);
+            bool ok = true;
+#pragma unroll
+            for (int p = 0; p < P; ++p) {
+                if (PW == 2 && p != p0) continue;
+                float v[32];
+                tc::tmem_ld32(tbase + ((uint32_t)(32 * q) << 16) + (uint32_t)(buf * CP::D1 + (p * CS::T1 + j) * S::C1), v);
+                if (PW == 2 || p == P - 1) {                     // the warp's last read of this accumulator
+                    tc::fence_before_sync();
+                    __syncwarp();
+                    if (lane == 0) tc::mbar_arrive(&d1_empty[buf]);
+                }
+                uint32_t re[8], im[8];
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const float *u = v + 16 * (i >> 2);
+                    const int e = 2 * (i & 3);
+                    const float2 xr = make_float2(u[e], u[e + 1]), xi = make_float2(u[8 + e], u[9 + e]);
+                    const float2 wr = make_float2(tw[i].x, tw[i].y), nwi = make_float2(tw[i].z, tw[i].w);
+                    const float2 yr = dftc::fma2(xi, nwi, dftc::mul2(xr, wr));
+                    const float2 yi = dftc::sub2(dftc::mul2(xi, wr), dftc::mul2(xr, nwi));
+                    re[i] = dftc::pack_hh(yr.x, yr.y);
+                    im[i] = dftc::pack_hh(yi.x, yi.y);
+                }
+                // stage 2 of sample t - 2 has read this operand buffer
+                if ((PW == 2 || p == 0) && !tc::mbar_wait_abortable(&a2_empty[buf], ph ^ 1u, dftc::kWaitCycles, abort_flag)) { ok = false; break; }
+                unsigned char *o = sA2 + buf * CP::A2 + p * CS::A2P + a2_t;
+#pragma unroll
+                for (int ch = 0; ch < 2; ++ch) {
+                    *reinterpret_cast<uint4 *>(o + ch * (W / 8) * K2 * 128) =
+                        make_uint4(re[4 * ch], re[4 * ch + 1], re[4 * ch + 2], re[4 * ch + 3]);
+                    *reinterpret_cast<uint4 *>(o + ch * (W / 8) * K2 * 128 + N2 * 128) =
+                        make_uint4(im[4 * ch], im[4 * ch + 1], im[4 * ch + 2], im[4 * ch + 3]);
+                }
+            }
+            if (!ok) break;
+            if (P == 1 && PW == 2 && p0 == 1) {                  // one pol, one tile: this group has no rows
+                tc::fence_before_sync();
+                __syncwarp();
+                if (lane == 0) tc::mbar_arrive(&d1_empty[buf]);
+            }
+            tc::fence_async_smem();
+            __syncwarp();
+            if (lane == 0) tc::mbar_arrive(&a2_full[buf]);
         }
-        ok &= tc::mbar_wait_bounded(&mbar[0], (uint32_t)(t & 1), dftc::kWaitCycles);
-        tc::fence_after_sync();
-        epi1();
-        tc::fence_async_smem();
-        tc::fence_before_sync();
-        ok = __syncthreads_and(ok);
-        if (!ok) break;
-        if (tid == 0) issue_s2();
+    } else if (warp < 16) {
+        // ---------------- square and sum (as k_cols_dft): warp group g takes stage-2 tile j2 or half the d range
+        if constexpr (P == 2) regs_inc<kCpRegsSquare>();
+        const int g = (warp - 8) >> 2;
+        const int j2 = CS::T2 == 2 ? g : 0, dbase = CS::T2 == 2 ? 0 : g * ND;
+        float2 acc[NPROD][ND / 2];
+#pragma unroll
+        for (int pq = 0; pq < NPROD; ++pq)
+#pragma unroll
+            for (int d = 0; d < ND / 2; ++d) acc[pq][d] = make_float2(0.f, 0.f);
+        bool ok = true;
+        for (int t = 0; t < a.nt; ++t) {
+            const int buf = t & 1;
+            if (!(ok = tc::mbar_wait_abortable(&d2_full[buf], (uint32_t)((t >> 1) & 1), dftc::kWaitCycles, abort_flag))) break;
+            tc::fence_after_sync();
+            const uint32_t col0 = tbase + ((uint32_t)(32 * q) << 16) +
+                                  (uint32_t)(2 * CP::D1 + buf * CP::D2 + j2 * C2 + 2 * dbase);
+#pragma unroll
+            for (int db = 0; db < ND / 8; ++db) {     // 8 d per TMEM load of each pol: real parts, then imaginary
+                float ex[16];
+                tc::tmem_ld16(col0 + 16 * db, ex);
+                if constexpr (P == 1) {
+                    if (db == ND / 8 - 1) {
+                        tc::fence_before_sync();
+                        __syncwarp();
+                        if (lane == 0) tc::mbar_arrive(&d2_empty[buf]);
+                    }
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const float2 xr = make_float2(ex[2 * i], ex[2 * i + 1]), xi = make_float2(ex[8 + 2 * i], ex[9 + 2 * i]);
+                        float2 &s0 = acc[0][4 * db + i];
+                        s0 = dftc::fma2(xr, xr, dftc::fma2(xi, xi, s0));
+                    }
+                } else {
+                    float ey[16];
+                    tc::tmem_ld16(col0 + 16 * db + (uint32_t)(CS::T2 * C2), ey);
+                    if (db == ND / 8 - 1) {
+                        tc::fence_before_sync();
+                        __syncwarp();
+                        if (lane == 0) tc::mbar_arrive(&d2_empty[buf]);
+                    }
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const float2 xr = make_float2(ex[2 * i], ex[2 * i + 1]), xi = make_float2(ex[8 + 2 * i], ex[9 + 2 * i]);
+                        const float2 yr = make_float2(ey[2 * i], ey[2 * i + 1]), yi = make_float2(ey[8 + 2 * i], ey[9 + 2 * i]);
+                        const int dp = 4 * db + i;
+                        acc[0][dp] = dftc::fma2(xr, xr, dftc::fma2(xi, xi, acc[0][dp]));
+                        acc[1][dp] = dftc::fma2(yr, yr, dftc::fma2(yi, yi, acc[1][dp]));
+                        acc[2][dp] = dftc::fma2(xr, yr, dftc::fma2(xi, yi, acc[2][dp]));
+                        acc[3][dp] = dftc::sub2(dftc::fma2(xi, yr, acc[3][dp]), dftc::mul2(xr, yi));
+                    }
+                }
+            }
+        }
+        if (ok) {   // undo the field's scale s_G / (16 N) (exact powers of two), squared, and fold into FP64
+            const double un = 16.0 * (double)N / ((double)a.sy[c] * (double)a.s_t);
+            const double sc2 = un * un;
+            const int se = (int)((__double2hiint(sc2) >> 20) & 2047) - 1023;
+            const int m2 = 128 * j2 + 32 * q + lane;
+            const int x = (m2 % (8 * W)) >> 3, cy = 8 * (m2 / (8 * W)) + (m2 & 7);
+#pragma unroll
+            for (int pq = 0; pq < NPROD; ++pq) {
+                double *dst = a.acc + ((long long)c * NPROD + pq) * N * N + x0 + x + (long long)(cy + 16 * dbase) * N;
+#pragma unroll
+                for (int d = 0; d < ND; ++d)
+                    red_scaled(dst + 16 * d * N, (d & 1) ? acc[pq][d >> 1].y : acc[pq][d >> 1].x, se, sc2);
+            }
+        }
+    } else {
+        if constexpr (P == 2) regs_dec<kCpRegsIssue>();
+        if (warp == 16 || warp == 19) {
+        // ---------------- producers (one warp per part, re / im): piece (p, h, i) = rows ry = 32 i + lane; in the
+        // operand row group H b + h at k = 2 a + ri (ry = N2 a + b), 16-byte chunk XOR-ed with k mod 8.  Rows
+        // no kernel reaches are zero: cleared once in every stage and never loaded.  Every offset is one of four
+        // swizzled thread constants plus a compile-time one (a copy is one instruction: with addresses computed
+        // per copy the issue itself was the slowest role, about 1500 cycles per sample).
+        constexpr int NI = N / 32, AI = 32 / N2;                 // a = AI i + al
+        const int ri = warp == 19;
+        const int al = lane / N2, b = lane % N2;
+        const uint32_t base = (uint32_t)(((H * b) >> 3) * CS::MH + al * 256 + ((((H * b) & 7) ^ (2 * al) ^ ri) << 4) + ri * 128);
+        uint32_t dt[4];                                          // variants: XOR with 2 v (N2 = 32: i mod 4), or 4 (i mod 2) + h
+#pragma unroll
+        for (int v = 0; v < 4; ++v) dt[v] = tc::smem_u32(sA1) + (base ^ (uint32_t)((AI == 1 ? 2 * v : 4 * (v >> 1) + (v & 1)) << 4));
+        uint32_t rows = 0;
+#pragma unroll
+        for (int i = 0; i < NI; ++i) rows |= ((a.row_nz[i] >> lane) & 1u) << i;
+        auto for_pieces = [&](auto &&f) {                        // f(i, smem offset, source offset in halves)
+#pragma unroll
+            for (int i = 0; i < NI; ++i)
+#pragma unroll
+                for (int p = 0; p < P; ++p)
+#pragma unroll
+                    for (int h = 0; h < H; ++h)
+                        f(i, AI == 1 ? i & 3 : 2 * (i & 1) + h, p * CS::A1P + 2 * AI * i * 128, p * N * 2 * N + field_offset(N, 32 * i, 0, h));
+        };
+        for (int s = 0; s < kCpStages; ++s)
+            for_pieces([&](int i, int v, int off, int) {
+                if (!((rows >> i) & 1u))
+                    asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};\n" ::"r"(dt[v] + s * CP::A1 + off), "r"(0u) : "memory");
+            });
+        const __half *src = a.H + (long long)cl * a.slab_c * P * N * 2 * N + field_offset(N, lane, ri, blockIdx.x * H);
+        const long long tstep = a.slab_t * P * N * 2 * N;
+        auto landed = [&](int t) {                               // this warp's copies of sample t are complete
+            tc::fence_async_smem();
+            __syncwarp();
+            if (lane == 0) tc::mbar_arrive(&full[t % kCpStages]);
+        };
+        // two samples stay in flight: a third would tie each hand-over to the stage freed right before it
+        constexpr int LAG = kCpStages - 2;
+        for (int t = 0; t < a.nt; ++t, src += tstep) {
+            const int st = t % kCpStages;
+            if (!tc::mbar_wait_abortable(&empty[st], (uint32_t)(((t / kCpStages) & 1) ^ 1), dftc::kWaitCycles, abort_flag)) break;
+            uint32_t d[4];
+#pragma unroll
+            for (int v = 0; v < 4; ++v) d[v] = dt[v] + st * CP::A1;
+            for_pieces([&](int i, int v, int off, int so) { cp_async16_if((rows >> i) & 1u, d[v] + off, src + so); });
+            cp_async_commit();
+            if (t >= LAG) {
+                cp_async_wait<LAG>();
+                landed(t - LAG);
+            }
+        }
+        cp_async_wait<0>();
+        for (int t = a.nt > LAG ? a.nt - LAG : 0; t < a.nt; ++t) landed(t);
+        } else if (warp == 17) {
+        // ---------------- stage-1 MMAs (the whole warp runs it, one elected lane issues)
+        const uint32_t one = tc::elect_one(), id1 = tc::idesc_f16(128, S::C1, true, false), b1 = tc::smem_u32(sB1);
+        for (int t = 0; t < a.nt; ++t) {
+            const int st = t % kCpStages, buf = t & 1;
+            if (!tc::mbar_wait_warp(&full[st], (uint32_t)((t / kCpStages) & 1), dftc::kWaitCycles, abort_flag)) break;
+            if (!tc::mbar_wait_warp(&d1_empty[buf], (uint32_t)(((t >> 1) & 1) ^ 1), dftc::kWaitCycles, abort_flag)) break;
+            tc::fence_after_sync();
+            const uint32_t a0 = tc::smem_u32(sA1 + st * CP::A1);
+#pragma unroll
+            for (int p = 0; p < P; ++p)
+#pragma unroll
+                for (int j = 0; j < CS::T1; ++j)
+#pragma unroll
+                    for (int ks = 0; ks < 2; ++ks)
+                        tc::mma_f16_warp(one, tbase + (uint32_t)(buf * CP::D1 + (p * CS::T1 + j) * S::C1),
+                                         tc::smem_desc_sw128(a0 + p * CS::A1P + j * 2 * CS::MH + ks * 2048, CS::MH, 1024),
+                                         tc::smem_desc(b1 + ks * 256, 128, 512), id1, ks > 0);
+            tc::mma_commit_warp(one, &d1_full[buf]);
+            tc::mma_commit_warp(one, &empty[st]);
+        }
+        } else {
+        // ---------------- stage-2 MMAs
+        const uint32_t one = tc::elect_one(), id2 = tc::idesc_f16(128, C2, true, false), b2 = tc::smem_u32(sB2);
+        constexpr uint32_t SBOB = (K2 / 8) * 128;
+        for (int t = 0; t < a.nt; ++t) {
+            const int buf = t & 1;
+            const uint32_t ph = (uint32_t)((t >> 1) & 1);
+            if (!tc::mbar_wait_warp(&a2_full[buf], ph, dftc::kWaitCycles, abort_flag)) break;
+            if (!tc::mbar_wait_warp(&d2_empty[buf], ph ^ 1u, dftc::kWaitCycles, abort_flag)) break;
+            tc::fence_after_sync();
+            const uint32_t a0 = tc::smem_u32(sA2 + buf * CP::A2);
+#pragma unroll
+            for (int p = 0; p < P; ++p)
+#pragma unroll
+                for (int j = 0; j < CS::T2; ++j)
+#pragma unroll
+                    for (int ks = 0; ks < K2 / 16; ++ks)
+                        tc::mma_f16_warp(one, tbase + (uint32_t)(2 * CP::D1 + buf * CP::D2 + (p * CS::T2 + j) * C2),
+                                         tc::smem_desc_sw128(a0 + p * CS::A2P + j * 2 * K2 * 128 + ks * 2048, K2 * 128, 1024),
+                                         tc::smem_desc(b2 + ks * 256, 128, SBOB), id2, ks > 0);
+            tc::mma_commit_warp(one, &d2_full[buf]);
+            tc::mma_commit_warp(one, &a2_empty[buf]);
+        }
+        }
     }
-    if (ok && a.nt > 0) {
-        ok &= tc::mbar_wait_bounded(&mbar[1], (uint32_t)((a.nt - 1) & 1), dftc::kWaitCycles);
-        tc::fence_after_sync();
-        epi2(a.nt - 1);
-    }
-    cp_async_wait<0>();
+    __syncwarp();
     tc::fence_before_sync();
-    ok = __syncthreads_and(ok);
+    __syncthreads();
     tc::fence_after_sync();
-    if (!ok && tid == 0) atomicExch(a.err, tc::kErrWaitTimeout);
-    if (warp == 0) tc::tmem_dealloc(tbase, RD::TCOLS);
+    if (*abort_flag && tid == 0) atomicExch(a.err, tc::kErrWaitTimeout);
+    if (warp == 0) tc::tmem_dealloc(tbase, CP::TCOLS);
 }
 
-template <int N, int P>
-cudaError_t launch_rows_dft_t(const RowDftArgs &a, cudaStream_t st) {
-    auto k = k_rows_dft<N, P>;
-    const size_t smem = RowDftShape<N, P>::SMEM;
+template <int N, int P, int W>
+cudaError_t launch_cols_pipe_t(const ColDftArgs &a, cudaStream_t st) {
+    auto k = k_cols_pipe<N, P, W>;
+    const size_t smem = ColPipeShape<N, P, W>::SMEM;
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    k<<<dim3(N / RowDftShape<N, P>::RS, a.nc), kBlock, smem, st>>>(a);
+    k<<<dim3(N / W, a.nc), kCpThreads, smem, st>>>(a);
     return cudaGetLastError();
 }
 
@@ -561,53 +676,72 @@ cudaError_t launch_cols_dft_t(const ColDftArgs &a, cudaStream_t st) {
 
 
 // ---------------------------------------------------------------------------------------------
-// Row transform for N = 512 as 8 x 64 with the second stage transposed.  With n = b + 64 a
-// (a < 8, b < 64): stage 1 is the 8-point DFT over a, [F 64 rows (f, b)] x [16 (a, re/im)] ->
-// 16 (re/im, c) columns per row; the twiddle exp(+2 pi i b c / 512) / 8 is formed from w_b =
-// exp(+2 pi i b / 512) by complex products in FP32 and applied there, the result rounded to FP16 into
-// the stage-2 operand Y'[(f, c)][(re/im, b)] (MN-major); stage 2 is the 64-point DFT over b as the
-// product D[(re/im, d)][(f, c)] = T[(re/im, d)][(re/im, b)] . Y', the DFT matrix T in real form the
-// K-major A operand.  T's four 64 x 64 blocks are C, -S / S, C (C, S the cosine and sine matrices),
-// kept once as [-S; C; S]: the real-input k-steps read rows C, S from the middle block on, the
-// imaginary-input ones -S, C from the top.  TMEM lane (re/im, d) then holds outputs k = c + 8 d,
-// c < 8, of every row f: eight consecutive outputs of one part, one 16-byte store per row, a warp's
-// 32 lanes (32 consecutive d) writing 512 contiguous bytes.  Output scale 1/8 x 1/64 = 1/512, as the
-// 16 x 32 kernel's.  73 KB of shared memory, 128 TMEM columns: three CTAs per SM.
-template <int P>
+// Row transform of the tensor-core gridding's tile-major field as N1 x N2 (8 x 64 on the 512 grid,
+// 16 x 16 on the 256 grid) with the second stage transposed.  One CTA = a stripe of RS grid rows of one channel
+// (512 grid: eight rows of one pol, whole 256-byte tile samples in and whole 128-byte lines of every strip out; 256
+// grid: eight rows of both pols or sixteen of the one) walking a chunk of samples.  With n = b + N2 a (a < N1, b < N2): stage 1 is the
+// N1-point DFT over a, [F N2 rows (f, b)] x [2 N1 (a, re/im)] -> 2 N1 columns per row; the twiddle
+// exp(+2 pi i b c / N) / N1 is applied in FP32 and the result rounded to FP16 into the stage-2 operand Y'
+// (MN-major); stage 2 is the N2-point DFT over b with the DFT matrix in real form as the K-major A operand.
+//   N = 512: D[(re/im, d) 128][(f, c) 64], K = (re/im, b).  The matrix's four 64 x 64 blocks are C, -S / S, C
+//            (C, S the cosine and sine matrices), kept once as [-S; C; S]: the real-input k-steps read
+//            rows C, S from the middle block on, the imaginary-input ones -S, C from the top.
+//   N = 256: the 16-point matrix X in real form is 32 x 32, so the 16 rows of a stripe are taken as four
+//            quarters h of four: D[(h, re/im, d) 128][(f mod 4, c) 64], K = (h, re/im, b), A = diag(X, X, X, X)
+//            kept once as [0; 0; 0; X; 0; 0; 0], the k-steps of quarter h reading from block 3 - h on.
+// A TMEM lane then holds N1 consecutive outputs k = c + N1 d of one part for consecutive grid rows, which the
+// field's layout (field_offset) takes as whole 32-byte stores.  Output scale 1/N.
+// At most 73 KB of shared memory and 128 TMEM columns: three CTAs per SM.  Bound by DRAM (field in and out).
+// Measured: 256 grid, 96 channels x 333 samples of 4096 antennas 3017 us (3934 us for a 16 x 16 kernel whose stage 2
+// was not transposed and whose rows left as half2 pairs swapped by shuffles); 512 grid, 24 x 250 of 16384 antennas
+// 1942 us (2046 us with rows of [re N][im N]; 2010 us and, on the 256 grid, 3851 us with kFieldRows = 4).
+template <int N_, int P>
 struct RowDft8Shape {
-    static constexpr int N = 512, N1 = 8, N2 = 64;
-    static constexpr int RS = 8 / P, F = P * RS;          // 8 transform rows per stripe, f = p RS + rl
-    static constexpr int M1 = F * N2, T1 = M1 / 128;      // stage-1 rows (f, b): four tiles
-    static constexpr int K1 = 16, C1 = 16;                // (a, re/im) -> (re/im, c)
+    static constexpr int PC = N_ == 512 ? 1 : P;          // pols per CTA: eight (or sixteen) grid rows of one pol or both
+    static constexpr int N = N_, N1 = N == 512 ? 8 : 16, N2 = N / N1;
+    static constexpr int HV = 64 / N2;                    // parts of the stripe's rows sharing one product
+    static constexpr int F = N == 512 ? 8 : 16, RS = F / PC;   // transform rows per stripe, f = p RS + rl
+    static constexpr int FH = F / HV;                     // rows f per part: f = h FH + f'
+    static constexpr int M1 = F * N2, T1 = M1 / 128;      // stage-1 rows (f, b)
+    static constexpr int K1 = 2 * N1, C1 = 2 * N1;        // (a, re/im) -> stage-1 columns
     static constexpr int LBO1 = (M1 / 8) * 128;
     static constexpr int A1B = M1 * K1 * 2;
-    static constexpr int NB = F * N1;                     // stage-2 N: (f, c)
-    static constexpr int K2 = 2 * N2;                     // stage-2 K: (re/im, b)
+    static constexpr int NB = FH * N1;                    // stage-2 N: (f', c)
+    static constexpr int K2 = 2 * N2 * HV;                // stage-2 K: (h, re/im, b)
     static constexpr int LBOB = (NB / 8) * 128;           // K-direction stride of the stage-2 B operand
     static constexpr int BB = NB * K2 * 2;
     static constexpr int B1_BYTES = C1 * K1 * 2;
-    static constexpr int TSBO = (N2 / 8) * 128;           // row-group stride of the [-S; C; S] image (K = 64)
-    static constexpr int T_BYTES = 3 * N2 * N2 * 2;
-    static constexpr int W_BYTES = N2 * 8;                // float2 w_b
+    static constexpr int KT = N == 512 ? 64 : 32;         // contraction of the stored blocks
+    static constexpr int TSBO = (KT / 8) * 128;           // their row-group stride
+    static constexpr int T_BYTES = (N == 512 ? 192 : 224) * KT * 2;
+    static constexpr int W_BYTES = N == 512 ? N2 * 8 : N1 * N2 * 8;   // float2 w_b, or exp(2 pi i b c / N) / 16 [c][b]
     static constexpr int TAB_BYTES = B1_BYTES + T_BYTES + W_BYTES;
     static constexpr int D1 = T1 * C1;                    // TMEM: stage-1 accumulators, then NB stage-2 columns
     static constexpr int TCOLS = 128;
-    static constexpr int NPIECE = F * N1 * 2 * (N2 / 8);  // 16-byte pieces per sample: (f, a, re/im, b8)
-    static constexpr int ITER = NPIECE / kBlock;
+    static constexpr int B8 = N2 / 8;                     // 16-byte pieces (8 b) per (f, a, re/im)
+    static constexpr int ITER = F * N1 * 2 * B8 / kBlock; // pieces per thread and sample
     static constexpr size_t SMEM = 16 + 2 * (size_t)A1B + BB + TAB_BYTES + 32;
-    static_assert(D1 + NB <= TCOLS && NPIECE % kBlock == 0 && kBlock == 256 && T1 == 4 && TAB_BYTES % 16 == 0,
-                  "8 x 64 row-transform shape");
+    static_assert(D1 + NB <= TCOLS && NB == 64 && K2 == 128 && kBlock == 256 && F % 8 == 0 && ITER == 4 &&
+                      TAB_BYTES % 16 == 0 && SMEM * 3 <= 226 * 1024,
+                  "row-transform shape");
 };
 
 __device__ __forceinline__ float2 cmul8(float2 a, float2 b) {
     return make_float2(fmaf(a.x, b.x, -a.y * b.y), fmaf(a.x, b.y, a.y * b.x));
 }
 
-template <int P>
+// 32 contiguous bytes (32-byte aligned) in one store: a whole L2 sector.
+__device__ __forceinline__ void st_sector(__half *dst, const uint32_t (&w)[8]) {
+    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};\n" ::"l"(dst), "r"(w[0]), "r"(w[1]), "r"(w[2]),
+                 "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7])
+                 : "memory");
+}
+
+template <int N, int P>
 __global__ void __launch_bounds__(kBlock) k_rows_dft8(const RowDftArgs a) {
-    using RD = RowDft8Shape<P>;
-    constexpr int N = RD::N, N2 = RD::N2, RS = RD::RS;
-    const int s = blockIdx.x, cl = blockIdx.y;
+    using RD = RowDft8Shape<N, P>;
+    constexpr int N1 = RD::N1, N2 = RD::N2, RS = RD::RS, FH = RD::FH;
+    const int s = blockIdx.x / (P / RD::PC), pc = blockIdx.x % (P / RD::PC), cl = blockIdx.y;   // pc: the first pol
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, q = warp & 3;
     const int ry0 = s * RS;
     {   // stripes no kernel reaches carry no field: nothing to transform or store
@@ -633,20 +767,30 @@ __global__ void __launch_bounds__(kBlock) k_rows_dft8(const RowDftArgs a) {
         tc::tmem_alloc(tslot, RD::TCOLS);
         tc::tmem_relinquish();
     }
-    // Piece i = k kBlock + tid = ((f 8 + aa) 2 + ri) 8 + b8: the thread fixes (aa, ri, b8) and f mod 2,
-    // k fixes f's high part.  In the stage-1 operand the piece is the 8 rows m = 64 f + 8 b8 + (0..7)
-    // at k = 2 aa + ri; pieces of tiles no kernel reaches are zero, cleared once.
-    const int b8 = tid & 7, ri = (tid >> 3) & 1, aa = (tid >> 4) & 7, f0 = tid >> 7;
-    const int kk = 2 * aa + ri;
-    const uint32_t dst_t = (uint32_t)(b8 * 128 + (kk >> 3) * RD::LBO1 + (kk & 7) * 16);
-    const int ty = ry0 >> 3, nty = N / 8, tx = 8 * aa + b8;   // the stripe lies in one tile row
-    const bool active = a.active[ty * nty + tx] != 0;
-    if (!active) {
+    // Piece (f, tile column tx, re/im ri): 8 consecutive b of a row.  Sixteen consecutive threads take the sixteen
+    // pieces of one tile (256 contiguous bytes; with the tiles across the lanes every 16-byte piece was half a sector
+    // of a line of its own, and the row kernel 25 % slower), rounds k of the block the next sixteen tiles.  In the
+    // stage-1 operand (N2 aa + 8 b8 = 8 tx) the piece is the 8 rows m = N2 f + 8 b8 + (0..7) at kk = 2 aa + ri; pieces
+    // of tiles no kernel reaches are zero, cleared once.
+    constexpr int B8 = RD::B8, NTX = N / 8;
+    const int ri = tid & 1, rl = (tid >> 1) & 7, e0 = tid >> 4;
+    auto piece_dst = [&](int k) -> uint32_t {
+        const int e = 16 * k + e0, tx = e % NTX, kk = 2 * (tx / B8) + ri, f = (e / NTX) * 8 + rl;
+        return (uint32_t)((f * B8 + tx % B8) * 128 + (kk >> 3) * RD::LBO1 + (kk & 7) * 16);
+    };
+    // input piece: the tile-major field, [channel][pol][tile row][tile col][sample][cy][re/im][cx]
+    const long long tstride = (long long)a.Tb * 128;
+    long long src_k[RD::ITER];
+    uint32_t act = 0;
 #pragma unroll
-        for (int k = 0; k < RD::ITER; ++k) {
-            const uint32_t d = (uint32_t)((2 * k + f0) * 8 * 128) + dst_t;
-            *reinterpret_cast<uint4 *>(sA1 + d) = make_uint4(0u, 0u, 0u, 0u);
-            *reinterpret_cast<uint4 *>(sA1 + RD::A1B + d) = make_uint4(0u, 0u, 0u, 0u);
+    for (int k = 0; k < RD::ITER; ++k) {
+        const int e = 16 * k + e0, tx = e % NTX, f = (e / NTX) * 8 + rl, p = f / RS, ty = (ry0 + f % RS) >> 3;
+        src_k[k] = ((((long long)cl * P + pc + p) * NTX + ty) * NTX + tx) * tstride + (rl * 2 + ri) * 8;
+        if (a.active[ty * NTX + tx]) {
+            act |= 1u << k;
+        } else {
+            *reinterpret_cast<uint4 *>(sA1 + piece_dst(k)) = make_uint4(0u, 0u, 0u, 0u);
+            *reinterpret_cast<uint4 *>(sA1 + RD::A1B + piece_dst(k)) = make_uint4(0u, 0u, 0u, 0u);
         }
     }
     tc::fence_before_sync();
@@ -654,37 +798,26 @@ __global__ void __launch_bounds__(kBlock) k_rows_dft8(const RowDftArgs a) {
     tc::fence_after_sync();
     const uint32_t tbase = *tslot;
     const float sc = 1.0f / (float)N2;
+    const uint32_t one = tc::elect_one();
 
-    // output row f of sample tt: [re N][im N] halves
-    auto row_base = [&](int tt, int f) -> long long {
-        const int p = f / RS, rl = f - p * RS;
-        return (((long long)tt * a.slab_t + (long long)cl * a.slab_c) * P + p) * N * 2 * N +
-               (long long)(ry0 + rl) * 2 * N;
-    };
-    // input piece: the tile-major field, [channel][pol][tile row][tile col][sample][cy][re/im][cx]
-    const long long tstride = (long long)a.Tb * 128;
     auto load = [&](int tt, int buf) {
-        if (active) {
-            unsigned char *dst = sA1 + buf * RD::A1B;
+        const uint32_t dst = tc::smem_u32(sA1 + buf * RD::A1B);
 #pragma unroll
-            for (int k = 0; k < RD::ITER; ++k) {
-                const int f = 2 * k + f0, p = f / RS, ry = ry0 + (f - p * RS);
-                const __half *src = a.G + ((((long long)cl * P + p) * nty + ty) * nty + tx) * tstride +
-                                    (long long)tt * 128 + ((ry & 7) * 2 + ri) * 8;
-                cp_async16(dst + (uint32_t)(f * 8 * 128) + dst_t, src);
-            }
-        }
+        for (int k = 0; k < RD::ITER; ++k) cp_async16_if((act >> k) & 1u, dst + piece_dst(k), a.G + src_k[k] + (long long)tt * 128);
         cp_async_commit();
     };
-    auto issue_s1 = [&](int buf) {
+    auto issue_s1 = [&](int buf) {   // by warp 0, one elected lane
         tc::fence_after_sync();
         const uint32_t id1 = tc::idesc_f16(128, RD::C1, true, false);
         const uint32_t a0 = tc::smem_u32(sA1 + buf * RD::A1B), b0 = tc::smem_u32(sB1);
 #pragma unroll
         for (int j = 0; j < RD::T1; ++j)
-            tc::mma_f16(tbase + (uint32_t)(j * RD::C1), tc::smem_desc(a0 + j * 2048, RD::LBO1, 128),
-                        tc::smem_desc(b0, 128, (RD::K1 / 8) * 128), id1, false);
-        tc::mma_commit(&mbar[0]);
+#pragma unroll
+            for (int ks = 0; ks < RD::K1 / 16; ++ks)
+                tc::mma_f16_warp(one, tbase + (uint32_t)(j * RD::C1),
+                            tc::smem_desc(a0 + j * 2048 + ks * 2 * RD::LBO1, RD::LBO1, 128),
+                            tc::smem_desc(b0 + ks * 256, 128, (RD::K1 / 8) * 128), id1, ks > 0);
+        tc::mma_commit_warp(one, &mbar[0]);
     };
     auto issue_s2 = [&]() {
         tc::fence_after_sync();
@@ -692,57 +825,82 @@ __global__ void __launch_bounds__(kBlock) k_rows_dft8(const RowDftArgs a) {
         const uint32_t t0 = tc::smem_u32(sT), b0 = tc::smem_u32(sB);
 #pragma unroll
         for (int ks = 0; ks < RD::K2 / 16; ++ks) {
-            // k-steps 0-3 (real parts of Y'): rows C, S from block 1; 4-7 (imaginary parts): -S, C from block 0
-            const uint32_t ta = t0 + (ks < 4 ? (uint32_t)(8 * RD::TSBO) : 0u) + (uint32_t)((ks & 3) * 256);
-            tc::mma_f16(tbase + (uint32_t)RD::D1, tc::smem_desc(ta, 128, RD::TSBO),
+            // N = 512: real parts of Y' (k-steps 0-3) meet rows C, S, imaginary ones -S, C; N = 256: quarter ks / 2
+            const uint32_t ta = t0 + (N == 512 ? (ks < 4 ? (uint32_t)(8 * RD::TSBO) : 0u) + (uint32_t)((ks & 3) * 256)
+                                               : (uint32_t)((3 - (ks >> 1)) * 4 * RD::TSBO + (ks & 1) * 256));
+            tc::mma_f16_warp(one, tbase + (uint32_t)RD::D1, tc::smem_desc(ta, 128, RD::TSBO),
                         tc::smem_desc(b0 + ks * 2 * RD::LBOB, RD::LBOB, 128), id2, ks > 0);
         }
-        tc::mma_commit(&mbar[1]);
+        tc::mma_commit_warp(one, &mbar[1]);
     };
-    // twiddle, then the stage-2 operand: thread (f, b) writes the eight c of its row at k = b (re)
-    // and k = N2 + b (im) of n-group f
+    // twiddle, then the stage-2 operand: thread (f, b) writes its row's N1 outputs c at k = (h, re, b)
+    // and (h, im, b) of n-group f'
     auto epi1 = [&]() {
         for (int u = warp >> 2; u < RD::T1; u += kBlock / 128) {
             const int m = 128 * u + 32 * q + lane, f = m / N2, b = m - f * N2;
-            float v[16];
-            tc::tmem_ld16(tbase + ((uint32_t)(32 * q) << 16) + (uint32_t)(u * RD::C1), v);
-            float2 w[8];
-            w[0] = make_float2(1.f, 0.f);
-            w[1] = sW[b];
-            w[2] = cmul8(w[1], w[1]);
-            w[3] = cmul8(w[2], w[1]);
-            w[4] = cmul8(w[2], w[2]);
-            w[5] = cmul8(w[4], w[1]);
-            w[6] = cmul8(w[3], w[3]);
-            w[7] = cmul8(w[4], w[3]);
-            uint32_t re[4], im[4];
+            const int h = f / FH, fp = f - h * FH, kr = h * 2 * N2 + b, ki = kr + N2;
+            float v[2 * N1];
+            float2 w[N1];
+            if constexpr (N == 512) {   // columns: the eight real parts, then the imaginary ones
+                tc::tmem_ld16(tbase + ((uint32_t)(32 * q) << 16) + (uint32_t)(u * RD::C1), v);
+                w[0] = make_float2(1.f, 0.f);
+                w[1] = sW[b];
+                w[2] = cmul8(w[1], w[1]);
+                w[3] = cmul8(w[2], w[1]);
+                w[4] = cmul8(w[2], w[2]);
+                w[5] = cmul8(w[4], w[1]);
+                w[6] = cmul8(w[3], w[3]);
+                w[7] = cmul8(w[4], w[3]);
+            } else {                    // columns: (re, im) of each c
+                tc::tmem_ld32(tbase + ((uint32_t)(32 * q) << 16) + (uint32_t)(u * RD::C1), v);
 #pragma unroll
-            for (int cc = 0; cc < 8; cc += 2) {
-                const float2 t0 = w[cc], t1 = w[cc + 1];
-                re[cc >> 1] = dftc::pack_hh((v[cc] * t0.x - v[8 + cc] * t0.y) * 0.125f,
-                                            (v[cc + 1] * t1.x - v[9 + cc] * t1.y) * 0.125f);
-                im[cc >> 1] = dftc::pack_hh((v[cc] * t0.y + v[8 + cc] * t0.x) * 0.125f,
-                                            (v[cc + 1] * t1.y + v[9 + cc] * t1.x) * 0.125f);
+                for (int c = 0; c < N1; ++c) w[c] = sW[c * N2 + b];
             }
-            const int kr = b, ki = N2 + b;
-            *reinterpret_cast<uint4 *>(sB + f * 128 + (kr >> 3) * RD::LBOB + (kr & 7) * 16) =
-                make_uint4(re[0], re[1], re[2], re[3]);
-            *reinterpret_cast<uint4 *>(sB + f * 128 + (ki >> 3) * RD::LBOB + (ki & 7) * 16) =
-                make_uint4(im[0], im[1], im[2], im[3]);
+            uint32_t re[N1 / 2], im[N1 / 2];
+#pragma unroll
+            for (int cc = 0; cc < N1; cc += 2) {
+                const float2 t0 = w[cc], t1 = w[cc + 1];
+                if constexpr (N == 512) {
+                    re[cc >> 1] = dftc::pack_hh((v[cc] * t0.x - v[8 + cc] * t0.y) * 0.125f,
+                                                (v[cc + 1] * t1.x - v[9 + cc] * t1.y) * 0.125f);
+                    im[cc >> 1] = dftc::pack_hh((v[cc] * t0.y + v[8 + cc] * t0.x) * 0.125f,
+                                                (v[cc + 1] * t1.y + v[9 + cc] * t1.x) * 0.125f);
+                } else {
+                    re[cc >> 1] = dftc::pack_hh(v[2 * cc] * t0.x - v[2 * cc + 1] * t0.y,
+                                                v[2 * cc + 2] * t1.x - v[2 * cc + 3] * t1.y);
+                    im[cc >> 1] = dftc::pack_hh(v[2 * cc] * t0.y + v[2 * cc + 1] * t0.x,
+                                                v[2 * cc + 2] * t1.y + v[2 * cc + 3] * t1.x);
+                }
+            }
+#pragma unroll
+            for (int ch = 0; ch < N1 / 8; ++ch) {
+                unsigned char *o = sB + (fp * (N1 / 8) + ch) * 128;
+                *reinterpret_cast<uint4 *>(o + (kr >> 3) * RD::LBOB + (kr & 7) * 16) =
+                    make_uint4(re[4 * ch], re[4 * ch + 1], re[4 * ch + 2], re[4 * ch + 3]);
+                *reinterpret_cast<uint4 *>(o + (ki >> 3) * RD::LBOB + (ki & 7) * 16) =
+                    make_uint4(im[4 * ch], im[4 * ch + 1], im[4 * ch + 2], im[4 * ch + 3]);
+            }
         }
     };
-    // stage-2 accumulators -> FP16 (x 1/N2) rows: lane (re/im, d) of warp group g holds the eight c
-    // of rows f = 4 g .. 4 g + 3
+    // stage-2 accumulators -> FP16 (x 1/N2): lane (h, re/im, d) of warp group g holds columns 32 g .. 32 g + 31 =
+    // (f', c): N = 512 the eight c of four consecutive grid rows (64 contiguous bytes of strip d), N = 256 the
+    // sixteen c of two (32 bytes of strips 2 d and 2 d + 1)
+    const int m2 = 32 * q + lane, hh = m2 / (2 * N2), part = (m2 / N2) & 1, d = m2 % N2;
+    const int f0o = hh * FH + 32 * (warp >> 2) / N1, po = f0o / RS;
+    const int out_t = (pc + po) * N * 2 * N + field_offset(N, ry0 + f0o - po * RS, part, d * (N1 / 8));
     auto epi2 = [&](int tt) {
-        const int g = warp >> 2, m2 = 32 * q + lane, part = m2 / N2, d = m2 - part * N2;
         float v[32];
-        tc::tmem_ld32(tbase + ((uint32_t)(32 * q) << 16) + (uint32_t)(RD::D1 + 32 * g), v);
+        tc::tmem_ld32(tbase + ((uint32_t)(32 * q) << 16) + (uint32_t)(RD::D1 + 32 * (warp >> 2)), v);
+        __half *o = a.H + ((long long)tt * a.slab_t + (long long)cl * a.slab_c) * P * N * 2 * N + out_t;
 #pragma unroll
-        for (int fl = 0; fl < 4; ++fl) {
-            uint32_t h[4];
+        for (int k = 0; k < 2; ++k) {   // N = 512: row pair k; N = 256: strip 2 d + k
+            uint32_t w[8];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) h[u] = dftc::pack_hh(v[8 * fl + 2 * u] * sc, v[8 * fl + 2 * u + 1] * sc);
-            *reinterpret_cast<uint4 *>(a.H + row_base(tt, 4 * g + fl) + part * N + 8 * d) = make_uint4(h[0], h[1], h[2], h[3]);
+            for (int u = 0; u < 8; ++u) {
+                const int i = N == 512 ? 16 * k + 2 * u : 16 * (u >> 2) + 8 * k + 2 * (u & 3);
+                w[u] = dftc::pack_hh(v[i] * sc, v[i + 1] * sc);
+            }
+            st_sector(o + (N == 512 ? field_offset(N, 2 * k, 0, 0) : field_offset(N, 0, 0, k)), w);
         }
     };
 
@@ -755,7 +913,7 @@ __global__ void __launch_bounds__(kBlock) k_rows_dft8(const RowDftArgs a) {
         tc::fence_before_sync();
         ok = __syncthreads_and(ok);
         if (!ok) break;
-        if (tid == 0) issue_s1(buf);
+        if (warp == 0) issue_s1(buf);
         if (t + 1 < a.nt) load(t + 1, buf ^ 1);
         if (t > 0) {
             ok &= tc::mbar_wait_bounded(&mbar[1], (uint32_t)((t - 1) & 1), dftc::kWaitCycles);
@@ -769,7 +927,7 @@ __global__ void __launch_bounds__(kBlock) k_rows_dft8(const RowDftArgs a) {
         tc::fence_before_sync();
         ok = __syncthreads_and(ok);
         if (!ok) break;
-        if (tid == 0) issue_s2();
+        if (warp == 0) issue_s2();
     }
     if (ok && a.nt > 0) {
         ok &= tc::mbar_wait_bounded(&mbar[1], (uint32_t)((a.nt - 1) & 1), dftc::kWaitCycles);
@@ -784,16 +942,15 @@ __global__ void __launch_bounds__(kBlock) k_rows_dft8(const RowDftArgs a) {
     if (warp == 0) tc::tmem_dealloc(tbase, RD::TCOLS);
 }
 
-template <int P>
+template <int N, int P>
 cudaError_t launch_rows_dft8_t(const RowDftArgs &a, cudaStream_t st) {
-    auto k = k_rows_dft8<P>;
-    const size_t smem = RowDft8Shape<P>::SMEM;
+    auto k = k_rows_dft8<N, P>;
+    const size_t smem = RowDft8Shape<N, P>::SMEM;
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    k<<<dim3(512 / RowDft8Shape<P>::RS, a.nc), kBlock, smem, st>>>(a);
+    k<<<dim3(N / RowDft8Shape<N, P>::RS * (P / RowDft8Shape<N, P>::PC), a.nc), kBlock, smem, st>>>(a);
     return cudaGetLastError();
 }
-
 
 }  // namespace
 
@@ -848,45 +1005,63 @@ std::vector<unsigned char> build_dft_table(int N, bool cols) {
     return img;
 }
 
-// Tables of the 8 x 64 row transform (N = 512), all in FP64 then rounded once: B1 [n = 8 re/im + c]
-// [k = 2 a + re/im] = the real form of exp(+2 pi i a c / 8) (K-major, 16 x 16); the stage-2 DFT
-// matrix's blocks [-S; C; S] (S, C [d][b] = sin, cos of 2 pi b d / 64; K-major, 192 rows x 64);
-// w_b = exp(+2 pi i b / 512) as float2.
-std::vector<unsigned char> build_rows8_table() {
-    constexpr int B1B = 16 * 16 * 2, TB = 3 * 64 * 64 * 2;
-    std::vector<unsigned char> img((size_t)B1B + TB + 64 * 8, 0);
+// Tables of the row transform, all in FP64 then rounded once.  N = 512: B1 [n = 8 re/im + c][k = 2 a +
+// re/im] = the real form of exp(+2 pi i a c / 8) (K-major, 16 x 16), the stage-2 blocks [-S; C; S] (S, C
+// [d][b] = sin, cos of 2 pi b d / 64; K-major, 192 rows x 64), w_b = exp(+2 pi i b / 512).  N = 256: B1
+// [n = 2 c + re/im][k = 2 a + re/im] (32 x 32), the blocks [0; 0; 0; X; 0; 0; 0] with X [re/im 16 + d][re/im 16 + b]
+// the real form of exp(+2 pi i b d / 16) (224 rows x 32), twiddles [c][b] = exp(+2 pi i b c / 256) / 16.
+std::vector<unsigned char> build_rows8_table(int N) {
+    const int N1 = N == 512 ? 8 : 16, N2 = N / N1, K1 = 2 * N1, KT = N == 512 ? 64 : 32;
+    const size_t b1 = (size_t)K1 * K1 * 2, tb = (size_t)(N == 512 ? 192 : 224) * KT * 2;
+    std::vector<unsigned char> img(b1 + tb + (size_t)(N == 512 ? N2 : N1 * N2) * 8, 0);
     auto put = [&](size_t off, double v) {
         const __half h = __float2half_rn((float)v);
         std::memcpy(img.data() + off, &h, 2);
     };
-    for (int c = 0; c < 8; ++c)
-        for (int aa = 0; aa < 8; ++aa) {
+    auto col = [&](int c, int ri) { return N == 512 ? 8 * ri + c : 2 * c + ri; };
+    for (int c = 0; c < N1; ++c)
+        for (int aa = 0; aa < N1; ++aa) {
             double wc, ws;
-            unit_root((long long)aa * c, 8, &wc, &ws);
-            put(kmajor_at(c, 2 * aa, 16), wc);
-            put(kmajor_at(c, 2 * aa + 1, 16), -ws);
-            put(kmajor_at(8 + c, 2 * aa, 16), ws);
-            put(kmajor_at(8 + c, 2 * aa + 1, 16), wc);
+            unit_root((long long)aa * c, N1, &wc, &ws);
+            put(kmajor_at(col(c, 0), 2 * aa, K1), wc);
+            put(kmajor_at(col(c, 0), 2 * aa + 1, K1), -ws);
+            put(kmajor_at(col(c, 1), 2 * aa, K1), ws);
+            put(kmajor_at(col(c, 1), 2 * aa + 1, K1), wc);
         }
-    for (int d = 0; d < 64; ++d)
-        for (int b = 0; b < 64; ++b) {
+    for (int d = 0; d < N2; ++d)
+        for (int b = 0; b < N2; ++b) {
             double vc, vs;
-            unit_root((long long)b * d, 64, &vc, &vs);
-            put(B1B + kmajor_at(d, b, 64), -vs);
-            put(B1B + kmajor_at(64 + d, b, 64), vc);
-            put(B1B + kmajor_at(128 + d, b, 64), vs);
+            unit_root((long long)b * d, N2, &vc, &vs);
+            if (N == 512) {
+                put(b1 + kmajor_at(d, b, KT), -vs);
+                put(b1 + kmajor_at(64 + d, b, KT), vc);
+                put(b1 + kmajor_at(128 + d, b, KT), vs);
+            } else {
+                put(b1 + kmajor_at(96 + d, b, KT), vc);
+                put(b1 + kmajor_at(96 + d, 16 + b, KT), -vs);
+                put(b1 + kmajor_at(112 + d, b, KT), vs);
+                put(b1 + kmajor_at(112 + d, 16 + b, KT), vc);
+            }
         }
-    for (int b = 0; b < 64; ++b) {
+    for (int i = 0; i < (N == 512 ? N2 : N1 * N2); ++i) {
         double wc, ws;
-        unit_root(b, 512, &wc, &ws);
+        if (N == 512) {
+            unit_root(i, N, &wc, &ws);
+        } else {
+            unit_root((long long)(i / N2) * (i % N2), N, &wc, &ws);
+            wc /= 16.0;
+            ws /= 16.0;
+        }
         const float2 v = make_float2((float)wc, (float)ws);
-        std::memcpy(img.data() + B1B + TB + (size_t)b * 8, &v, 8);
+        std::memcpy(img.data() + b1 + tb + (size_t)i * 8, &v, 8);
     }
     return img;
 }
 
-cudaError_t launch_rows_dft8(int P, const RowDftArgs &a, cudaStream_t st) {
-    return P == 1 ? launch_rows_dft8_t<1>(a, st) : launch_rows_dft8_t<2>(a, st);
+cudaError_t launch_rows_dft8(int N, int P, const RowDftArgs &a, cudaStream_t st) {
+    if (N == 512) return P == 1 ? launch_rows_dft8_t<512, 1>(a, st) : launch_rows_dft8_t<512, 2>(a, st);
+    if (N == 256) return P == 1 ? launch_rows_dft8_t<256, 1>(a, st) : launch_rows_dft8_t<256, 2>(a, st);
+    return cudaErrorInvalidValue;
 }
 
 // Columns per CTA by default: 8 (two CTAs per SM, so one CTA's epilogue runs while the other
@@ -908,17 +1083,11 @@ size_t cols_dft_smem_bytes(int N, int P, int W) {
 cudaError_t launch_cols_dft(int N, int P, int W, const ColDftArgs &a, cudaStream_t st) {
     if (W == 16) {
         if (N == 512) return P == 1 ? launch_cols_dft_t<512, 1, 16>(a, st) : launch_cols_dft_t<512, 2, 16>(a, st);
-        if (N == 256) return P == 1 ? launch_cols_dft_t<256, 1, 16>(a, st) : launch_cols_dft_t<256, 2, 16>(a, st);
+        if (N == 256) return P == 1 ? launch_cols_pipe_t<256, 1, 16>(a, st) : launch_cols_pipe_t<256, 2, 16>(a, st);
     } else {
-        if (N == 512) return P == 1 ? launch_cols_dft_t<512, 1, 8>(a, st) : launch_cols_dft_t<512, 2, 8>(a, st);
-        if (N == 256) return P == 1 ? launch_cols_dft_t<256, 1, 8>(a, st) : launch_cols_dft_t<256, 2, 8>(a, st);
+        if (N == 512) return P == 1 ? launch_cols_pipe_t<512, 1, 8>(a, st) : launch_cols_pipe_t<512, 2, 8>(a, st);
+        if (N == 256) return P == 1 ? launch_cols_pipe_t<256, 1, 8>(a, st) : launch_cols_pipe_t<256, 2, 8>(a, st);
     }
-    return cudaErrorInvalidValue;
-}
-
-cudaError_t launch_rows_dft(int N, int P, const RowDftArgs &a, cudaStream_t st) {
-    if (N == 512) return P == 1 ? launch_rows_dft_t<512, 1>(a, st) : launch_rows_dft_t<512, 2>(a, st);
-    if (N == 256) return P == 1 ? launch_rows_dft_t<256, 1>(a, st) : launch_rows_dft_t<256, 2>(a, st);
     return cudaErrorInvalidValue;
 }
 

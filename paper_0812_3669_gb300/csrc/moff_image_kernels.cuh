@@ -125,7 +125,7 @@ static_assert(fft_radix(32, 0) == FftPlan<32>::R0 && fft_radix(32, 1) == FftPlan
 // CPL = grid cells per lane: 1, 2 (cells (f, e), (f, e + 1) of one row) or 4 (the 2 x 2
 // block (f, e), (f, e + 1), (f + 1, e), (f + 1, e + 1), f even); each entry carries CPL taps.
 // DFT: the row transform runs as factored DFT contractions on the tensor cores
-// (moff_dft.cuh) and the field leaves as FP16 rows [re N][im N] (a.h16).
+// (moff_dft.cuh) and the field leaves in FP16 (a.h16, field_offset).
 // (s, cl): this CTA's stripe and channel of the launch; n_str: stripes per set (the grid's x extent).
 template <int N, int P, int TB, bool STAGED, bool GRID_ONLY, int CPL, bool WIDE, bool DFT = false>
 __device__ __forceinline__ void grid_rows(const GridArgs &a, const int s, const int cl, const int n_str) {
@@ -161,13 +161,12 @@ __device__ __forceinline__ void grid_rows(const GridArgs &a, const int s, const 
             }
             if (!any) return;
         }
-        if constexpr (DFT) {   // FP16 rows [re N][im N]: 8 halves per 16-byte store
-            constexpr int PER_T16 = P * ROWS * 2 * N / 8;
+        if constexpr (DFT) {   // FP16 field: one 16-byte piece (8 columns of a row and part) per store
+            constexpr int PIECES = N / 8 * 2, PER_T16 = P * PIECES * ROWS;
             for (int i = tid; i < a.nt * PER_T16; i += kBlock) {
-                const int t = i / PER_T16, e = 8 * (i - t * PER_T16);
-                const int p = e / (ROWS * 2 * N), rem = e - p * (ROWS * 2 * N), rl = rem / (2 * N), x = rem - rl * 2 * N;
-                __half *o = a.h16 + (((long long)t * a.slab_t + (long long)cl * a.slab_c) * P * N + (long long)p * N +
-                                     (long long)s * ROWS + rl) * 2 * N + x;
+                const int t = i / PER_T16, e = i - t * PER_T16, rl = e % ROWS, k = (e / ROWS) % PIECES, p = e / (ROWS * PIECES);
+                __half *o = a.h16 + (((long long)t * a.slab_t + (long long)cl * a.slab_c) * P + p) * N * 2 * N +
+                            field_offset(N, s * ROWS + rl, k & 1, k >> 1);
                 *reinterpret_cast<uint4 *>(o) = make_uint4(0u, 0u, 0u, 0u);
             }
             return;
@@ -393,13 +392,13 @@ __device__ __forceinline__ void grid_rows(const GridArgs &a, const int s, const 
                            ry0 + rl) * N;
         };
         if constexpr (DFT) {
-            // Global FP16 row [re N][im N] of transform row fa (nullptr past the chunk).
+            // First piece (strip 0, real part) of transform row fa in the FP16 field (nullptr past the chunk).
             auto rowout = [&](int fa) -> __half * {
                 const int t = fa / PR, f = fa - t * PR;
                 if (t >= nb) return nullptr;
                 const int p = f / ROWS, rl = f - p * ROWS;
-                return a.h16 + (((long long)(tb0 + t) * a.slab_t + (long long)cl * a.slab_c) * P * N +
-                                (long long)p * N + ry0 + rl) * 2 * N;
+                return a.h16 + (((long long)(tb0 + t) * a.slab_t + (long long)cl * a.slab_c) * P + p) * N * 2 * N +
+                       field_offset(N, ry0 + rl, 0, 0);
             };
             dft_ok = dftc::rows_dft<N, F, LDR, kBlock>(s_buf, sG, s_dft, s_mbar, tbase, mphase,
                                                       reinterpret_cast<__half *>(s_buf), rowout);

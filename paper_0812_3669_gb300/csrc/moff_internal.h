@@ -55,9 +55,8 @@ struct GridArgs {
     // g (n_stripes n_slices + 1) and lane_cell + g n_stripes n_slices 32, and their values
     // already index the shared st_ant / con_tap / con_y.  nullptr: one set.
     const int *chan_group;
-    // Dense tensor-core transform (k_grid_rows_dft): the row-transformed field as FP16 rows
-    // [re N][im N] (slab [P][N] rows of 2N halves at index t * slab_t + cl * slab_c), scaled by
-    // sy[c] * s_t (powers of two) / N; dft_tab the factored-DFT table image; err set when an
+    // Dense tensor-core transform (k_grid_rows_dft): the row-transformed field in FP16
+    // (field_offset), scaled by sy[c] * s_t (powers of two) / N; dft_tab the factored-DFT table image; err set when an
     // MMA does not complete within its wait limit.
     __half *h16;
     const float *sy;
@@ -66,9 +65,20 @@ struct GridArgs {
     int *err;
 };
 
+// The dense routes' FP16 row-transformed field of one (sample, channel, pol): [row / R][re, im][column / 8][row mod R]
+// [8 columns], R = kFieldRows.  A column CTA reads strips of 8 columns, a row CTA writes whole rows: with R rows of a
+// strip side by side both move 16 R contiguous bytes (rows of [re N][im N] gave the columns 16 bytes of a sector
+// each; strips over all N rows gave the rows 32 bytes at 16 KB steps).  Rows + columns on the 256 and the 512 grid
+// (96 channels x 333 samples, 24 x 250): R = 2 6538 and 4602 us, R = 4 7350 and 4616, R = 8 7348 and 5108.
+constexpr int kFieldRows = 2;
+__host__ __device__ constexpr int field_offset(int N, int row, int part, int strip) {   // in halves, < 2 N N
+    return (row / kFieldRows) * 2 * N * kFieldRows + part * N * kFieldRows + strip * 8 * kFieldRows + (row % kFieldRows) * 8;
+}
+
 // Dense tensor-core column transform + square-and-integrate (k_cols_dft).
 struct ColDftArgs {
-    const __half *H;          // FP16 rows [re N][im N]; slab [P][N] at t * slab_t + cl * slab_c
+    // FP16 row-transformed field (field_offset): slab t * slab_t + cl * slab_c holds [P] blocks of field_offset order.
+    const __half *H;
     long long slab_t, slab_c;
     int nt, c0, nc;
     double *acc;              // [C][n_prod][N][N] FP64 accumulators (added to)
@@ -79,12 +89,12 @@ struct ColDftArgs {
     int *err;
 };
 
-// Dense tensor-core row transform of a gridded field in global memory (k_rows_dft).
+// Dense tensor-core row transform of a gridded field in global memory (k_rows_dft8).
 struct RowDftArgs {
     const __half *G;          // FP16 gridded field, tile-major [Cb][P][N/8][N/8][Tb][8 cy][re/im][8 cx]
     int Tb;
-    __half *H;                // FP16 row-transformed rows [re N][im N]; slab [P][N] at t * slab_t + cl * slab_c;
-                              // the value carries 1/N more than the field
+    __half *H;                // FP16 row-transformed field (field_offset); the value carries 1/N more
+                              // than the gridded field
     long long slab_t, slab_c;
     int nt, c0, nc;
     const uint32_t *row_nz;   // stripes with no reached row are skipped
@@ -128,10 +138,9 @@ cudaError_t launch_grid_tc(const GridTcArgs &a, const CUtensorMap &are, const CU
                            int n_tiles, int cgroups, size_t smem, cudaStream_t st);
 // Store map of the tile-major gridded field (rows of 128 halves; box 64 x 32, 128-byte swizzle).
 cudaError_t encode_gridtc_store_map(CUtensorMap *map, void *G, long long rows);
-cudaError_t launch_rows_dft(int N, int P, const RowDftArgs &a, cudaStream_t st);
-// The N = 512 row transform as 8 x 64 with the second stage transposed (its own table image).
-cudaError_t launch_rows_dft8(int P, const RowDftArgs &a, cudaStream_t st);
-std::vector<unsigned char> build_rows8_table();
+// The row transform (8 x 64 or 16 x 16) with the second stage transposed (its own table image).
+cudaError_t launch_rows_dft8(int N, int P, const RowDftArgs &a, cudaStream_t st);
+std::vector<unsigned char> build_rows8_table(int N);
 
 // Column transform + square-and-integrate (Eq. m6 steps 3-4, second axis).
 struct ColArgs {

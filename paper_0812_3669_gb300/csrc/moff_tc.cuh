@@ -101,6 +101,43 @@ __device__ __forceinline__ void mma_f16(uint32_t d_tmem, uint64_t adesc, uint64_
         "l"(adesc), "l"(bdesc), "r"(idesc), "r"((uint32_t)accumulate)
         : "memory");
 }
+// The same two for a warp whose lanes all execute the call: the elected lane (`issue` != 0, from elect_one)
+// issues.  With no branch around them the descriptors and barrier addresses stay in uniform registers, which the
+// instruction reads; inside `if (lane == 0)` the compiler moves each of them there first, and the single thread's
+// issue takes over 100 cycles per MMA.
+__device__ __forceinline__ uint32_t elect_one() {
+    uint32_t r;
+    asm volatile(
+        "{\n"
+        ".reg .pred p;\n"
+        "elect.sync _|p, 0xffffffff;\n"
+        "selp.u32 %0, 1, 0, p;\n"
+        "}\n"
+        : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ void mma_f16_warp(uint32_t issue, uint32_t d_tmem, uint64_t adesc, uint64_t bdesc,
+                                             uint32_t idesc, bool accumulate) {
+    asm volatile(
+        "{\n"
+        ".reg .pred p, q;\n"
+        "setp.ne.b32 p, %4, 0;\n"
+        "setp.ne.b32 q, %5, 0;\n"
+        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n"
+        "}\n" ::"r"(d_tmem),
+        "l"(adesc), "l"(bdesc), "r"(idesc), "r"((uint32_t)accumulate), "r"(issue)
+        : "memory");
+}
+__device__ __forceinline__ void mma_commit_warp(uint32_t issue, uint64_t *mbar) {
+    asm volatile(
+        "{\n"
+        ".reg .pred q;\n"
+        "setp.ne.b32 q, %1, 0;\n"
+        "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n"
+        "}\n" ::"r"(smem_u32(mbar)),
+        "r"(issue)
+        : "memory");
+}
 // Arrive once on the mbarrier when every MMA issued so far by this thread is done.
 __device__ __forceinline__ void mma_commit(uint64_t *mbar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(smem_u32(mbar))
@@ -128,6 +165,7 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t *mbar, uint32_t parity) {
 // cycles.  Returns false on time-out (the caller records an error and
 // unwinds instead of spinning forever).
 __device__ __forceinline__ bool mbar_wait_bounded(uint64_t *mbar, uint32_t parity, long long max_cycles) {
+    if (mbar_try_wait(mbar, parity)) return true;   // the clock is read only if the first poll fails
     const long long t0 = clock64();
     while (!mbar_try_wait(mbar, parity)) {
         if (clock64() - t0 > max_cycles) return false;
@@ -148,6 +186,7 @@ __device__ __forceinline__ void mbar_arrive(uint64_t *mbar) {
 // `abort` (shared memory), so one time-out unwinds every role.
 __device__ __forceinline__ bool mbar_wait_abortable(uint64_t *mbar, uint32_t parity, long long max_cycles,
                                                     volatile int *abort) {
+    if (mbar_try_wait(mbar, parity)) return true;
     const long long t0 = clock64();
     while (!mbar_try_wait(mbar, parity)) {
         if (*abort) return false;
@@ -157,6 +196,11 @@ __device__ __forceinline__ bool mbar_wait_abortable(uint64_t *mbar, uint32_t par
         }
     }
     return true;
+}
+
+// The same for a warp that goes on as one (its vote keeps the loop around it uniform).
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t *mbar, uint32_t parity, long long max_cycles, volatile int *abort) {
+    return __all_sync(0xffffffffu, mbar_wait_abortable(mbar, parity, max_cycles, abort));
 }
 
 // ---- TMEM -> registers: this warp's 32 lanes x 32 consecutive FP32 columns.
