@@ -262,7 +262,7 @@ struct moff_plan {
     int *d_rs_kp = nullptr, *d_rs_chunk_row = nullptr, *d_rs_chunk_off = nullptr, *d_rs_perm = nullptr,
         *d_err = nullptr;
     long long *d_rs_bimg_off = nullptr;
-    CUtensorMap a_map_re{}, a_map_im{};   // TMA maps of the voltage planes (d_yre, d_yim)
+    CUtensorMap a_map{};                  // TMA load map of both voltage planes (d_yre, d_yim)
     CUtensorMap vp_smap_re{}, vp_smap_im{};   // their store maps (row plane kernel)
     bool vp_tma = true;                       // the row plane kernel stores by TMA boxes (MOFF_VP_TMA=0: directly)
     float *d_rs_row_sh = nullptr, *d_rs_row_inv = nullptr;
@@ -297,7 +297,7 @@ struct moff_plan {
     long long *d_gt_bimg_off = nullptr;
     __half *d_gt_bimg = nullptr;
     unsigned char *d_gt_active = nullptr;
-    CUtensorMap gt_map_re{}, gt_map_im{}, gt_map_g{};
+    CUtensorMap gt_map_y{}, gt_map_g{};
     __half *d_G = nullptr;
 
     long long n_samples = 0;
@@ -380,6 +380,10 @@ moff_status palloc(moff_plan *pl, T **p, size_t bytes) {
     *p = reinterpret_cast<T *>(q);
     return MOFF_OK;
 }
+
+// Bytes from the real voltage plane to the imaginary one (one allocation holds both: the TMA load map's
+// outermost stride).
+size_t plane_gap(const moff_plan *pl) { return (pl->y_bytes + 1023) / 1024 * 1024; }
 
 void pfree(moff_plan *pl, void *p) {
     if (!p) return;
@@ -692,7 +696,7 @@ moff_status run_image_tc(moff_plan *pl, const uint8_t *volt, int n_time, long lo
                 pl->h_map_nt = nt;
             }
             TimedLaunch tg(pl, 1);
-            MOFF_CK(launch_rowspec(pl->N, ra, pl->h_map, pl->a_map_re, pl->a_map_im, std::min(pl->rs_cgroups, nc),
+            MOFF_CK(launch_rowspec(pl->N, ra, pl->h_map, pl->a_map, std::min(pl->rs_cgroups, nc),
                                    pl->rs_smem, pl->st));
             tg.done();
             ColArgs ca{};
@@ -848,7 +852,7 @@ moff_status run_image_gtc(moff_plan *pl, const uint8_t *volt, int n_time, long l
             ga.Tb = pl->Tb;
             ga.err = pl->d_err;
             TimedLaunch tg(pl, 1);
-            MOFF_CK(launch_grid_tc(ga, pl->gt_map_re, pl->gt_map_im, pl->gt_map_g, pl->gt_tiles,
+            MOFF_CK(launch_grid_tc(ga, pl->gt_map_y, pl->gt_map_g, pl->gt_tiles,
                                    std::min(pl->gt_cgroups, nc), pl->gt_smem, pl->st));
             tg.done();
             RowDftArgs ra{};
@@ -2032,8 +2036,7 @@ moff_status plan_run_served(moff_plan *pl, void *scratch, const uint8_t *volt, i
         pl->d_yim = reinterpret_cast<__half *>(base + off);
         off += align_up(pl->y_bytes, 1024);
         const long long rows = (long long)pl->Cb * pl->gt_rows;
-        if (encode_plane_map(&pl->gt_map_re, pl->d_yre, pl->Tb, rows, 16) != cudaSuccess ||
-            encode_plane_map(&pl->gt_map_im, pl->d_yim, pl->Tb, rows, 16) != cudaSuccess ||
+        if (encode_plane_map(&pl->gt_map_y, pl->d_yre, pl->Tb, rows, plane_gap(pl), 16) != cudaSuccess ||
             encode_plane_store_map(&pl->vp_smap_re, pl->d_yre, pl->Tb, rows) != cudaSuccess ||
             encode_plane_store_map(&pl->vp_smap_im, pl->d_yim, pl->Tb, rows) != cudaSuccess)
             return fail(MOFF_ECUDA, "tensor maps of the voltage planes could not be encoded");
@@ -2048,8 +2051,7 @@ moff_status plan_run_served(moff_plan *pl, void *scratch, const uint8_t *volt, i
         if (encode_field_map(&pl->h_map, pl->d_H, pl->N, pl->P, pl->Cb, pl->Tb) != cudaSuccess)
             return fail(MOFF_ECUDA, "tensor map of the row-transformed field could not be encoded");
         const long long rows = (long long)pl->Cb * (pl->A * pl->P + kRowSpecPad);
-        if (encode_plane_map(&pl->a_map_re, pl->d_yre, pl->Tb, rows) != cudaSuccess ||
-            encode_plane_map(&pl->a_map_im, pl->d_yim, pl->Tb, rows) != cudaSuccess ||
+        if (encode_plane_map(&pl->a_map, pl->d_yre, pl->Tb, rows, plane_gap(pl)) != cudaSuccess ||
             encode_plane_store_map(&pl->vp_smap_re, pl->d_yre, pl->Tb, rows) != cudaSuccess ||
             encode_plane_store_map(&pl->vp_smap_im, pl->d_yim, pl->Tb, rows) != cudaSuccess)
             return fail(MOFF_ECUDA, "tensor maps of the voltage planes could not be encoded");
@@ -2238,11 +2240,10 @@ moff_status moff_plan_create(moff_plan **out, int n_ant, const double *pos, int 
             if ((s = palloc(pl, &pl->d_H, pl->h_bytes)) != MOFF_OK) return bail(s);
             if (pl->gtc) {
                 if ((s = palloc(pl, &pl->d_G, pl->h_bytes)) != MOFF_OK) return bail(s);
-                if ((s = palloc(pl, &pl->d_yre, pl->y_bytes)) != MOFF_OK) return bail(s);
-                if ((s = palloc(pl, &pl->d_yim, pl->y_bytes)) != MOFF_OK) return bail(s);
+                if ((s = palloc(pl, &pl->d_yre, 2 * plane_gap(pl))) != MOFF_OK) return bail(s);
+                pl->d_yim = pl->d_yre + plane_gap(pl) / 2;
                 const long long rows = (long long)pl->Cb * pl->gt_rows;
-                if (encode_plane_map(&pl->gt_map_re, pl->d_yre, pl->Tb, rows, 16) != cudaSuccess ||
-                    encode_plane_map(&pl->gt_map_im, pl->d_yim, pl->Tb, rows, 16) != cudaSuccess ||
+                if (encode_plane_map(&pl->gt_map_y, pl->d_yre, pl->Tb, rows, plane_gap(pl), 16) != cudaSuccess ||
                     encode_plane_store_map(&pl->vp_smap_re, pl->d_yre, pl->Tb, rows) != cudaSuccess ||
                     encode_plane_store_map(&pl->vp_smap_im, pl->d_yim, pl->Tb, rows) != cudaSuccess)
                     return bail(fail(MOFF_ECUDA, "tensor maps of the voltage planes could not be encoded"));
@@ -2366,11 +2367,10 @@ moff_status moff_plan_create(moff_plan **out, int n_ant, const double *pos, int 
         if ((s = palloc(pl, &pl->d_rs_bimg, std::max<size_t>(rs.bimg.size(), 8) * 2)) != MOFF_OK) return bail(s);
         pl->y_bytes = ny * 2;
         if (!pl->served) {
-            if ((s = palloc(pl, &pl->d_yre, ny * 2)) != MOFF_OK) return bail(s);
-            if ((s = palloc(pl, &pl->d_yim, ny * 2)) != MOFF_OK) return bail(s);
+            if ((s = palloc(pl, &pl->d_yre, 2 * plane_gap(pl))) != MOFF_OK) return bail(s);
+            pl->d_yim = pl->d_yre + plane_gap(pl) / 2;
             const long long rows = (long long)pl->Cb * (n_ant * n_pol + kRowSpecPad);
-            if (encode_plane_map(&pl->a_map_re, pl->d_yre, pl->Tb, rows) != cudaSuccess ||
-                encode_plane_map(&pl->a_map_im, pl->d_yim, pl->Tb, rows) != cudaSuccess ||
+            if (encode_plane_map(&pl->a_map, pl->d_yre, pl->Tb, rows, plane_gap(pl)) != cudaSuccess ||
                 encode_plane_store_map(&pl->vp_smap_re, pl->d_yre, pl->Tb, rows) != cudaSuccess ||
                 encode_plane_store_map(&pl->vp_smap_im, pl->d_yim, pl->Tb, rows) != cudaSuccess)
                 return bail(fail(MOFF_ECUDA, "tensor maps of the voltage planes could not be encoded"));

@@ -20,6 +20,11 @@
 //              (128-byte swizzle, MN-major), one lane issues tcgen05.mma into one
 //              of two TMEM accumulators, and eight warps convert the accumulator
 //              to FP16 and store the tile's field rows [re 8][im 8] per (pol, row).
+//
+// One warp each feeds the ring and issues the MMAs, so their per-chunk overhead sets the pace: with the warp running
+// as one (mma_f16_warp), both planes in one box, plane rows in registers and the ring counted instead of divided, 24
+// channels x 250 samples of 16384 antennas take 846 us instead of 1170, the Jones lattice of 32768 (24 x 256) 1700
+// instead of 2331.  Bound by DRAM then (planes in, field out) at about 0.75 of the copy bandwidth.
 #include <cuda_fp16.h>
 
 #include <algorithm>
@@ -45,8 +50,7 @@ constexpr int kGtBoxBytes = 32 * 128;                    // epilogue box: 32 sam
 
 template <int P>
 __global__ void __launch_bounds__(kGtThreads, 1)
-    k_grid_tc(const GridTcArgs a, const __grid_constant__ CUtensorMap amap_re,
-              const __grid_constant__ CUtensorMap amap_im, const __grid_constant__ CUtensorMap gmap) {
+    k_grid_tc(const GridTcArgs a, const __grid_constant__ CUtensorMap amap, const __grid_constant__ CUtensorMap gmap) {
     constexpr int NT = 128 * P;                           // output columns (p, cy, re/im, cx)
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int item = blockIdx.x;
@@ -99,74 +103,70 @@ __global__ void __launch_bounds__(kGtThreads, 1)
     const uint32_t tbase = *tslot;
 
     if (warp == kGtEpiWarps) {
-        // ---------------- producer (one lane): the tile's kernel matrix B by one bulk copy
-        // (completing on b_full), then chunk g into stage g % ns, four TMA boxes (re / im rows x
-        // two 64-sample halves) completing on a_full
-        if (lane == 0) {
+        // ---------------- producer (the whole warp runs it, one elected lane issues): the tile's kernel matrix B by
+        // one bulk copy (completing on b_full), then chunk after chunk into the ring, one box of both planes
+        // per 64-sample half completing on a_full.  The chunks' plane rows stay in the lanes' registers (a tile has
+        // at most kp_max / 32 <= 20 chunks) and ring slot and phase are counted, not divided out.
+        const uint32_t one = tc::elect_one();
+        if (one) {
             tc::mbar_arrive_expect_tx(b_full, bbytes_item);
             tc::bulk_load(tc::smem_u32(sB), reinterpret_cast<const unsigned char *>(a.bimg) + a.bimg_off[item],
                           bbytes_item, b_full);
-            int g = 0;
-            for (int i = 0; i < nitems && !*abort_flag; ++i) {
-                const int cl = cb + i / ntb, t0b = (i % ntb) * 128;
-                bool ok = true;
-                for (int ch = 0; ch < nchunk; ++ch, ++g) {
-                    const int st = g % ns;
-                    if (!tc::mbar_wait_abortable(&a_empty[st], (uint32_t)(((g / ns) & 1) ^ 1), kGtWaitCycles,
-                                                 abort_flag)) {
-                        ok = false;
-                        break;
-                    }
-                    const uint32_t sa = tc::smem_u32(sA + st * kGtStageBytes);
-                    const int y = cl * a.AP + a.chunk_row[ch0 + ch];
-                    tc::mbar_arrive_expect_tx(&a_full[st], kGtStageBytes);
-#pragma unroll
-                    for (int hm = 0; hm < 2; ++hm) {
-                        tc::tma_load_2d(sa + hm * kGtHalfBytes, &amap_re, t0b + 64 * hm, y, &a_full[st]);
-                        tc::tma_load_2d(sa + hm * kGtHalfBytes + kGtHalfBytes / 2, &amap_im, t0b + 64 * hm, y,
-                                        &a_full[st]);
-                    }
-                }
-                if (!ok) break;
-            }
-            for (int gg = g - ns > 0 ? g - ns : 0; gg < g; ++gg)
-                tc::mbar_wait_bounded(&a_full[gg % ns], (uint32_t)((gg / ns) & 1), kGtWaitCycles);
-            tc::mbar_wait_bounded(b_full, 0, kGtWaitCycles);   // B has landed before the memory is released
         }
-        __syncwarp();
+        const int row_l = lane < nchunk ? a.chunk_row[ch0 + lane] : 0;
+        int g = 0, st = 0;
+        uint32_t ph = 1;
+        bool ok = true;
+        for (int i = 0; i < nitems && ok; ++i) {
+            const int y0 = (cb + i / ntb) * a.AP, t0b = (i % ntb) * 128;
+            for (int ch = 0; ch < nchunk; ++ch, ++g) {
+                if (!(ok = tc::mbar_wait_warp(&a_empty[st], ph, kGtWaitCycles, abort_flag))) break;
+                const uint32_t sa = tc::smem_u32(sA) + (uint32_t)(st * kGtStageBytes);
+                const int y = y0 + (ch < 32 ? __shfl_sync(0xffffffffu, row_l, ch) : a.chunk_row[ch0 + ch]);
+                tc::mbar_expect_tx_warp(one, &a_full[st], kGtStageBytes);
+                tc::tma_load_3d_warp(one, sa, &amap, t0b, y, 0, &a_full[st]);
+                tc::tma_load_3d_warp(one, sa + kGtHalfBytes, &amap, t0b + 64, y, 0, &a_full[st]);
+                if (++st == ns) {
+                    st = 0;
+                    ph ^= 1u;
+                }
+            }
+        }
+        for (int gg = g - ns > 0 ? g - ns : 0; gg < g; ++gg)
+            tc::mbar_wait_bounded(&a_full[gg % ns], (uint32_t)((gg / ns) & 1), kGtWaitCycles);
+        tc::mbar_wait_bounded(b_full, 0, kGtWaitCycles);   // B has landed before the memory is released
     } else if (warp == kGtEpiWarps + 1) {
-        // ---------------- MMA issuer (one lane)
-        if (lane == 0) {
-            const uint32_t idesc = tc::idesc_f16(128, NT, /*a_mn=*/true, /*b_mn=*/false);
-            const uint32_t sb_sbo = (uint32_t)(kp / 8) * 128;
-            const uint32_t sbb = tc::smem_u32(sB);
-            int g = 0;
-            bool ok = tc::mbar_wait_abortable(b_full, 0, kGtWaitCycles, abort_flag);
-            for (int i = 0; i < nitems && ok; ++i) {
-                const int b = i & 1;
-                ok = tc::mbar_wait_abortable(&d_empty[b], (uint32_t)(((i >> 1) & 1) ^ 1), kGtWaitCycles, abort_flag);
-                if (!ok) break;
-                const uint32_t d = tbase + (uint32_t)(b * NT);
-                for (int ch = 0; ch < nchunk; ++ch, ++g) {
-                    const int st = g % ns;
-                    ok = tc::mbar_wait_abortable(&a_full[st], (uint32_t)((g / ns) & 1), kGtWaitCycles,
-                                                 abort_flag);
-                    if (!ok) break;
-                    tc::fence_after_sync();
-                    const uint32_t sa = tc::smem_u32(sA + st * kGtStageBytes);
+        // ---------------- MMA issuer (one elected lane of the warp issues)
+        const uint32_t one = tc::elect_one();
+        const uint32_t idesc = tc::idesc_f16(128, NT, /*a_mn=*/true, /*b_mn=*/false);
+        const uint32_t sb_sbo = (uint32_t)(kp / 8) * 128;
+        const uint32_t sbb = tc::smem_u32(sB);
+        int st = 0;
+        uint32_t ph = 0;
+        bool ok = tc::mbar_wait_warp(b_full, 0, kGtWaitCycles, abort_flag);
+        for (int i = 0; i < nitems && ok; ++i) {
+            const int b = i & 1;
+            if (!(ok = tc::mbar_wait_warp(&d_empty[b], (uint32_t)(((i >> 1) & 1) ^ 1), kGtWaitCycles, abort_flag))) break;
+            const uint32_t d = tbase + (uint32_t)(b * NT);
+            for (int ch = 0; ch < nchunk; ++ch) {
+                if (!(ok = tc::mbar_wait_warp(&a_full[st], ph, kGtWaitCycles, abort_flag))) break;
+                tc::fence_after_sync();
+                const uint32_t sa = tc::smem_u32(sA) + (uint32_t)(st * kGtStageBytes);
 #pragma unroll
-                    for (int ks = 0; ks < 2; ++ks) {
-                        // k-step 0: the chunk's 16 real rows, 1: its 16 imaginary rows
-                        const uint64_t ad = tc::smem_desc_sw128(sa + ks * 16 * 128, kGtHalfBytes, 1024);
-                        const uint64_t bd = tc::smem_desc(sbb + (ch * (kGtChunkK / 8) + 2 * ks) * 128, 128, sb_sbo);
-                        tc::mma_f16(d, ad, bd, idesc, ch > 0 || ks > 0);
-                    }
-                    tc::mma_commit(&a_empty[st]);
+                for (int ks = 0; ks < 2; ++ks) {
+                    // k-step 0: the chunk's 16 real rows, 1: its 16 imaginary rows
+                    const uint64_t ad = tc::smem_desc_sw128(sa + ks * 16 * 128, kGtHalfBytes, 1024);
+                    const uint64_t bd = tc::smem_desc(sbb + (ch * (kGtChunkK / 8) + 2 * ks) * 128, 128, sb_sbo);
+                    tc::mma_f16_warp(one, d, ad, bd, idesc, ch > 0 || ks > 0);
                 }
-                if (ok) tc::mma_commit(&d_full[b]);
+                tc::mma_commit_warp(one, &a_empty[st]);
+                if (++st == ns) {
+                    st = 0;
+                    ph ^= 1u;
+                }
             }
+            if (ok) tc::mma_commit_warp(one, &d_full[b]);
         }
-        __syncwarp();
     } else {
         // ---------------- epilogue warps 0-7: TMEM lanes 32 (w % 4) .. + 31 = samples; warp w / 4
         // drains half of the columns.  Column n = ((p 8 + cy) 2 + re/im) 8 + cx: every 8 columns are
@@ -411,12 +411,12 @@ moff_status build_gridtc(int A, int K, int N, int P, bool jones, const double *p
     return MOFF_OK;
 }
 
-cudaError_t launch_grid_tc(const GridTcArgs &a, const CUtensorMap &are, const CUtensorMap &aim, const CUtensorMap &gmap,
-                           int n_tiles, int cgroups, size_t smem, cudaStream_t st) {
+cudaError_t launch_grid_tc(const GridTcArgs &a, const CUtensorMap &amap, const CUtensorMap &gmap, int n_tiles,
+                           int cgroups, size_t smem, cudaStream_t st) {
     auto k = a.P == 1 ? k_grid_tc<1> : k_grid_tc<2>;
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    k<<<dim3(n_tiles, cgroups), kGtThreads, smem, st>>>(a, are, aim, gmap);
+    k<<<dim3(n_tiles, cgroups), kGtThreads, smem, st>>>(a, amap, gmap);
     return cudaGetLastError();
 }
 

@@ -134,8 +134,8 @@ moff_status build_gridtc(int A, int K, int N, int P, bool jones, const double *p
                          GridTc *gt);
 size_t gridtc_smem_bytes(int P, int kp_max, int stages, int boxes);
 int gridtc_stages(int P, int kp_max, int boxes);
-cudaError_t launch_grid_tc(const GridTcArgs &a, const CUtensorMap &are, const CUtensorMap &aim, const CUtensorMap &gmap,
-                           int n_tiles, int cgroups, size_t smem, cudaStream_t st);
+cudaError_t launch_grid_tc(const GridTcArgs &a, const CUtensorMap &amap, const CUtensorMap &gmap, int n_tiles,
+                           int cgroups, size_t smem, cudaStream_t st);
 // Store map of the tile-major gridded field (rows of 128 halves; box 64 x 32, 128-byte swizzle).
 cudaError_t encode_gridtc_store_map(CUtensorMap *map, void *G, long long rows);
 // The row transform (8 x 64 or 16 x 16) with the second stage transposed (its own table image).
@@ -392,11 +392,10 @@ cudaError_t launch_volt_prep(const uint8_t *volt, long long tstride, int t0, int
                              const CUtensorMap *smap_im = nullptr);
 // Store maps of the voltage planes for the row plane kernel (box 32 samples x 32 rows, 64-byte swizzle).
 cudaError_t encode_plane_store_map(CUtensorMap *map, void *plane, int Tpad, long long rows);
-cudaError_t launch_rowspec(int N, const RowSpecArgs &a, const CUtensorMap &hmap, const CUtensorMap &amap_re,
-                           const CUtensorMap &amap_im, int cgroups, size_t smem, cudaStream_t st);
+cudaError_t launch_rowspec(int N, const RowSpecArgs &a, const CUtensorMap &hmap, const CUtensorMap &amap, int cgroups, size_t smem, cudaStream_t st);
 // Tensor map of one FP16 voltage plane [rows][Tpad] (rows = Cb * A * P), box 64 samples x
 // 32 rows, 128-byte swizzle, rows past the end read as zero: the A loads of k_rowspec_tc.
-cudaError_t encode_plane_map(CUtensorMap *map, void *plane, int Tpad, long long rows, int box_rows = 32);
+cudaError_t encode_plane_map(CUtensorMap *map, void *plane, int Tpad, long long rows, size_t im_off, int box_rows = 32);
 // Tensor map of the FP16 row-transformed field [nt][Cb][P*N][N] (half2 as 32-bit
 // elements), box 32 kx x 32 samples, 128-byte swizzle: the store target of
 // k_rowspec_tc.  Stores of samples >= nt fall outside the map and are dropped.

@@ -248,12 +248,23 @@ __device__ __forceinline__ void bulk_load(uint32_t dst_smem, const void *src, ui
                  "l"(src), "r"(bytes), "r"(smem_u32(mbar))
                  : "memory");
 }
-// x (innermost, elements) times the element size must be a multiple of 16 bytes.
-__device__ __forceinline__ void tma_load_2d(uint32_t dst_smem, const void *tmap, int x, int y, uint64_t *mbar) {
+// One box of a 3-D tensor map, issued by the elected lane (`issue`) of a warp that executes the call as one (see
+// mma_f16_warp), with the arrival that announces `bytes` on the mbarrier.  x (innermost, elements) times the
+// element size must be a multiple of 16 bytes.
+__device__ __forceinline__ void mbar_expect_tx_warp(uint32_t issue, uint64_t *mbar, uint32_t bytes) {
     asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], "
-        "[%4];\n" ::"r"(dst_smem),
-        "l"(tmap), "r"(x), "r"(y), "r"(smem_u32(mbar))
+        "{\n.reg .pred q;\nsetp.ne.b32 q, %2, 0;\n@q mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n}\n" ::"r"(
+            smem_u32(mbar)),
+        "r"(bytes), "r"(issue)
+        : "memory");
+}
+__device__ __forceinline__ void tma_load_3d_warp(uint32_t issue, uint32_t dst_smem, const void *tmap, int x, int y, int z,
+                                                 uint64_t *mbar) {
+    asm volatile(
+        "{\n.reg .pred q;\nsetp.ne.b32 q, %6, 0;\n"
+        "@q cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], "
+        "[%5];\n}\n" ::"r"(dst_smem),
+        "l"(tmap), "r"(x), "r"(y), "r"(z), "r"(smem_u32(mbar)), "r"(issue)
         : "memory");
 }
 

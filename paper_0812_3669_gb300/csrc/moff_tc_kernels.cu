@@ -306,8 +306,7 @@ constexpr long long kWaitCycles = 4000000000LL;     // ~2 s at the SM clock
 
 template <int N>
 __global__ void __launch_bounds__(kTcRoleThreads, 1)
-    k_rowspec_tc(const RowSpecArgs a, const __grid_constant__ CUtensorMap hmap,
-                 const __grid_constant__ CUtensorMap amap_re, const __grid_constant__ CUtensorMap amap_im) {
+    k_rowspec_tc(const RowSpecArgs a, const __grid_constant__ CUtensorMap hmap, const __grid_constant__ CUtensorMap amap) {
     using S = TcShape<N>;
     constexpr int KX = S::KX, NT = S::NT;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -370,69 +369,60 @@ __global__ void __launch_bounds__(kTcRoleThreads, 1)
     const uint32_t tbase = *tslot;
 
     if (warp == kEpiWarps) {
-        // ---------------- producer (one lane): chunk g (global counter) into stage g % kAStages,
-        // four TMA tiles (re / im x two 64-sample halves) completing on a_full.
-        if (lane == 0) {
-            int g = 0;
-            for (int i = 0; i < nitems && !*abort_flag; ++i) {
-                const int cl = cb + i / ntb, t0b = (i % ntb) * 128;
-                bool ok = true;
-                for (int ch = 0; ch < nchunk; ++ch, ++g) {
-                    const int st = g % kAStages;
-                    if (!tc::mbar_wait_abortable(&a_empty[st], (uint32_t)(((g / kAStages) & 1) ^ 1), kWaitCycles,
-                                                 abort_flag)) {
-                        ok = false;
-                        break;
-                    }
-                    const uint32_t sa = tc::smem_u32(sA + st * kAChunkBytes);
-                    const int y = cl * a.AP + a.chunk_row[ch0 + ch];
-                    tc::mbar_arrive_expect_tx(&a_full[st], kAChunkBytes);
-#pragma unroll
-                    for (int hm = 0; hm < 2; ++hm) {
-                        tc::tma_load_2d(sa + hm * kAHalfBytes, &amap_re, t0b + 64 * hm, y, &a_full[st]);
-                        tc::tma_load_2d(sa + hm * kAHalfBytes + kAHalfBytes / 2, &amap_im, t0b + 64 * hm, y,
-                                        &a_full[st]);
-                    }
-                }
-                if (!ok) break;
+        // ---------------- producer (the whole warp runs it, one elected lane issues): chunk after chunk into the
+        // ring, one box of both planes per 64-sample half completing on a_full; the chunks' plane rows (at most
+        // four) stay in the lanes' registers.
+        const uint32_t one = tc::elect_one();
+        const int row_l = lane < nchunk ? a.chunk_row[ch0 + lane] : 0;
+        int g = 0, st = 0;
+        uint32_t ph = 1;
+        bool ok = true;
+        for (int i = 0; i < nitems && ok; ++i) {
+            const int y0 = (cb + i / ntb) * a.AP, t0b = (i % ntb) * 128;
+            for (int ch = 0; ch < nchunk; ++ch, ++g) {
+                if (!(ok = tc::mbar_wait_warp(&a_empty[st], ph, kWaitCycles, abort_flag))) break;
+                const uint32_t sa = tc::smem_u32(sA) + (uint32_t)(st * kAChunkBytes);
+                const int y = y0 + (ch < 32 ? __shfl_sync(0xffffffffu, row_l, ch) : a.chunk_row[ch0 + ch]);
+                tc::mbar_expect_tx_warp(one, &a_full[st], kAChunkBytes);
+                tc::tma_load_3d_warp(one, sa, &amap, t0b, y, 0, &a_full[st]);
+                tc::tma_load_3d_warp(one, sa + kAHalfBytes, &amap, t0b + 64, y, 0, &a_full[st]);
+                st = (st + 1) % kAStages;
+                ph ^= st == 0 ? 1u : 0u;
             }
-            // tiles still landing (the MMA lane stopped early): let them finish before the
-            // shared memory is released
-            for (int gg = g - kAStages > 0 ? g - kAStages : 0; gg < g; ++gg)
-                tc::mbar_wait_bounded(&a_full[gg % kAStages], (uint32_t)((gg / kAStages) & 1), kWaitCycles);
         }
-        __syncwarp();
+        // tiles still landing (the MMA warp stopped early): let them finish before the shared memory is released
+        for (int gg = g - kAStages > 0 ? g - kAStages : 0; gg < g; ++gg)
+            tc::mbar_wait_bounded(&a_full[gg % kAStages], (uint32_t)((gg / kAStages) & 1), kWaitCycles);
     } else if (warp == kEpiWarps + 1) {
-        // ---------------- MMA issuer (one lane)
-        if (lane == 0) {
-            const uint32_t idesc = tc::idesc_f16(128, NT, /*a_mn=*/true, /*b_mn=*/false);
-            const uint32_t sb_sbo = (uint32_t)(kp / 8) * 128;
-            const uint32_t sbb = tc::smem_u32(sB);
-            int g = 0;
-            bool ok = true;
-            for (int i = 0; i < nitems && ok; ++i) {
-                const int b = i & 1;
-                ok = tc::mbar_wait_abortable(&d_empty[b], (uint32_t)(((i >> 1) & 1) ^ 1), kWaitCycles, abort_flag);
-                if (!ok) break;
-                const uint32_t d = tbase + (uint32_t)(b * NT);
-                for (int ch = 0; ch < nchunk; ++ch, ++g) {
-                    const int st = g % kAStages;
-                    ok = tc::mbar_wait_abortable(&a_full[st], (uint32_t)((g / kAStages) & 1), kWaitCycles, abort_flag);
-                    if (!ok) break;
-                    tc::fence_after_sync();
-                    const uint32_t sa = tc::smem_u32(sA + st * kAChunkBytes);
-                    for (int ks = 0; ks < kKChunk / 16; ++ks) {
-                        // 128-byte swizzled MN-major: LBO = the 64-sample halves' stride, SBO = 8 rows
-                        const uint64_t ad = tc::smem_desc_sw128(sa + ks * 16 * 128, kAHalfBytes, 1024);
-                        const uint64_t bd = tc::smem_desc(sbb + (ch * (kKChunk / 8) + 2 * ks) * 128, 128, sb_sbo);
-                        tc::mma_f16(d, ad, bd, idesc, ch > 0 || ks > 0);
-                    }
-                    tc::mma_commit(&a_empty[st]);   // stage free once these MMAs finish
+        // ---------------- MMA issuer (one elected lane of the warp issues)
+        const uint32_t one = tc::elect_one();
+        const uint32_t idesc = tc::idesc_f16(128, NT, /*a_mn=*/true, /*b_mn=*/false);
+        const uint32_t sb_sbo = (uint32_t)(kp / 8) * 128;
+        const uint32_t sbb = tc::smem_u32(sB);
+        int st = 0;
+        uint32_t ph = 0;
+        bool ok = true;
+        for (int i = 0; i < nitems && ok; ++i) {
+            const int b = i & 1;
+            if (!(ok = tc::mbar_wait_warp(&d_empty[b], (uint32_t)(((i >> 1) & 1) ^ 1), kWaitCycles, abort_flag))) break;
+            const uint32_t d = tbase + (uint32_t)(b * NT);
+            for (int ch = 0; ch < nchunk; ++ch) {
+                if (!(ok = tc::mbar_wait_warp(&a_full[st], ph, kWaitCycles, abort_flag))) break;
+                tc::fence_after_sync();
+                const uint32_t sa = tc::smem_u32(sA) + (uint32_t)(st * kAChunkBytes);
+#pragma unroll
+                for (int ks = 0; ks < kKChunk / 16; ++ks) {
+                    // 128-byte swizzled MN-major: LBO = the 64-sample halves' stride, SBO = 8 rows
+                    const uint64_t ad = tc::smem_desc_sw128(sa + ks * 16 * 128, kAHalfBytes, 1024);
+                    const uint64_t bd = tc::smem_desc(sbb + (ch * (kKChunk / 8) + 2 * ks) * 128, 128, sb_sbo);
+                    tc::mma_f16_warp(one, d, ad, bd, idesc, ch > 0 || ks > 0);
                 }
-                if (ok) tc::mma_commit(&d_full[b]); // accumulator ready
+                tc::mma_commit_warp(one, &a_empty[st]);   // stage free once these MMAs finish
+                st = (st + 1) % kAStages;
+                ph ^= st == 0 ? 1u : 0u;
             }
+            if (ok) tc::mma_commit_warp(one, &d_full[b]); // accumulator ready
         }
-        __syncwarp();
     } else {
         // ---------------- epilogue warps 0-7: TMEM lanes 32 (w % 4) .. + 31 = samples
         unsigned char *sw = sE + warp * kEpiBufs * kBoxBytes;
@@ -550,28 +540,30 @@ cudaError_t launch_volt_prep(const uint8_t *volt, long long tstride, int t0, int
 }
 
 template <int N>
-cudaError_t launch_rowspec_t(const RowSpecArgs &a, const CUtensorMap &hmap, const CUtensorMap &are,
-                             const CUtensorMap &aim, int cgroups, size_t smem, cudaStream_t st) {
+cudaError_t launch_rowspec_t(const RowSpecArgs &a, const CUtensorMap &hmap, const CUtensorMap &amap, int cgroups,
+                             size_t smem, cudaStream_t st) {
     auto k = k_rowspec_tc<N>;
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    k<<<dim3(a.P * N * TcShape<N>::NTILES, cgroups), kTcRoleThreads, smem, st>>>(a, hmap, are, aim);
+    k<<<dim3(a.P * N * TcShape<N>::NTILES, cgroups), kTcRoleThreads, smem, st>>>(a, hmap, amap);
     return cudaGetLastError();
 }
 
-cudaError_t launch_rowspec(int N, const RowSpecArgs &a, const CUtensorMap &hmap, const CUtensorMap &amap_re,
-                           const CUtensorMap &amap_im, int cgroups, size_t smem, cudaStream_t st) {
+cudaError_t launch_rowspec(int N, const RowSpecArgs &a, const CUtensorMap &hmap, const CUtensorMap &amap, int cgroups,
+                           size_t smem, cudaStream_t st) {
     switch (N) {
-        case 32: return launch_rowspec_t<32>(a, hmap, amap_re, amap_im, cgroups, smem, st);
-        case 64: return launch_rowspec_t<64>(a, hmap, amap_re, amap_im, cgroups, smem, st);
-        case 128: return launch_rowspec_t<128>(a, hmap, amap_re, amap_im, cgroups, smem, st);
-        case 256: return launch_rowspec_t<256>(a, hmap, amap_re, amap_im, cgroups, smem, st);
-        case 512: return launch_rowspec_t<512>(a, hmap, amap_re, amap_im, cgroups, smem, st);
+        case 32: return launch_rowspec_t<32>(a, hmap, amap, cgroups, smem, st);
+        case 64: return launch_rowspec_t<64>(a, hmap, amap, cgroups, smem, st);
+        case 128: return launch_rowspec_t<128>(a, hmap, amap, cgroups, smem, st);
+        case 256: return launch_rowspec_t<256>(a, hmap, amap, cgroups, smem, st);
+        case 512: return launch_rowspec_t<512>(a, hmap, amap, cgroups, smem, st);
     }
     return cudaErrorInvalidValue;
 }
 
-cudaError_t encode_plane_map(CUtensorMap *map, void *plane, int Tpad, long long rows, int box_rows) {
+// Load map of the voltage planes: (sample, plane row, re / im), the imaginary plane im_off bytes after the real one
+// (a multiple of the row's bytes); box 64 samples x box_rows rows x both planes, 128-byte swizzle.
+cudaError_t encode_plane_map(CUtensorMap *map, void *plane, int Tpad, long long rows, size_t im_off, int box_rows) {
     void *fn = nullptr;
     cudaDriverEntryPointQueryResult q;
     cudaError_t e = cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &q);
@@ -580,11 +572,11 @@ cudaError_t encode_plane_map(CUtensorMap *map, void *plane, int Tpad, long long 
     using Encode = CUresult (*)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
                                 const cuuint64_t *, const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave,
                                 CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-    const cuuint64_t dims[2] = {(cuuint64_t)Tpad, (cuuint64_t)rows};
-    const cuuint64_t strides[1] = {(cuuint64_t)Tpad * 2};
-    const cuuint32_t box[2] = {64, (cuuint32_t)box_rows};
-    const cuuint32_t estr[2] = {1, 1};
-    const CUresult r = reinterpret_cast<Encode>(fn)(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, plane, dims, strides, box,
+    const cuuint64_t dims[3] = {(cuuint64_t)Tpad, (cuuint64_t)rows, 2};
+    const cuuint64_t strides[2] = {(cuuint64_t)Tpad * 2, (cuuint64_t)im_off};
+    const cuuint32_t box[3] = {64, (cuuint32_t)box_rows, 2};
+    const cuuint32_t estr[3] = {1, 1, 1};
+    const CUresult r = reinterpret_cast<Encode>(fn)(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 3, plane, dims, strides, box,
                                                     estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
                                                     CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                                                     CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
