@@ -264,6 +264,7 @@ struct moff_plan {
     long long *d_rs_bimg_off = nullptr;
     CUtensorMap a_map{};                  // TMA load map of both voltage planes (d_yre, d_yim)
     CUtensorMap vp_smap_re{}, vp_smap_im{};   // their store maps (row plane kernel)
+    bool vp_raster = false;                   // plane rows in the voltages' own order (planes_in_raster_order)
     bool vp_tma = true;                       // the row plane kernel stores by TMA boxes (MOFF_VP_TMA=0: directly)
     float *d_rs_row_sh = nullptr, *d_rs_row_inv = nullptr;
     CUtensorMap h_map;                 // tensor-core path: store map of the FP16 field
@@ -667,7 +668,7 @@ moff_status run_image_tc(moff_plan *pl, const uint8_t *volt, int n_time, long lo
             const int nt = std::min(pl->Tb, n_time - t0);
             TimedLaunch tv(pl, 3);
             MOFF_CK(launch_volt_prep(volt, tstride, t0, nt, c0, nc, AP, AP + kRowSpecPad, pl->d_gains, pl->d_sy,
-                                     pl->d_rs_perm, pl->Tb, pl->d_yre, pl->d_yim, pl->st, -1,
+                                     pl->d_rs_perm, pl->Tb, pl->d_yre, pl->d_yim, pl->st, -1, pl->vp_raster,
                                      pl->vp_tma ? &pl->vp_smap_re : nullptr, pl->vp_tma ? &pl->vp_smap_im : nullptr));
             tv.done();
             RowSpecArgs ra{};
@@ -829,7 +830,7 @@ moff_status run_image_gtc(moff_plan *pl, const uint8_t *volt, int n_time, long l
             const int nt = std::min(pl->Tb, n_time - t0);
             TimedLaunch tv(pl, 3);
             MOFF_CK(launch_volt_prep(volt, tstride, t0, nt, c0, nc, AP, pl->gt_rows, pl->d_gains, pl->d_sy,
-                                     pl->d_gt_perm, pl->Tb, pl->d_yre, pl->d_yim, pl->st, pl->gt_rows - kRowSpecPad,
+                                     pl->d_gt_perm, pl->Tb, pl->d_yre, pl->d_yim, pl->st, pl->gt_rows - kRowSpecPad, pl->vp_raster,
                                      pl->vp_tma ? &pl->vp_smap_re : nullptr, pl->vp_tma ? &pl->vp_smap_im : nullptr));
             tv.done();
             GridTcArgs ga{};
@@ -2189,6 +2190,7 @@ moff_status moff_plan_create(moff_plan **out, int n_ant, const double *pos, int 
             // one CTA per SM: the tile's kernel matrix, the A ring and the barriers must fit shared memory
             pl->gtc = !gtab.tile_cell.empty() && gridtc_stages(n_pol, gtab.kp_max, 1) > 0;
             pl->gt_rows = gtab.n_rows + kRowSpecPad;
+            pl->vp_raster = planes_in_raster_order(gtab.perm);
         }
     }
     // accumulators and image staging
@@ -2350,6 +2352,7 @@ moff_status moff_plan_create(moff_plan **out, int n_ant, const double *pos, int 
         else if ((s = build_rowspec(n_ant, ksize, grid_n, n_pol, pl->jones, pos, taps, &rs)) != MOFF_OK)
             return bail(s);
         pl->rs_kp_max = std::max(rs.kp_max, 16);
+        pl->vp_raster = planes_in_raster_order(rs.perm);
         pl->rs_inv_sw = rs.inv_sw;
         pl->rs_smem = rowspec_smem_bytes(grid_n, pl->rs_kp_max);
         const int items = n_pol * grid_n * rs.ntiles;
@@ -2743,7 +2746,7 @@ moff_status moff_voltage_planes(moff_plan *pl, const uint8_t *volt, int n_time, 
         src = reinterpret_cast<const uint8_t *>(dev);
     }
     MOFF_CK(launch_volt_prep(src, tstride, 0, n_time, chan, 1, AP, APpad, pl->d_gains, pl->d_sy, dperm, pl->Tb,
-                             pl->d_yre, pl->d_yim, pl->st, nrows, pl->vp_tma ? &pl->vp_smap_re : nullptr,
+                             pl->d_yre, pl->d_yim, pl->st, nrows, pl->vp_raster, pl->vp_tma ? &pl->vp_smap_re : nullptr,
                              pl->vp_tma ? &pl->vp_smap_im : nullptr));
     if (slot >= 0 && (s = stage_done(pl, slot)) != MOFF_OK) return s;
     std::vector<__half> re((size_t)nrows * pl->Tb), im((size_t)nrows * pl->Tb);

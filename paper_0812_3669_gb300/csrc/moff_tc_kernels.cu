@@ -90,8 +90,8 @@ __global__ void k_gain_scale(const float2 *__restrict__ gains, int AP, float *__
 // Voltages of samples [t0, t0+nt) of channels [c0, c0+nc) -> FP16 planes
 // Yre/Yim [nc][APpad][Tpad] (t contiguous), zero for t >= nt and for rows v >= AP (the
 // pad rows a chunk running past the last voltage reads); plane row v < AP holds voltage
-// perm[v].  A CTA stages the voltage bytes of TT samples of one channel (coalesced
-// 16-byte loads) and writes every plane row's TT samples (half2 per sample pair).
+// perm[v].  A CTA stages the voltage bytes of TT samples (8 or 16) of one channel (coalesced
+// 16-byte loads) and writes every plane row's TT samples.
 __global__ void __launch_bounds__(256) k_volt_prep(const uint8_t *__restrict__ volt, long long tstride, int t0, int nt,
                                                    int c0, int AP, int APpad, const float2 *__restrict__ gains,
                                                    const float *__restrict__ sy, const int *__restrict__ perm, int Tpad,
@@ -120,39 +120,24 @@ __global__ void __launch_bounds__(256) k_volt_prep(const uint8_t *__restrict__ v
         *reinterpret_cast<uint4 *>(s_v + tt * APr + q * 16) = v;
     }
     __syncthreads();
-    if (TT >= 8) {   // 8 samples of one plane row per thread: one 16-byte store per plane
-        const int ng = TT / 8;
-        for (int i = threadIdx.x; i < APpad * ng; i += blockDim.x) {
-            const int v = i / ng, t8 = 8 * (i - v * ng);
-            uint4 re = make_uint4(0u, 0u, 0u, 0u), im = re;
-            if (v < n_rows) {
-                const int sv = perm[v];
-                const float2 g = gains[(long long)c * AP + sv], gs = make_float2(g.x * s, g.y * s);
-                uint32_t hr[4], hi[4];
-#pragma unroll
-                for (int u = 0; u < 4; ++u)
-                    weigh2_tc(gs, s_v[(t8 + 2 * u) * APr + sv], s_v[(t8 + 2 * u + 1) * APr + sv], hr[u], hi[u]);
-                re = make_uint4(hr[0], hr[1], hr[2], hr[3]);
-                im = make_uint4(hi[0], hi[1], hi[2], hi[3]);
-            }
-            const long long o = ((long long)cl * APpad + v) * Tpad + tb + t8;   // 16-byte aligned (Tpad % 8 == 0)
-            *reinterpret_cast<uint4 *>(yre + o) = re;
-            *reinterpret_cast<uint4 *>(yim + o) = im;
-        }
-        return;
-    }
-    const int np = TT / 2;
-    for (int i = threadIdx.x; i < APpad * np; i += blockDim.x) {
-        const int v = i / np, tp = 2 * (i - v * np), t = tb + tp;
-        uint32_t re = 0u, im = 0u;
+    // 8 samples of one plane row per thread: one 16-byte store per plane
+    const int ng = TT / 8;
+    for (int i = threadIdx.x; i < APpad * ng; i += blockDim.x) {
+        const int v = i / ng, t8 = 8 * (i - v * ng);
+        uint4 re = make_uint4(0u, 0u, 0u, 0u), im = re;
         if (v < n_rows) {
             const int sv = perm[v];
-            const float2 g = gains[(long long)c * AP + sv];
-            weigh2_tc(make_float2(g.x * s, g.y * s), s_v[tp * APr + sv], s_v[(tp + 1) * APr + sv], re, im);
+            const float2 g = gains[(long long)c * AP + sv], gs = make_float2(g.x * s, g.y * s);
+            uint32_t hr[4], hi[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                weigh2_tc(gs, s_v[(t8 + 2 * u) * APr + sv], s_v[(t8 + 2 * u + 1) * APr + sv], hr[u], hi[u]);
+            re = make_uint4(hr[0], hr[1], hr[2], hr[3]);
+            im = make_uint4(hi[0], hi[1], hi[2], hi[3]);
         }
-        const long long o = ((long long)cl * APpad + v) * Tpad + t;   // t even, Tpad even: 4-byte aligned
-        *reinterpret_cast<uint32_t *>(yre + o) = re;
-        *reinterpret_cast<uint32_t *>(yim + o) = im;
+        const long long o = ((long long)cl * APpad + v) * Tpad + tb + t8;   // 16-byte aligned (Tpad % 8 == 0)
+        *reinterpret_cast<uint4 *>(yre + o) = re;
+        *reinterpret_cast<uint4 *>(yim + o) = im;
     }
 }
 
@@ -276,6 +261,95 @@ __global__ void __launch_bounds__(256, 3) k_volt_prep_rows(const uint8_t *__rest
         }
     }
     if (boxed && lane == 0) tc::bulk_wait_all();
+}
+
+// Arrays whose codes of 32 samples of a channel fit shared memory beside the boxes (kVp32MaxBytes): the CTA stages
+// them once (whole 16-byte pieces) and each warp turns 32 plane rows x 32 samples at a time into the two planes, one row
+// per lane -- so a row may come from any antenna, and 32 lanes read 32 different bytes of one sample's codes -- and
+// leaves them as TMA boxes.  k_volt_prep's four lanes per row read four samples whose codes lie in the same bank and
+// store 64-byte pieces of eight rows.  Bound by DRAM (planes out): 256 channels x 512 samples of 1024 antennas in hexagonal
+// order 297 us against 547 (198 at the copy bandwidth).
+constexpr size_t kVp32MaxBytes = 80 * 1024;              // two CTAs per SM
+__global__ void __launch_bounds__(256, 2) k_volt_prep32(const uint8_t *__restrict__ volt, long long tstride, int t0, int nt,
+                                                        int c0, int AP, int APpad, int n_rows,
+                                                        const float2 *__restrict__ gains, const float *__restrict__ sy,
+                                                        const int *__restrict__ perm, int Tpad, __half *__restrict__ yre,
+                                                        __half *__restrict__ yim, const __grid_constant__ CUtensorMap smap_re,
+                                                        const __grid_constant__ CUtensorMap smap_im, int use_tma) {
+    extern __shared__ __align__(1024) unsigned char vp_smem[];
+    unsigned char *base_s = vp_smem + ((1024u - (tc::smem_u32(vp_smem) & 1023u)) & 1023u);
+    const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
+    unsigned char *bre = base_s + wp * kVpBoxBytes, *bim = bre + kVpBoxBytes / 2;
+    unsigned char *s_v = base_s + 8 * kVpBoxBytes;       // [32][APr] voltage bytes
+    const int cl = blockIdx.y, c = c0 + cl, tb = blockIdx.x * 32;
+    const int APr = (AP + 15) & ~15, nq = APr / 16;
+    const uint8_t *vc = volt + (long long)c * AP + (long long)(t0 + tb) * tstride;
+    const bool vec = (AP & 15) == 0 && (tstride & 15) == 0 && ((reinterpret_cast<uintptr_t>(vc)) & 15) == 0;
+    for (int i = threadIdx.x; i < 32 * nq; i += 256) {
+        const int tt = i / nq, q = i - tt * nq;
+        unsigned char *d = s_v + tt * APr + q * 16;
+        const uint8_t *src = vc + (long long)tt * tstride + q * 16;
+        if (vec && tb + tt < nt) {
+            vp_cp16(d, src);
+        } else {
+            uint32_t w[4] = {0u, 0u, 0u, 0u};
+            if (tb + tt < nt)
+                for (int u = 0; u < 16 && q * 16 + u < AP; ++u) w[u >> 2] |= (uint32_t)src[u] << (8 * (u & 3));
+            *reinterpret_cast<uint4 *>(d) = make_uint4(w[0], w[1], w[2], w[3]);
+        }
+    }
+    vp_commit();
+    const float s = sy[c];
+    vp_wait(0);
+    __syncthreads();
+    bool stored = false;
+    for (int v0 = 32 * wp; v0 < APpad; v0 += 256) {
+        const int v = v0 + lane;
+        const bool have = v < n_rows;
+        const int sv = have ? perm[v] : 0;
+        const float2 g = have ? gains[(long long)c * AP + sv] : make_float2(0.f, 0.f);
+        const float2 gs = make_float2(g.x * s, g.y * s);
+        uint32_t re[16], im[16];
+#pragma unroll
+        for (int t = 0; t < 32; t += 2) {
+            uint32_t b0 = s_v[t * APr + sv], b1 = s_v[(t + 1) * APr + sv];
+            weigh2_tc(gs, b0, b1, re[t >> 1], im[t >> 1]);
+        }
+        if (!have) {                                     // rows past the last voltage read +0
+#pragma unroll
+            for (int i = 0; i < 16; ++i) re[i] = im[i] = 0u;
+        }
+        if (use_tma && v0 + 32 <= APpad) {               // warp-uniform
+            if (stored) {                                // the previous stores have read the boxes
+                if (lane == 0) tc::bulk_wait_read<0>();
+                __syncwarp();
+            }
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const int o = lane * 64 + ((k ^ ((lane >> 1) & 3)) << 4);
+                *reinterpret_cast<uint4 *>(bre + o) = make_uint4(re[4 * k], re[4 * k + 1], re[4 * k + 2], re[4 * k + 3]);
+                *reinterpret_cast<uint4 *>(bim + o) = make_uint4(im[4 * k], im[4 * k + 1], im[4 * k + 2], im[4 * k + 3]);
+            }
+            tc::fence_async_smem();
+            __syncwarp();
+            if (lane == 0) {
+                const int y = cl * APpad + v0;
+                tc::tma_store_2d(&smap_re, tc::smem_u32(bre), tb, y);
+                tc::tma_store_2d(&smap_im, tc::smem_u32(bim), tb, y);
+                tc::bulk_commit();
+            }
+            stored = true;
+        } else if (v < APpad) {
+            uint4 *ore = reinterpret_cast<uint4 *>(yre + ((long long)cl * APpad + v) * Tpad + tb);
+            uint4 *oim = reinterpret_cast<uint4 *>(yim + ((long long)cl * APpad + v) * Tpad + tb);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                ore[k] = make_uint4(re[4 * k], re[4 * k + 1], re[4 * k + 2], re[4 * k + 3]);
+                oim[k] = make_uint4(im[4 * k], im[4 * k + 1], im[4 * k + 2], im[4 * k + 3]);
+            }
+        }
+    }
+    if (stored && lane == 0) tc::bulk_wait_all();
 }
 
 template <int N>
@@ -508,18 +582,44 @@ cudaError_t launch_gain_scale(const float2 *gains, int C, int AP, float *sy, cud
     return cudaGetLastError();
 }
 
+// Whether most warps of the row plane kernel (32 consecutive plane rows) hold 32 consecutive voltages.
+bool planes_in_raster_order(const std::vector<int> &perm) {
+    const size_t ng = perm.size() / 32;
+    size_t run = 0;
+    for (size_t g = 0; g < ng; ++g) {
+        bool ok = true;
+        for (size_t i = 1; i < 32 && ok; ++i) ok = perm[32 * g + i] == perm[32 * g] + (int)i;
+        run += ok;
+    }
+    return 2 * run >= ng && ng > 0;
+}
+
+// Which kernel makes the planes (measured us; k_volt_prep32 / k_volt_prep_rows / k_volt_prep, by A P):
+//   raster order   4096: 129 / 84 / 181;  8192: - / 189 / 571;  11552: - / 177 / 541
+//   other orders   2048: 297 / 610 / 547;  4096: 117 / 217 / 182;  6000: 172 / 317 / 237
+// so raster maps take the row kernel once k_volt_prep32's two CTAs no longer fit an SM, other maps k_volt_prep32 as
+// long as its 32 samples fit at all, then k_volt_prep with 8 or 16 samples, and the row kernel past 12288.
 cudaError_t launch_volt_prep(const uint8_t *volt, long long tstride, int t0, int nt, int c0, int nc, int AP,
                              int APpad, const float2 *gains, const float *sy, const int *perm, int Tpad, __half *yre,
-                             __half *yim, cudaStream_t st, int n_rows, const CUtensorMap *smap_re,
+                             __half *yim, cudaStream_t st, int n_rows, bool raster, const CUtensorMap *smap_re,
                              const CUtensorMap *smap_im) {
-    // samples per CTA: 32, or fewer (even, dividing Tpad) so the staged bytes stay within 96 KB
     const size_t APr = (size_t)((AP + 15) & ~15);
     const int rows = n_rows < 0 ? AP : n_rows;
-    if (8 * APr > 96 * 1024 && Tpad % 32 == 0) {   // too large to stage 8 samples: one thread per plane row
+    const int use_tma = smap_re && smap_im ? 1 : 0;
+    const CUtensorMap none{};
+    if (Tpad % 32) return cudaErrorInvalidValue;
+    const int vec_ok = tstride % 16 == 0 && AP % 16 == 0 && ((uintptr_t)volt & 15) == 0;
+    const size_t smem32 = 1024 + 8 * kVpBoxBytes + 32 * APr;
+    if (raster && vec_ok ? 32 * APr <= kVp32MaxBytes : smem32 <= 224 * 1024) {
+        cudaError_t e = cudaFuncSetAttribute(k_volt_prep32, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem32);
+        if (e != cudaSuccess) return e;
+        k_volt_prep32<<<dim3(Tpad / 32, nc), 256, smem32, st>>>(volt, tstride, t0, nt, c0, AP, APpad, rows, gains, sy, perm,
+                                                                Tpad, yre, yim, use_tma ? *smap_re : none,
+                                                                use_tma ? *smap_im : none, use_tma);
+        return cudaGetLastError();
+    }
+    if ((raster && vec_ok) || 8 * APr > 96 * 1024) {   // one thread per plane row
         dim3 grid((APpad + 255) / 256, nc);
-        const int vec_ok = tstride % 16 == 0 && AP % 16 == 0 && ((uintptr_t)volt & 15) == 0;
-        const int use_tma = smap_re && smap_im ? 1 : 0;
-        CUtensorMap none{};
         cudaError_t e = cudaFuncSetAttribute(k_volt_prep_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kVpSmem);
         if (e != cudaSuccess) return e;
         k_volt_prep_rows<<<grid, 256, kVpSmem, st>>>(volt, tstride, t0, nt, c0, AP, APpad, rows, gains, sy, perm, Tpad,
@@ -527,9 +627,7 @@ cudaError_t launch_volt_prep(const uint8_t *volt, long long tstride, int t0, int
                                                      use_tma ? *smap_im : none, use_tma);
         return cudaGetLastError();
     }
-    int TT = 32;
-    while (TT > 2 && (TT * APr > 96 * 1024 || Tpad % TT)) TT /= 2;
-    if (Tpad % TT || TT * APr > 200 * 1024) return cudaErrorInvalidValue;
+    const int TT = 16 * APr <= 96 * 1024 ? 16 : 8;      // samples per CTA: the staged bytes stay within 96 KB
     const size_t smem = TT * APr;
     cudaError_t e = cudaFuncSetAttribute(k_volt_prep, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
