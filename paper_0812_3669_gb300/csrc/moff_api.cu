@@ -122,9 +122,26 @@ std::vector<float2> pass_twiddles_n(int n) {
 
 bool is_pow2(long long v) { return v > 0 && (v & (v - 1)) == 0; }
 
-__global__ void k_to_f32(const double *__restrict__ a, float *__restrict__ o, long long n) {
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
+// FP64 sums -> FP32 image; RESET also starts the next integration (one pass instead of a memset behind it).  Nothing is
+// read or reset once a kernel of the plan has recorded a failed wait (err).
+template <bool RESET>
+__global__ void __launch_bounds__(256) k_to_f32(double *__restrict__ a, float *__restrict__ o, long long n4,
+                                                const int *__restrict__ err) {
+    if (err && *err) return;
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n4; i += (long long)gridDim.x * blockDim.x) {
+        double2 *p = reinterpret_cast<double2 *>(a) + 2 * i;
+        const double2 u = p[0], v = p[1];
+        if (RESET) p[0] = p[1] = make_double2(0.0, 0.0);
+        reinterpret_cast<float4 *>(o)[i] = make_float4((float)u.x, (float)u.y, (float)v.x, (float)v.y);
+    }
+}
+__global__ void __launch_bounds__(256) k_to_f32_any(double *__restrict__ a, float *__restrict__ o, long long n,
+                                                    const int *__restrict__ err, int reset) {
+    if (err && *err) return;
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
         o[i] = (float)a[i];
+        if (reset) a[i] = 0.0;
+    }
 }
 
 }  // namespace
@@ -201,9 +218,14 @@ cudaError_t launch_persist(int N, int P, int cpl, bool wide, const PersistArgs &
     return cudaErrorInvalidValue;
 }
 
-cudaError_t launch_to_f32(const double *acc, float *out, long long n, cudaStream_t st) {
-    const long long blocks = std::min<long long>((n + 255) / 256, 152LL * 16);
-    k_to_f32<<<(unsigned)std::max<long long>(blocks, 1), 256, 0, st>>>(acc, out, n);
+cudaError_t launch_to_f32(double *acc, float *out, long long n, cudaStream_t st, const int *err, bool reset) {
+    // images are whole multiples of 1024 values; an output that is no 16-byte aligned buffer goes value by value
+    const bool vec = n % 4 == 0 && (((uintptr_t)acc | (uintptr_t)out) & 15) == 0;
+    const long long m = vec ? n / 4 : n;
+    const unsigned blocks = (unsigned)std::max(1LL, std::min<long long>((m + 255) / 256, 152LL * 16));
+    if (!vec) k_to_f32_any<<<blocks, 256, 0, st>>>(acc, out, n, err, reset ? 1 : 0);
+    else if (reset) k_to_f32<true><<<blocks, 256, 0, st>>>(acc, out, m, err);
+    else k_to_f32<false><<<blocks, 256, 0, st>>>(acc, out, m, err);
     return cudaGetLastError();
 }
 
@@ -261,6 +283,7 @@ struct moff_plan {
     float rs_inv_sw = 1.f;
     int *d_rs_kp = nullptr, *d_rs_chunk_row = nullptr, *d_rs_chunk_off = nullptr, *d_rs_perm = nullptr,
         *d_err = nullptr;
+    int *h_err = nullptr;              // pinned copy of the status word d_err
     long long *d_rs_bimg_off = nullptr;
     CUtensorMap a_map{};                  // TMA load map of both voltage planes (d_yre, d_yim)
     CUtensorMap vp_smap_re{}, vp_smap_im{};   // their store maps (row plane kernel)
@@ -398,6 +421,7 @@ void destroy_plan(moff_plan *pl) {
     if (pl->st) cudaStreamSynchronize(pl->st);
     if (pl->cst) cudaStreamSynchronize(pl->cst);
     for (void *p : pl->allocs) cudaFree(p);
+    if (pl->h_err) cudaFreeHost(pl->h_err);
     for (int i = 0; i < 2; ++i) {
         if (pl->ev_copied[i]) cudaEventDestroy(pl->ev_copied[i]);
         if (pl->ev_consumed[i]) cudaEventDestroy(pl->ev_consumed[i]);
@@ -414,17 +438,21 @@ void destroy_plan(moff_plan *pl) {
     delete pl;
 }
 
+// Without a limit the runtime waits; with one, polling without pause for the first 0.2 ms (a pause of 50 us takes
+// about 100, which a short block's two waits felt: 200 of the 362 us of a tiny array's block), then with pauses.
 moff_status wait_event(cudaEvent_t ev, int timeout_ms) {
+    if (timeout_ms < 0) {
+        const cudaError_t e = cudaEventSynchronize(ev);
+        return e == cudaSuccess ? MOFF_OK : fail(MOFF_ECUDA, "waiting for the GPU: %s", cudaGetErrorString(e));
+    }
     const auto t0 = std::chrono::steady_clock::now();
     for (;;) {
         cudaError_t e = cudaEventQuery(ev);
         if (e == cudaSuccess) return MOFF_OK;
         if (e != cudaErrorNotReady) return fail(MOFF_ECUDA, "waiting for the GPU: %s", cudaGetErrorString(e));
-        if (timeout_ms >= 0) {
-            const auto ms = std::chrono::duration_cast<std::chrono::milliseconds>(std::chrono::steady_clock::now() - t0).count();
-            if (ms >= timeout_ms) return fail(MOFF_ETIMEDOUT, "GPU work not finished after %d ms", timeout_ms);
-        }
-        std::this_thread::sleep_for(std::chrono::microseconds(50));
+        const auto us = std::chrono::duration_cast<std::chrono::microseconds>(std::chrono::steady_clock::now() - t0).count();
+        if (us >= 1000LL * timeout_ms) return fail(MOFF_ETIMEDOUT, "GPU work not finished after %d ms", timeout_ms);
+        if (us > 200) std::this_thread::sleep_for(std::chrono::microseconds(50));
     }
 }
 
@@ -2432,6 +2460,10 @@ moff_status moff_plan_create(moff_plan **out, int n_ant, const double *pos, int 
     }
     pl->scratch_bytes = align_up(pl->h_bytes, 1024) + (pl->tc && !pl->dft ? 2 * align_up(pl->y_bytes, 1024) : 0) +
                         (pl->gtc ? align_up(pl->h_bytes, 1024) + 2 * align_up(pl->y_bytes, 1024) : 0);
+    if (pl->d_err && cudaMallocHost(&pl->h_err, sizeof(int)) != cudaSuccess) {
+        cudaGetLastError();
+        return bail(fail(MOFF_ENOMEM, "pinned status word"));
+    }
     if (cudaDeviceSynchronize() != cudaSuccess) return bail(fail(MOFF_ECUDA, "plan set-up failed"));
     if (const char *lg = getenv("MOFF_LOG"); lg && atoi(lg) > 0) {   // the plan's decisions, one line on stderr
         static const char *routes[4] = {"fp32", "fp16_rowspec", "fp16_dft", "fp16_tcgrid"};
@@ -2779,22 +2811,33 @@ moff_status moff_read_image(moff_plan *pl, float *out, long long *n_samples, int
     moff_status s = check_plan(pl);
     if (s != MOFF_OK) return s;
     if (!out) return fail(MOFF_EINVAL, "out is NULL");
+    const long long n = (long long)pl->C * pl->nprod * pl->N * pl->N;
+    auto done = [&]() -> moff_status {
+        if (n_samples) *n_samples = pl->n_samples;
+        if (reset) {
+            pl->n_samples = 0;
+            if (pl->auto_on) {   // the autocorrelation sums follow the integration
+                MOFF_CK(cudaMemsetAsync(pl->d_auto_pw, 0, (size_t)pl->C * pl->A * 3 * 16, pl->st));
+                pl->auto_samples = 0;
+            }
+        }
+        return MOFF_OK;
+    };
+    if (out_on_device) {   // conversion, reset and status word behind the plan's work, one wait for all of it
+        if (timeout_ms >= 0 && (s = sync_plan(pl, timeout_ms)) != MOFF_OK) return s;
+        MOFF_CK(launch_to_f32(pl->d_acc, out, n, pl->st, pl->d_err, reset != 0));
+        if (pl->d_err) MOFF_CK(cudaMemcpyAsync(pl->h_err, pl->d_err, sizeof(int), cudaMemcpyDeviceToHost, pl->st));
+        if ((s = sync_plan(pl, -1)) != MOFF_OK) return s;
+        if (pl->d_err && *pl->h_err) return check_device_err(pl);
+        return done();
+    }
     if ((s = sync_plan(pl, timeout_ms)) != MOFF_OK) return s;
     if ((s = check_device_err(pl)) != MOFF_OK) return s;
-    const long long n = (long long)pl->C * pl->nprod * pl->N * pl->N;
-    MOFF_CK(launch_to_f32(pl->d_acc, out_on_device ? out : pl->d_img, n, pl->st));
-    if (!out_on_device) MOFF_CK(cudaMemcpyAsync(out, pl->d_img, (size_t)n * 4, cudaMemcpyDeviceToHost, pl->st));
+    MOFF_CK(launch_to_f32(pl->d_acc, pl->d_img, n, pl->st));
+    MOFF_CK(cudaMemcpyAsync(out, pl->d_img, (size_t)n * 4, cudaMemcpyDeviceToHost, pl->st));
     if ((s = sync_plan(pl, -1)) != MOFF_OK) return s;
-    if (n_samples) *n_samples = pl->n_samples;
-    if (reset) {
-        MOFF_CK(cudaMemsetAsync(pl->d_acc, 0, (size_t)n * 8, pl->st));
-        pl->n_samples = 0;
-        if (pl->auto_on) {   // the autocorrelation sums follow the integration
-            MOFF_CK(cudaMemsetAsync(pl->d_auto_pw, 0, (size_t)pl->C * pl->A * 3 * 16, pl->st));
-            pl->auto_samples = 0;
-        }
-    }
-    return MOFF_OK;
+    if (reset) MOFF_CK(cudaMemsetAsync(pl->d_acc, 0, (size_t)n * 8, pl->st));
+    return done();
 }
 
 moff_status moff_sync(moff_plan *pl, int timeout_ms) {
