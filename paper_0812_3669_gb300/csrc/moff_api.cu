@@ -1033,7 +1033,7 @@ moff_status fail_msg(moff_status s, const char *msg) { return fail(s, "%s", msg)
 // lists (host only).  The stripe height is the largest power of two <= 16
 // whose lists fit the gridding kernel's shared-memory budget.
 moff_status build_bins(int A, int K, int N, int P, bool jones, const double *pos, const float *taps, Bins *b,
-                       const GridChoice *force, bool dft) {
+                       const GridChoice *force, bool dft, bool narrow) {
     const int h = K / 2;
     std::vector<int> ax(A), ay(A);
     for (int a = 0; a < A; ++a) {
@@ -1048,8 +1048,8 @@ moff_status build_bins(int A, int K, int N, int P, bool jones, const double *pos
     const int tw_total = fft_tw_total(N);
     const char *wide_env = getenv("MOFF_GRID_WIDE");
     // the tensor-core row transform runs on stripes of grid_fft_rows(N) rows with entries through L2
-    const bool wide = !dft && (force ? force->wide : (wide_env && atoi(wide_env) != 0));
-    const int F = grid_fft_rows(N) * (wide ? 2 : 1);
+    bool wide = !dft && (force ? force->wide : (wide_env && atoi(wide_env) != 0));
+    int F = grid_fft_rows(N) * (wide ? 2 : 1);
     const size_t budget = 110 * 1024;   // two CTAs per SM
     const size_t big = 225 * 1024;      // one CTA per SM: dense arrays, where more samples per pass reuse each tap
     // Contributions per grid cell (p_out, row, col), independent of the stripe shape.
@@ -1076,8 +1076,9 @@ moff_status build_bins(int A, int K, int N, int P, bool jones, const double *pos
     const bool quads = force ? force->quads : (quads_env && atoi(quads_env) != 0);
     const bool pairs = !quads && (force ? force->pairs : !(pairs_env && atoi(pairs_env) == 0));
     struct Cand { int tb, rows, nloc; long long entries; size_t sm_staged, sm_plain; };
+    auto shapes = [&](int F, std::initializer_list<int> tbs) {
     std::vector<Cand> cands;
-    for (int tb = 8; tb >= 1; tb /= 2) {
+    for (int tb : tbs) {
         int rows = F / (tb * P);
         if (rows < 1) continue;
         rows = std::min(rows, N);
@@ -1111,12 +1112,51 @@ moff_status build_bins(int A, int K, int N, int P, bool jones, const double *pos
                 dft ? grid_smem_bytes_dft(N, P, tb, rows, mnl) : grid_smem_bytes(N, P, tb, rows, mnl, tw_total, 0, pairs)};
         cands.push_back(cd);
     }
+    return cands;
+    };
+    std::vector<Cand> cands;
     // Entries are read through L2 by default (more CTAs per SM measured faster
     // than shared-memory staging); MOFF_GRID_STAGE=1 prefers staging.
     const char *stage_env = getenv("MOFF_GRID_STAGE");
     const bool prefer_staged = !dft && stage_env && atoi(stage_env) != 0;
     const Cand *pick = nullptr;
     bool staged = false;
+    // The rule's first choice: cell pairs on stripes of twice the rows with 8 or 4 samples per pass, on one CTA per SM
+    // if need be, by the grid and by the contributions per cell of the reached rows (rho): many favour 8 samples (each
+    // kernel entry read once for more of them), few the four CTAs per SM that 4 samples leave room for; on the 512 grid
+    // few favour the narrow stripes.  Measured ms per chunk (wide 8 / wide 4 / narrow 4 samples):
+    //   64 grid    rho 1.4  1.16 / 1.32 / 1.17    128 grid  rho 0.7  1.89 / 1.53 / 1.95    256 grid  rho 1.2  2.07 / 1.77 / 2.30
+    //              rho 12   0.45 / -    / 0.48              rho 3.0  2.79 / 2.64 / 3.00              rho 5.9  0.69 / 0.69 / 0.87
+    //   512 grid   rho 1.7  1.60 / 1.69 / 1.47              rho 3.7  0.94 / 0.97 / 1.04              rho 8.2  1.19 / 1.33 / 1.73
+    //              rho 2.9  0.69 / -    / 0.72              rho 12   1.57 / 1.77 / 1.82
+    //              rho 6.0  does not fit / 2.56 / 2.87 (one sample, which the rule took before: 3.06)
+    // Each cell's sum keeps its order in every shape.
+    if (!force && !dft && !narrow && !wide_env && pairs && !prefer_staged) {
+        long long total = 0;
+        int reached = 0;
+        for (int y = 0; y < N; ++y) {
+            long long row = 0;
+            for (int po = 0; po < P; ++po)
+                for (int x = 0; x < N; ++x) row += cnt_all[((size_t)po * N + y) * N + x];
+            total += row;
+            reached += row > 0;
+        }
+        const double rho = reached ? (double)total / ((double)reached * N * P) : 0.0;
+        std::vector<int> wants;
+        if (N <= 64) wants = {8};
+        else if (N <= 256) wants = rho >= 3.3 ? std::vector<int>{8, 4} : std::vector<int>{4};
+        else if (rho >= 2.3) wants = {8, 4};
+        for (int want : wants) {
+            const std::vector<Cand> w = shapes(2 * F, {want});
+            if (w.empty() || w[0].sm_plain > big) continue;
+            cands = w;
+            pick = &cands[0];
+            wide = true;
+            F *= 2;
+            break;
+        }
+    }
+    if (!pick) cands = shapes(F, {8, 4, 2, 1});
     if (force) {
         for (const Cand &cd : cands)
             if (cd.tb == force->tb) {
@@ -2345,7 +2385,11 @@ moff_status moff_plan_create(moff_plan **out, int n_ant, const double *pos, int 
         if ((s = bin_plan(pl, pos, taps, pl->tune_source ? &tuned : nullptr)) != MOFF_OK) return bail(s);
         if (pl->persist && (pl->tb != 4 || pl->staged)) {
             GridChoice ch{4, false, pl->pairs, pl->wide, pl->quads};
-            if ((s = bin_plan(pl, pos, taps, &ch)) != MOFF_OK) return bail(s);
+            if ((s = bin_plan(pl, pos, taps, &ch)) != MOFF_OK && ch.wide) {   // half the rows need less shared memory
+                ch.wide = false;
+                s = bin_plan(pl, pos, taps, &ch);
+            }
+            if (s != MOFF_OK) return bail(s);
         }
     }
     if (pl->dft) {   // the column kernel's width: the default, or timed (needs the plan's reached-row mask)

@@ -327,7 +327,7 @@ struct GridChoice {
 // force = nullptr: the built-in rule; else exactly that shape (MOFF_EINVAL if infeasible).
 // dft: shapes of the gridding kernel with the tensor-core row transform (k_grid_rows_dft).
 moff_status build_bins(int A, int K, int N, int P, bool jones, const double *pos, const float *taps, Bins *b,
-                       const GridChoice *force = nullptr, bool dft = false);
+                       const GridChoice *force = nullptr, bool dft = false, bool narrow = false);
 std::vector<float2> pass_twiddles_for(int n);   // pass-twiddle table of the n-point transform (FP64-built)
 
 // Row spectra of the kernel rows for the tensor-core path (host side).
