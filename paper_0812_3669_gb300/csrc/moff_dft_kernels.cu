@@ -334,24 +334,6 @@ __device__ __forceinline__ void regs_dec() { asm volatile("setmaxnreg.dec.sync.a
 template <int R>
 __device__ __forceinline__ void regs_inc() { asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;\n" ::"n"(R)); }
 
-// *a += s v, with s a power of two, without the FP64 pipe (two operations a cycle and SM): the product's bits are put
-// together from v's and the addition is left to L2 (a reduction without return; one owner per element, so the sum
-// is that of a load, add and store).  Values whose product is subnormal, infinite or NaN take the plain path.
-__device__ __forceinline__ void red_scaled(double *a, float v, int scale_exp, double s) {
-    const uint32_t u = __float_as_uint(v);
-    const int e = (int)((u >> 23) & 255u);
-    double d;
-    if (e != 0 && e != 255) {
-        const uint32_t m = u & 0x7FFFFFu;
-        d = __hiloint2double((int)((u & 0x80000000u) | ((uint32_t)(e + 896 + scale_exp) << 20) | (m >> 3)), (int)(m << 29));
-    } else if ((u << 1) == 0u) {
-        return;                                                  // adding zero
-    } else {
-        d = (double)v * s;
-    }
-    atomicAdd(a, d);
-}
-
 template <int N, int P, int W>
 struct ColPipeShape {
     using S = DftShape<N>;
@@ -533,7 +515,7 @@ __global__ void __launch_bounds__(kCpThreads, 1) k_cols_pipe(const ColDftArgs a)
         if (ok) {   // undo the field's scale s_G / (16 N) (exact powers of two), squared, and fold into FP64
             const double un = 16.0 * (double)N / ((double)a.sy[c] * (double)a.s_t);
             const double sc2 = un * un;
-            const int se = (int)((__double2hiint(sc2) >> 20) & 2047) - 1023;
+            const int se = pow2_exp(sc2);
             const int m2 = 128 * j2 + 32 * q + lane;
             const int x = (m2 % (8 * W)) >> 3, cy = 8 * (m2 / (8 * W)) + (m2 & 7);
 #pragma unroll

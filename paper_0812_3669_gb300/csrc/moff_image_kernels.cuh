@@ -13,6 +13,7 @@
 //                 registers, then added to FP64 accumulators).
 // The row-transformed field goes through global memory between the two.
 #pragma once
+#include <cooperative_groups.h>
 #include <cuda_fp16.h>
 
 #include "moff_dft.cuh"
@@ -126,9 +127,11 @@ static_assert(fft_radix(32, 0) == FftPlan<32>::R0 && fft_radix(32, 1) == FftPlan
 // block (f, e), (f, e + 1), (f + 1, e), (f + 1, e + 1), f even); each entry carries CPL taps.
 // DFT: the row transform runs as factored DFT contractions on the tensor cores
 // (moff_dft.cuh) and the field leaves in FP16 (a.h16, field_offset).
-// (s, cl): this CTA's stripe and channel of the launch; n_str: stripes per set (the grid's x extent).
+// (s, cl): this CTA's stripe and channel of the launch; n_str: stripes per set (the grid's x extent); samples
+// [tlo, thi) of the launch's.
 template <int N, int P, int TB, bool STAGED, bool GRID_ONLY, int CPL, bool WIDE, bool DFT = false>
-__device__ __forceinline__ void grid_rows(const GridArgs &a, const int s, const int cl, const int n_str) {
+__device__ __forceinline__ void grid_rows(const GridArgs &a, const int s, const int cl, const int n_str, const int tlo,
+                                          const int thi) {
     constexpr bool PAIRS = CPL >= 2;
     using FP = FftPlan<N>;
     using TW = FftTw<N>;
@@ -163,7 +166,7 @@ __device__ __forceinline__ void grid_rows(const GridArgs &a, const int s, const 
         }
         if constexpr (DFT) {   // FP16 field: one 16-byte piece (8 columns of a row and part) per store
             constexpr int PIECES = N / 8 * 2, PER_T16 = P * PIECES * ROWS;
-            for (int i = tid; i < a.nt * PER_T16; i += kBlock) {
+            for (int i = tlo * PER_T16 + tid; i < thi * PER_T16; i += kBlock) {
                 const int t = i / PER_T16, e = i - t * PER_T16, rl = e % ROWS, k = (e / ROWS) % PIECES, p = e / (ROWS * PIECES);
                 __half *o = a.h16 + (((long long)t * a.slab_t + (long long)cl * a.slab_c) * P + p) * N * 2 * N +
                             field_offset(N, s * ROWS + rl, k & 1, k >> 1);
@@ -172,7 +175,7 @@ __device__ __forceinline__ void grid_rows(const GridArgs &a, const int s, const 
             return;
         }
         constexpr int PER_T = P * ROWS * N / 2;     // 16-byte stores per sample
-        for (int i = tid; i < a.nt * PER_T; i += kBlock) {
+        for (int i = tlo * PER_T + tid; i < thi * PER_T; i += kBlock) {
             const int t = i / PER_T, e = 2 * (i - t * PER_T);
             const int p = e / (ROWS * N), rem = e - p * (ROWS * N), rl = rem / N, x = rem - rl * N;
             float2 *o = a.out + (((long long)t * a.slab_t + (long long)cl * a.slab_c) * P * N + (long long)p * N +
@@ -242,7 +245,7 @@ __device__ __forceinline__ void grid_rows(const GridArgs &a, const int s, const 
     const uint8_t *vchan = a.volt + (long long)c * a.A * P;
     uint32_t vb[YPT][TB];
     auto fetch = [&](int tbn) {
-        const int nbn = min(TB, a.nt - tbn);
+        const int nbn = min(TB, thi - tbn);
 #pragma unroll
         for (int m = 0; m < YPT; ++m) {
             const int yi = tid + m * kBlock;
@@ -253,11 +256,11 @@ __device__ __forceinline__ void grid_rows(const GridArgs &a, const int s, const 
             for (int t = 0; t < TB; ++t) vb[m][t] = (yi < nyi && t < nbn) ? src[t * a.volt_tstride] : 0u;
         }
     };
-    if (pre) fetch(0);
+    if (pre) fetch(tlo);
 
     const int ry0 = s * ROWS;
-    for (int tb0 = 0; tb0 < a.nt; tb0 += TB) {
-        const int nb = min(TB, a.nt - tb0);
+    for (int tb0 = tlo; tb0 < thi; tb0 += TB) {
+        const int nb = min(TB, thi - tb0);
         // Step 1: decode and weight the voltages of the antennas touching this stripe.
         if (pre) {
 #pragma unroll
@@ -270,7 +273,7 @@ __device__ __forceinline__ void grid_rows(const GridArgs &a, const int s, const 
                     for (int t = 0; t < TB; ++t) yrow[t] = t < nb ? cmul(g, decode4(vb[m][t])) : make_float2(0.f, 0.f);
                 }
             }
-            if (tb0 + TB < a.nt) fetch(tb0 + TB);     // in flight during this pass
+            if (tb0 + TB < thi) fetch(tb0 + TB);     // in flight during this pass
         } else {
             for (int yi = tid; yi < nyi; yi += kBlock) {
                 const int la = yi / P, q = yi - la * P;
@@ -433,23 +436,32 @@ __device__ __forceinline__ void grid_rows(const GridArgs &a, const int s, const 
     }
 }
 
+// The z-th part of the launch's samples, whole passes of TB.
+template <int TB>
+__device__ __forceinline__ int2 time_part(int nt) {
+    const int per = ((nt + TB - 1) / TB + (int)gridDim.z - 1) / (int)gridDim.z * TB;
+    return make_int2(min(nt, (int)blockIdx.z * per), min(nt, ((int)blockIdx.z + 1) * per));
+}
+
 // Row transform out of place: the register count is the compiler's choice (an
 // explicit minimum of one CTA per SM lets it take about twice as many).
 template <int N, int P, int TB, bool STAGED, bool GRID_ONLY, int CPL, bool WIDE>
 __global__ void __launch_bounds__(kBlock) k_grid_rows(const GridArgs a) {
-    grid_rows<N, P, TB, STAGED, GRID_ONLY, CPL, WIDE>(a, blockIdx.x, blockIdx.y, gridDim.x);
+    const int2 t = time_part<TB>(a.nt);
+    grid_rows<N, P, TB, STAGED, GRID_ONLY, CPL, WIDE>(a, blockIdx.x, blockIdx.y, gridDim.x, t.x, t.y);
 }
 
 // Gridding with the row transform on the tensor cores (FP16 field out).
 template <int N, int P, int TB, int CPL>
 __global__ void __launch_bounds__(kBlock) k_grid_rows_dft(const GridArgs a) {
-    grid_rows<N, P, TB, false, false, CPL, false, true>(a, blockIdx.x, blockIdx.y, gridDim.x);
+    grid_rows<N, P, TB, false, false, CPL, false, true>(a, blockIdx.x, blockIdx.y, gridDim.x, 0, a.nt);
 }
 
 // Row transform in place: registers capped so that grid_min_blocks CTAs fit an SM.
 template <int N, int P, int TB, bool STAGED, bool GRID_ONLY, int CPL, bool WIDE>
 __global__ void __launch_bounds__(kBlock, grid_min_blocks<N, P, TB, CPL, WIDE>()) k_grid_rows_ip(const GridArgs a) {
-    grid_rows<N, P, TB, STAGED, GRID_ONLY, CPL, WIDE>(a, blockIdx.x, blockIdx.y, gridDim.x);
+    const int2 t = time_part<TB>(a.nt);
+    grid_rows<N, P, TB, STAGED, GRID_ONLY, CPL, WIDE>(a, blockIdx.x, blockIdx.y, gridDim.x, t.x, t.y);
 }
 
 template <int N>
@@ -460,9 +472,35 @@ struct ColShape {
     static constexpr int NS = N / RL;                          // slots per column in the last pass
 };
 
-// (sx, cl): this CTA's column strip and channel of the launch.
-template <int N, int P, bool H16, bool TAPS>
-__device__ __forceinline__ void cols_acc(const ColArgs &a, const int sx, const int cl) {
+template <int N>
+__host__ __device__ constexpr size_t col_smem_bytes_t(int P, bool h16 = false) {
+    using FP = FftPlan<N>;
+    const size_t tile = (size_t)P * N * ColShape<N>::W;
+    return (size_t)((FftTw<N>::TOTAL + 1) & ~1) * 8 + tile * (h16 ? 4 : 8) * 2 + tile * 8 * (FP::NP == 3 ? 2 : 1);
+}
+// Bytes of one CTA's sums, and the parts that a launch's samples are split into: short of CTAs, a cluster of up to eight
+// shares a strip's samples (at least eight each), up to four CTAs per SM.  FP32 fields split only where a persistent
+// launch, which gives the same image, has room for the sums of the parts before beside its tiles.
+template <int N>
+__host__ __device__ constexpr size_t col_sums_bytes_t(int P) { return (size_t)(P == 1 ? 1 : 4) * ColShape<N>::RL * kBlock * 4; }
+template <int N, int P, bool H16>
+__host__ __device__ inline int cols_parts(int nt, int nc) {
+    if (!H16 && col_smem_bytes_t<N>(P) + col_sums_bytes_t<N>(P) > 225 * 1024) return 1;
+    const long long ctas = (long long)(N / ColShape<N>::W) * nc;
+    int nz = 1;
+    while (nz < 8 && 2 * nz * ctas <= 4 * 152 && nt >= 16 * nz) nz *= 2;
+    return nz;
+}
+
+// (sx, cl): this CTA's column strip and channel of the launch; samples [tlo, thi) of the launch's.  nz CTAs of a
+// cluster share the strip's samples: their FP32 sums are added in rank order through distributed shared memory, then
+// folded once, so a sum does not depend on which CTA ends first.
+// MODE 0: the whole block (with run-time bounds it took 8 % longer), 1: a cluster's part, 2 (persistent launch): the
+// cluster's parts one after the other, their sums added in the same order through s_tot (unused if nz is 1).
+template <int N, int P, bool H16, bool TAPS, int MODE>
+__device__ __forceinline__ void cols_acc(const ColArgs &a, const int sx, const int cl, const int nz = 1) {
+    const int2 part_t = MODE == 1 ? time_part<1>(a.nt) : make_int2(0, a.nt);
+    const int tlo = part_t.x, thi = part_t.y;
     using FP = FftPlan<N>;
     using TW = FftTw<N>;
     using CS = ColShape<N>;
@@ -534,10 +572,10 @@ __device__ __forceinline__ void cols_acc(const ColArgs &a, const int sx, const i
             if (kx0 + colL == a.beam_kx[j] && ky >= jL && (ky - jL) % CS::NS == 0) bmask |= 1u << j;
         }
     }
-    if (a.nt > 0) stage(0, s_in);
+    if (tlo < thi) stage(tlo, s_in + (tlo & 1) * TILE * EB);
 
-    for (int tt = 0; tt < a.nt; ++tt) {
-        if (tt + 1 < a.nt) {
+    for (int tt = tlo; tt < thi; ++tt) {
+        if (tt + 1 < thi) {
             stage(tt + 1, s_in + ((tt + 1) & 1) * TILE * EB);
             cp_async_wait<1>();
         } else {
@@ -650,26 +688,68 @@ __device__ __forceinline__ void cols_acc(const ColArgs &a, const int sx, const i
             }
         }
         // s_a is rewritten by the next pass 0 only after the next barrier.
+        if constexpr (MODE == 2) {
+            if (nz > 1) {                            // end of a part: one more term of the sums (thread-private)
+                const int per = (a.nt + nz - 1) / nz;
+                if ((tt + 1) % per == 0 || tt + 1 == a.nt) {
+                    float *s_tot = reinterpret_cast<float *>(s_a + TILE * (FP::NP == 3 ? 2 : 1)) + tid;
+#pragma unroll
+                    for (int q = 0; q < NPROD; ++q)
+#pragma unroll
+                        for (int r = 0; r < RL; ++r) {
+                            float &v = s_tot[(q * RL + r) * kBlock];
+                            v = tt < per ? acc[q][r] : v + acc[q][r];
+                            acc[q][r] = tt + 1 == a.nt ? v : 0.f;
+                        }
+                }
+            }
+        }
     }
 
+    if constexpr (MODE == 1) {
+        const int nz = gridDim.z;
+        namespace cg = cooperative_groups;
+        cg::cluster_group cl_g = cg::this_cluster();
+        float *part = reinterpret_cast<float *>(s_in);   // [NPROD RL][kBlock]; no copy is in flight here
+        static_assert((size_t)NPROD * RL * kBlock * 4 <= 2 * (size_t)TILE * EB + (size_t)TILE * 8, "partial sums fit");
+        const int rank = (int)cl_g.block_rank();
+        __syncthreads();                                 // the last sample's pass outputs have been read
+        if (rank > 0) {
+#pragma unroll
+            for (int q = 0; q < NPROD; ++q)
+#pragma unroll
+                for (int r = 0; r < RL; ++r) part[(q * RL + r) * kBlock + tid] = acc[q][r];
+        }
+        cl_g.sync();
+        if (rank == 0) {
+            for (int z = 1; z < nz; ++z) {
+                const float *o = cl_g.map_shared_rank(part, z);
+#pragma unroll
+                for (int q = 0; q < NPROD; ++q)
+#pragma unroll
+                    for (int r = 0; r < RL; ++r) acc[q][r] += o[(q * RL + r) * kBlock + tid];
+            }
+        }
+        cl_g.sync();                                     // the partial sums have been read
+        if (rank > 0) return;
+    }
     // Fold this chunk's FP32 sums into the FP64 accumulators (one owner per pixel).
-    const double sc2 = (double)sc * (double)sc;
+    // The additions happen in L2 (in a persistent launch another SM folded the previous chunk): on the FP64 pipe the
+    // conversion and the sum were 4 to 7 % of a 128-sample chunk.
+    const double sc2 = H16 ? (double)sc * (double)sc : 1.0;
+    const int se = H16 ? pow2_exp(sc2) : 0;
     const int kx = kx0 + colL;
 #pragma unroll
     for (int q = 0; q < NPROD; ++q) {
-        double *d = a.acc + ((long long)c * NPROD + q) * N * N + kx;
+        double *d = a.acc + ((long long)c * NPROD + q) * N * N + (long long)jL * N + kx;
 #pragma unroll
-        for (int r = 0; r < RL; ++r) {
-            const int ky = jL + r * CS::NS;
-            // read through L2: in a persistent launch another SM folded the previous chunk
-            d[(long long)ky * N] = __ldcg(d + (long long)ky * N) + (H16 ? (double)acc[q][r] * sc2 : (double)acc[q][r]);
-        }
+        for (int r = 0; r < RL; ++r) red_scaled(d + r * CS::NS * N, acc[q][r], se, sc2);
     }
 }
 
-template <int N, int P, bool H16, bool TAPS>
+template <int N, int P, bool H16, bool TAPS, bool SPLIT>
 __global__ void __launch_bounds__(kBlock) k_cols_acc(const ColArgs a) {
-    cols_acc<N, P, H16, TAPS>(a, blockIdx.x, blockIdx.y);
+    cols_acc<N, P, H16, TAPS, SPLIT ? 1 : 0>(a, blockIdx.x, blockIdx.y);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -753,13 +833,13 @@ __global__ void __launch_bounds__(kBlock) k_image_persist(const __grid_constant_
             g.nt = ch.y;
             g.c0 = ch.z;
             g.nc = ch.w;
-            grid_rows<N, P, TB, false, false, CPL, WIDE>(g, w.z, w.w, pa.n_stripes);
+            grid_rows<N, P, TB, false, false, CPL, WIDE>(g, w.z, w.w, pa.n_stripes, 0, g.nt);
         } else {
             ColArgs ca = pa.ca;
             ca.nt = ch.y;
             ca.c0 = ch.z;
             ca.nc = ch.w;
-            cols_acc<N, P, false, false>(ca, w.z, w.w);
+            cols_acc<N, P, false, false, 2>(ca, w.z, w.w, cols_parts<N, P, false>(ca.nt, ca.nc));
         }
         __threadfence();
         __syncthreads();
@@ -770,6 +850,9 @@ __global__ void __launch_bounds__(kBlock) k_image_persist(const __grid_constant_
 template <int N, int P, int CPL, bool WIDE>
 cudaError_t launch_persist_t(const PersistArgs &pa, size_t smem, int sms, cudaStream_t st) {
     auto k = k_image_persist<N, P, 4, CPL, WIDE>;
+    for (int i = 0; i < pa.n_chunks; ++i)   // room for the sums of a split block's parts
+        if (cols_parts<N, P, false>(pa.chunks[i].y, pa.chunks[i].w) > 1)
+            smem = std::max(smem, col_smem_bytes_t<N>(P) + col_sums_bytes_t<N>(P));
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     int per_sm = 0;
@@ -802,13 +885,6 @@ cudaError_t launch_persist_p(int cpl, bool wide, const PersistArgs &pa, size_t s
                       : launch_persist_p<NN, 2>(cpl, wide, pa, smem, sms, st);                      \
     }
 
-template <int N>
-size_t col_smem_bytes_t(int P, bool h16 = false) {
-    using FP = FftPlan<N>;
-    const size_t tile = (size_t)P * N * ColShape<N>::W;
-    return (size_t)((FftTw<N>::TOTAL + 1) & ~1) * 8 + tile * (h16 ? 4 : 8) * 2 + tile * 8 * (FP::NP == 3 ? 2 : 1);
-}
-
 template <int N, int P, int TB, bool ST, bool GO, int CPL, bool WD>
 cudaError_t launch_grid_t(const GridArgs &a, int n_stripes, size_t smem, cudaStream_t st) {
     // 2 x 2 blocks need an even stripe height and entries read through L2
@@ -820,7 +896,11 @@ cudaError_t launch_grid_t(const GridArgs &a, int n_stripes, size_t smem, cudaStr
     else k = k_grid_rows<N, P, TB, ST, GO, CPL, WD>;
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    k<<<dim3(n_stripes, a.nc), kBlock, smem, st>>>(a);
+    // Short of CTAs, the samples are split over the grid's z: every CTA sets its stripe up anew, so parts keep at
+    // least two passes, and the split stops at four CTAs per SM.
+    const long long ctas = (long long)n_stripes * a.nc;
+    const int nz = (int)std::max(1LL, std::min<long long>(((a.nt + TB - 1) / TB) / 2, 4 * 152 / ctas));
+    k<<<dim3(n_stripes, a.nc, nz), kBlock, smem, st>>>(a);
     return cudaGetLastError();
     }
 }
@@ -864,13 +944,27 @@ cudaError_t launch_grid_p(int TB, bool staged, bool go, const GridArgs &a, int n
 
 template <int N, int P, bool H16>
 cudaError_t launch_cols_t(const ColArgs &a, cudaStream_t st) {
+    const int nz = cols_parts<N, P, H16>(a.nt, a.nc);
     // pixel taps (feedback calibration, beams) compiled in only where asked for
-    auto k = (a.etap || a.n_beam) ? k_cols_acc<N, P, H16, true> : k_cols_acc<N, P, H16, false>;
+    const bool taps = a.etap || a.n_beam;
+    auto k = nz > 1 ? (taps ? k_cols_acc<N, P, H16, true, true> : k_cols_acc<N, P, H16, false, true>)
+                    : (taps ? k_cols_acc<N, P, H16, true, false> : k_cols_acc<N, P, H16, false, false>);
     const size_t smem = col_smem_bytes_t<N>(P, H16);
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    k<<<dim3(N / ColShape<N>::W, a.nc), kBlock, smem, st>>>(a);
-    return cudaGetLastError();
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(N / ColShape<N>::W, a.nc, nz);
+    cfg.blockDim = dim3(kBlock);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = 1;
+    at.val.clusterDim.y = 1;
+    at.val.clusterDim.z = (unsigned)nz;
+    cfg.attrs = &at;
+    cfg.numAttrs = nz > 1 ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, k, a);
 }
 
 #define MOFF_DEFINE_N(NN)                                                                            \
