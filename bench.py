@@ -499,7 +499,7 @@ KERNEL_SOURCES = {
     "grid_rows": [("paper_0812_3669_gb300/csrc/moff_image_kernels.cuh", "struct ColShape"),
                   "paper_0812_3669_gb300/csrc/moff_fft.cuh"],
     "cols_integrate": [("paper_0812_3669_gb300/csrc/moff_image_kernels.cuh", "template <int N>\nstruct ColShape",
-                        "size_t col_smem_bytes_t"),
+                        "template <int N, int P, int TB, bool ST, bool GO"),
                        "paper_0812_3669_gb300/csrc/moff_fft.cuh"],
     "pfb_fstage": ["paper_0812_3669_gb300/csrc/moff_fstage.cu", "paper_0812_3669_gb300/csrc/moff_fft.cuh"],
     # the factored-DFT tensor-core route of the dense workloads

@@ -16,6 +16,8 @@
 #include <cooperative_groups.h>
 #include <cuda_fp16.h>
 
+#include <type_traits>
+
 #include "moff_dft.cuh"
 #include "moff_fft.cuh"
 #include "moff_internal.h"
@@ -472,9 +474,30 @@ struct ColShape {
     static constexpr int NS = N / RL;                          // slots per column in the last pass
 };
 
+// Two pols in step (cols_pol): slots of the first pass and samples per round.
+template <int N>
+struct ColPolShape {
+    static constexpr int SL = ColShape<N>::W * (N / FftPlan<N>::R0);
+    static constexpr int S = kBlock / SL;
+    static_assert(SL * S == kBlock, "whole rounds");
+    static constexpr size_t SMEM = ((size_t)FftTw<N>::TOTAL + (size_t)(S + (FftPlan<N>::NP == 3)) * N * ColShape<N>::W) * 16;
+};
+// The passes on different warps (cols_duo).
+template <int N>
+struct ColDuoShape {
+    static constexpr int W = ColShape<N>::W, STRIP = 2 * N * W;   // elements of one sample's strip
+    static constexpr size_t SMEM = (size_t)FftTw<N>::TOTAL * 16 + 2 * (size_t)STRIP * 4 + 2 * (size_t)N * W * 16;
+};
+template <int N, int P, bool H16>
+__host__ __device__ constexpr bool cols_use_duo() { return P == 2 && H16 && N <= 128; }
+template <int N, int P, bool H16>
+__host__ __device__ constexpr bool cols_use_pol() { return P == 2 && !cols_use_duo<N, P, H16>() && N >= 256; }
 template <int N>
 __host__ __device__ constexpr size_t col_smem_bytes_t(int P, bool h16 = false) {
     using FP = FftPlan<N>;
+    if constexpr (N <= 128)
+        if (P == 2 && h16) return ColDuoShape<N>::SMEM;
+    if (P == 2 && (h16 ? cols_use_pol<N, 2, true>() : cols_use_pol<N, 2, false>())) return ColPolShape<N>::SMEM;
     const size_t tile = (size_t)P * N * ColShape<N>::W;
     return (size_t)((FftTw<N>::TOTAL + 1) & ~1) * 8 + tile * (h16 ? 4 : 8) * 2 + tile * 8 * (FP::NP == 3 ? 2 : 1);
 }
@@ -490,6 +513,66 @@ __host__ __device__ inline int cols_parts(int nt, int nc) {
     int nz = 1;
     while (nz < 8 && 2 * nz * ctas <= 4 * 152 && nt >= 16 * nz) nz *= 2;
     return nz;
+}
+
+// Sequential parts (persistent launch): at the end of a part its sums become one more term of the total, which stays in
+// shared memory (thread-private) until the last part.
+template <int NPROD, int RL>
+__device__ __forceinline__ void cols_part_end(int nt, int nz, int tt, float *s_tot, float (&acc)[NPROD][RL]) {
+    const int per = (nt + nz - 1) / nz;
+    if ((tt + 1) % per != 0 && tt + 1 != nt) return;
+#pragma unroll
+    for (int q = 0; q < NPROD; ++q)
+#pragma unroll
+        for (int r = 0; r < RL; ++r) {
+            float &v = s_tot[(q * RL + r) * kBlock + threadIdx.x];
+            v = tt < per ? acc[q][r] : v + acc[q][r];
+            acc[q][r] = tt + 1 == nt ? v : 0.f;
+        }
+}
+
+// End of a strip: the cluster's parts added in rank order (MODE 1, through `part`, which no thread uses any more after
+// the barrier), then this chunk's FP32 sums folded into the FP64 accumulators (one owner per pixel).  The additions
+// happen in L2 (in a persistent launch another SM folded the previous chunk): on the FP64 pipe the conversion and the
+// sum were 4 to 7 % of a 128-sample chunk.  The thread's pixels: ky = j + r NS of column kx.
+template <int N, int P, bool H16, int MODE>
+__device__ __forceinline__ void cols_finish(const ColArgs &a, float (&acc)[P == 1 ? 1 : 4][ColShape<N>::RL], int kx, int j, int c,
+                                            float sc, float *part) {
+    using CS = ColShape<N>;
+    constexpr int NPROD = P == 1 ? 1 : 4, RL = CS::RL;
+    const int tid = threadIdx.x;
+    if constexpr (MODE == 1) {
+        namespace cg = cooperative_groups;
+        cg::cluster_group cl_g = cg::this_cluster();
+        const int rank = (int)cl_g.block_rank(), nz = gridDim.z;
+        __syncthreads();                                 // the last sample's pass outputs have been read
+        if (rank > 0) {
+#pragma unroll
+            for (int q = 0; q < NPROD; ++q)
+#pragma unroll
+                for (int r = 0; r < RL; ++r) part[(q * RL + r) * kBlock + tid] = acc[q][r];
+        }
+        cl_g.sync();
+        if (rank == 0) {
+            for (int z = 1; z < nz; ++z) {
+                const float *o = cl_g.map_shared_rank(part, z);
+#pragma unroll
+                for (int q = 0; q < NPROD; ++q)
+#pragma unroll
+                    for (int r = 0; r < RL; ++r) acc[q][r] += o[(q * RL + r) * kBlock + tid];
+            }
+        }
+        cl_g.sync();                                     // the partial sums have been read
+        if (rank > 0) return;
+    }
+    const double sc2 = H16 ? (double)sc * (double)sc : 1.0;
+    const int se = H16 ? pow2_exp(sc2) : 0;
+#pragma unroll
+    for (int q = 0; q < NPROD; ++q) {
+        double *d = a.acc + ((long long)c * NPROD + q) * N * N + (long long)j * N + kx;
+#pragma unroll
+        for (int r = 0; r < RL; ++r) red_scaled(d + r * CS::NS * N, acc[q][r], se, sc2);
+    }
 }
 
 // (sx, cl): this CTA's column strip and channel of the launch; samples [tlo, thi) of the launch's.  nz CTAs of a
@@ -689,67 +772,403 @@ __device__ __forceinline__ void cols_acc(const ColArgs &a, const int sx, const i
         }
         // s_a is rewritten by the next pass 0 only after the next barrier.
         if constexpr (MODE == 2) {
-            if (nz > 1) {                            // end of a part: one more term of the sums (thread-private)
-                const int per = (a.nt + nz - 1) / nz;
-                if ((tt + 1) % per == 0 || tt + 1 == a.nt) {
-                    float *s_tot = reinterpret_cast<float *>(s_a + TILE * (FP::NP == 3 ? 2 : 1)) + tid;
+            if (nz > 1) cols_part_end<NPROD, RL>(a.nt, nz, tt, reinterpret_cast<float *>(s_a + TILE * (FP::NP == 3 ? 2 : 1)), acc);
+        }
+    }
+    cols_finish<N, P, H16, MODE>(a, acc, kx0 + colL, jL, c, sc, reinterpret_cast<float *>(s_in));
+}
+
+// ---------------------------------------------------------------------------------------------
+// Two pols in step: every value of the transform is a pair (x pol, y pol), so all its arithmetic is packed FP32 (one
+// instruction for both pols; scalar rotations and products were a third of the instructions before), the passes
+// exchange 16-byte elements, and XX, YY are one packed sum.  The field's elements go straight from global memory into
+// the registers of the first pass, S samples a round so that all threads have a slot, loaded one round ahead -- no
+// staging tiles, so two or three CTAs share an SM where the 512 grid had one.
+struct Pol2 {
+    float2 re, im;   // (x, y)
+};
+__device__ __forceinline__ Pol2 padd(Pol2 a, Pol2 b) { return {cadd(a.re, b.re), cadd(a.im, b.im)}; }
+__device__ __forceinline__ Pol2 psub(Pol2 a, Pol2 b) { return {csub(a.re, b.re), csub(a.im, b.im)}; }
+// a + i b, a - i b
+__device__ __forceinline__ Pol2 padd_i(Pol2 a, Pol2 b) { return {csub(a.re, b.im), cadd(a.im, b.re)}; }
+__device__ __forceinline__ Pol2 psub_i(Pol2 a, Pol2 b) { return {cadd(a.re, b.im), csub(a.im, b.re)}; }
+// a (c + i s)
+__device__ __forceinline__ Pol2 prot(Pol2 a, float c, float s) {
+    const float2 cc = make_float2(c, c), ss = make_float2(s, s), ns = make_float2(-s, -s);
+    return {dftc::fma2(a.re, cc, dftc::mul2(a.im, ns)), dftc::fma2(a.re, ss, dftc::mul2(a.im, cc))};
+}
+__device__ __forceinline__ void pdft4(Pol2 &a0, Pol2 &a1, Pol2 &a2, Pol2 &a3) {
+    const Pol2 t0 = padd(a0, a2), t1 = psub(a0, a2), t2 = padd(a1, a3), d = psub(a1, a3);
+    a0 = padd(t0, t2);
+    a2 = psub(t0, t2);
+    a1 = padd_i(t1, d);
+    a3 = psub_i(t1, d);
+}
+__device__ __forceinline__ void pdft8(Pol2 &x0, Pol2 &x1, Pol2 &x2, Pol2 &x3, Pol2 &x4, Pol2 &x5, Pol2 &x6, Pol2 &x7) {
+    Pol2 e0 = x0, e1 = x2, e2 = x4, e3 = x6, o0 = x1, o1 = x3, o2 = x5, o3 = x7;
+    pdft4(e0, e1, e2, e3);
+    pdft4(o0, o1, o2, o3);
+    o1 = prot(o1, MOFF_C8, MOFF_C8);
+    o3 = prot(o3, -MOFF_C8, MOFF_C8);
+    x0 = padd(e0, o0); x4 = psub(e0, o0);
+    x1 = padd(e1, o1); x5 = psub(e1, o1);
+    x2 = padd_i(e2, o2); x6 = psub_i(e2, o2);
+    x3 = padd(e3, o3); x7 = psub(e3, o3);
+}
+template <int R>
+__device__ __forceinline__ void pdft(Pol2 (&v)[R]) {   // exp(+2 pi i n k / R)
+    if constexpr (R == 4) {
+        pdft4(v[0], v[1], v[2], v[3]);
+    } else if constexpr (R == 8) {
+        pdft8(v[0], v[1], v[2], v[3], v[4], v[5], v[6], v[7]);
+    } else {
+        static_assert(R == 16, "unsupported radix");
+        Pol2 e[8], o[8];
 #pragma unroll
-                    for (int q = 0; q < NPROD; ++q)
+        for (int i = 0; i < 8; ++i) { e[i] = v[2 * i]; o[i] = v[2 * i + 1]; }
+        pdft8(e[0], e[1], e[2], e[3], e[4], e[5], e[6], e[7]);
+        pdft8(o[0], o[1], o[2], o[3], o[4], o[5], o[6], o[7]);
+        o[1] = prot(o[1], MOFF_C16, MOFF_S16);
+        o[2] = prot(o[2], MOFF_C8, MOFF_C8);
+        o[3] = prot(o[3], MOFF_S16, MOFF_C16);
+        o[5] = prot(o[5], -MOFF_S16, MOFF_C16);
+        o[6] = prot(o[6], -MOFF_C8, MOFF_C8);
+        o[7] = prot(o[7], -MOFF_C16, MOFF_S16);
 #pragma unroll
-                        for (int r = 0; r < RL; ++r) {
-                            float &v = s_tot[(q * RL + r) * kBlock];
-                            v = tt < per ? acc[q][r] : v + acc[q][r];
-                            acc[q][r] = tt + 1 == a.nt ? v : 0.f;
-                        }
+        for (int i = 0; i < 8; ++i) {
+            v[i] = i == 4 ? padd_i(e[i], o[i]) : padd(e[i], o[i]);
+            v[i + 8] = i == 4 ? psub_i(e[i], o[i]) : psub(e[i], o[i]);
+        }
+    }
+}
+// v[r] *= w of slot j; the table holds (re, re, -im, -im)
+template <int R, int NS>
+__device__ __forceinline__ void ptwiddle(Pol2 (&v)[R], int j, const float4 *tw) {
+    const int m = j % NS;
+#pragma unroll
+    for (int r = 1; r < R; ++r) {
+        const float4 w = tw[(r - 1) * NS + m];
+        const float2 wr = make_float2(w.x, w.y), nwi = make_float2(w.z, w.w), re = v[r].re, im = v[r].im;
+        v[r].re = dftc::fma2(im, nwi, dftc::mul2(re, wr));
+        v[r].im = csub(dftc::mul2(im, wr), dftc::mul2(re, nwi));
+    }
+}
+__device__ __forceinline__ float4 pol_pack(Pol2 v) { return make_float4(v.re.x, v.re.y, v.im.x, v.im.y); }
+__device__ __forceinline__ Pol2 pol_unpack(float4 q) { return {make_float2(q.x, q.y), make_float2(q.z, q.w)}; }
+
+// Pixel taps of sample tt (feedback calibration, tied-array beams): this thread holds ky = j + r NS of column kx.
+template <int RL, int NS>
+__device__ __forceinline__ void pol_taps(const ColArgs &a, const Pol2 (&v)[RL], int tt, int cl, int c, int kx, int j, float sc) {
+    auto put = [&](int ky, float2 *o) {
+        if (ky < j || (ky - j) % NS) return;
+#pragma unroll
+        for (int r = 0; r < RL; ++r)
+            if (j + r * NS == ky) {
+                o[0] = make_float2(v[r].re.x * sc, v[r].im.x * sc);
+                o[1] = make_float2(v[r].re.y * sc, v[r].im.y * sc);
+            }
+    };
+    if (a.etap && kx == a.tap_kx) put(a.tap_ky, a.etap + ((long long)tt * a.nc + cl) * 2);
+    for (int b = 0; b < a.n_beam; ++b)
+        if (kx == a.beam_kx[b]) put(a.beam_ky[b], a.beam_out + (((long long)(a.beam_t0 + tt) * a.beam_C + c) * a.n_beam + b) * 2);
+}
+
+// (sx, cl), MODE and nz as cols_acc.
+template <int N, bool H16, bool TAPS, int MODE>
+__device__ __forceinline__ void cols_pol(const ColArgs &a, const int sx, const int cl, const int nz = 1) {
+    using FP = FftPlan<N>;
+    using TW = FftTw<N>;
+    using CS = ColShape<N>;
+    using PS = ColPolShape<N>;
+    constexpr int W = CS::W, RL = CS::RL, NS = CS::NS, R0 = FP::R0, NSL = N / R0, SL = PS::SL, S = PS::S;
+    using Elem = typename std::conditional<H16, uint32_t, float2>::type;   // half2 or float2 of one pol
+    const int2 part_t = MODE == 1 ? time_part<1>(a.nt) : make_int2(0, a.nt);
+    const int tlo = part_t.x, thi = part_t.y;
+    const int kx0 = sx * W, c = a.c0 + cl, tid = threadIdx.x;
+
+    extern __shared__ __align__(16) unsigned char smem[];
+    float4 *s_tw = reinterpret_cast<float4 *>(smem);
+    float4 *s_a = s_tw + TW::TOTAL;                     // [S][N][W] outputs of the first pass
+    float4 *s_b = s_a + S * N * W;                      // [N][W] outputs of the second (three-pass lengths)
+    for (int i = tid; i < TW::TOTAL; i += kBlock) {
+        const float2 w = a.twp[i];
+        s_tw[i] = make_float4(w.x, w.x, -w.y, -w.y);
+    }
+    const float sc = H16 ? a.row_inv[0] * a.inv_sw / a.sy[c] : 1.f;   // as cols_acc
+
+    // first pass: sample ss of the round, column col, slot j; rows no kernel reaches are zero and never read
+    const int ss = tid / SL, sl = tid - ss * SL, col = sl % W, j = sl / W;
+    uint32_t act = 0;
+#pragma unroll
+    for (int r = 0; r < R0; ++r) {
+        const int ry = j + r * NSL;
+        if (!a.row_nz || ((a.row_nz[ry >> 5] >> (ry & 31)) & 1u)) act |= 1u << r;
+    }
+    Elem ex[R0], ey[R0];
+#pragma unroll
+    for (int r = 0; r < R0; ++r) ex[r] = ey[r] = Elem{};
+    const Elem *src0 = reinterpret_cast<const Elem *>(a.H) + (long long)cl * a.slab_c * 2 * N * N + kx0 + j * N + col;
+    auto load = [&](int tt) {
+        if (tt < thi) {
+            const Elem *src = src0 + (long long)tt * a.slab_t * 2 * N * N;
+#pragma unroll
+            for (int r = 0; r < R0; ++r)
+                if ((act >> r) & 1u) {
+                    ex[r] = __ldcg(src + r * NSL * N);
+                    ey[r] = __ldcg(src + N * N + r * NSL * N);
+                }
+        }
+    };
+    auto pair_of = [&](int r) -> Pol2 {
+        if constexpr (H16) {
+            const float2 x = __half22float2(*reinterpret_cast<const __half2 *>(&ex[r]));
+            const float2 y = __half22float2(*reinterpret_cast<const __half2 *>(&ey[r]));
+            return {make_float2(x.x, y.x), make_float2(x.y, y.y)};
+        } else {
+            return {make_float2(ex[r].x, ey[r].x), make_float2(ex[r].y, ey[r].y)};
+        }
+    };
+
+    const int colL = tid % W, jL = tid / W;             // last pass: ky = jL + r NS of column kx0 + colL
+    float2 pw[RL];                                      // XX, YY
+    float xr[RL], xi[RL];                               // Re, Im XY
+#pragma unroll
+    for (int r = 0; r < RL; ++r) {
+        pw[r] = make_float2(0.f, 0.f);
+        xr[r] = xi[r] = 0.f;
+    }
+    load(tlo + ss);
+    for (int t0 = tlo; t0 < thi; t0 += S) {
+        {
+            Pol2 v[R0];
+#pragma unroll
+            for (int r = 0; r < R0; ++r) v[r] = pair_of(r);
+            if (R0 < 16) load(t0 + S + ss);             // lands during this round
+            pdft<R0>(v);
+            if (FP::NP == 2 && t0 > tlo) __syncthreads();   // the last round's outputs have been read
+#pragma unroll
+            for (int r = 0; r < R0; ++r) s_a[(ss * N + stockham_out<R0, 1>(j, r)) * W + col] = pol_pack(v[r]);
+            if (R0 == 16) load(t0 + S + ss);            // (registers: only once the 16 values have left)
+        }
+        __syncthreads();
+        if constexpr (FP::NP == 3) {
+            constexpr int R = FP::R1, NS1 = FP::R0;
+            static_assert(W * (N / R) == kBlock && S == 1, "one slot per thread");
+            const int c1 = tid % W, j1 = tid / W;
+            Pol2 v[R];
+#pragma unroll
+            for (int r = 0; r < R; ++r) v[r] = pol_unpack(s_a[(j1 + r * (N / R)) * W + c1]);
+            ptwiddle<R, NS1>(v, j1, s_tw + TW::OFF1);
+            pdft<R>(v);
+#pragma unroll
+            for (int r = 0; r < R; ++r) s_b[stockham_out<R, NS1>(j1, r) * W + c1] = pol_pack(v[r]);
+            __syncthreads();
+        }
+#pragma unroll
+        for (int s = 0; s < S; ++s) {
+            const int tt = t0 + s;
+            if (S > 1 && tt >= thi) break;
+            const float4 *src = FP::NP == 3 ? s_b : s_a + s * N * W;
+            Pol2 v[RL];
+#pragma unroll
+            for (int r = 0; r < RL; ++r) v[r] = pol_unpack(src[(jL + r * NS) * W + colL]);
+            ptwiddle<RL, NS>(v, jL, s_tw + (FP::NP == 3 ? TW::OFF2 : TW::OFF1));
+            pdft<RL>(v);
+            if constexpr (TAPS) pol_taps<RL, NS>(a, v, tt, cl, c, kx0 + colL, jL, sc);
+#pragma unroll
+            for (int r = 0; r < RL; ++r) {
+                pw[r] = dftc::fma2(v[r].re, v[r].re, dftc::fma2(v[r].im, v[r].im, pw[r]));
+                xr[r] = fmaf(v[r].re.x, v[r].re.y, fmaf(v[r].im.x, v[r].im.y, xr[r]));
+                xi[r] = fmaf(v[r].im.x, v[r].re.y, fmaf(-v[r].re.x, v[r].im.y, xi[r]));
+            }
+            if constexpr (MODE == 2) {
+                if (nz > 1) {
+                    float acc[4][RL];
+#pragma unroll
+                    for (int r = 0; r < RL; ++r) { acc[0][r] = pw[r].x; acc[1][r] = pw[r].y; acc[2][r] = xr[r]; acc[3][r] = xi[r]; }
+                    cols_part_end<4, RL>(a.nt, nz, tt, reinterpret_cast<float *>(s_a + (S + (FP::NP == 3)) * N * W), acc);
+#pragma unroll
+                    for (int r = 0; r < RL; ++r) { pw[r] = make_float2(acc[0][r], acc[1][r]); xr[r] = acc[2][r]; xi[r] = acc[3][r]; }
                 }
             }
         }
     }
+    float acc[4][RL];
+#pragma unroll
+    for (int r = 0; r < RL; ++r) { acc[0][r] = pw[r].x; acc[1][r] = pw[r].y; acc[2][r] = xr[r]; acc[3][r] = xi[r]; }
+    cols_finish<N, 2, H16, MODE>(a, acc, kx0 + colL, jL, c, sc, reinterpret_cast<float *>(s_a));
+}
 
-    if constexpr (MODE == 1) {
-        const int nz = gridDim.z;
-        namespace cg = cooperative_groups;
-        cg::cluster_group cl_g = cg::this_cluster();
-        float *part = reinterpret_cast<float *>(s_in);   // [NPROD RL][kBlock]; no copy is in flight here
-        static_assert((size_t)NPROD * RL * kBlock * 4 <= 2 * (size_t)TILE * EB + (size_t)TILE * 8, "partial sums fit");
-        const int rank = (int)cl_g.block_rank();
-        __syncthreads();                                 // the last sample's pass outputs have been read
-        if (rank > 0) {
+// ---------------------------------------------------------------------------------------------
+// The FP16 field's two-pass columns (N = 32, 64, 128; two pols in step) with the passes on different warps: threads
+// 0-127 copy sample t + 1's strip (cp.async) and run the first pass of sample t, threads 128-255 the last pass and
+// the products of sample t - 1, one barrier a sample.  Each half needs only its own registers (16 values, or the sums),
+// so two CTAs fit an SM without spills, and one half's arithmetic covers the other's waits.  Bound by FP32 arithmetic.
+template <int N, bool TAPS, int MODE>
+__device__ __forceinline__ void cols_duo(const ColArgs &a, const int sx, const int cl) {
+    using FP = FftPlan<N>;
+    using TW = FftTw<N>;
+    using CS = ColShape<N>;
+    using DS = ColDuoShape<N>;
+    constexpr int W = CS::W, RL = CS::RL, NS = CS::NS, R0 = FP::R0, NSL = N / R0, HB = kBlock / 2;
+    static_assert(FP::NP == 2, "two passes");
+    const int2 part_t = MODE == 1 ? time_part<1>(a.nt) : make_int2(0, a.nt);
+    const int tlo = part_t.x, thi = part_t.y;
+    const int kx0 = sx * W, c = a.c0 + cl, tid = threadIdx.x, u = tid & (HB - 1);
+    const bool second = tid >= HB;
+
+    extern __shared__ __align__(16) unsigned char smem[];
+    float4 *s_tw = reinterpret_cast<float4 *>(smem);
+    float4 *s_a = s_tw + TW::TOTAL;                                 // [2][N][W] outputs of the first pass
+    uint32_t *s_in = reinterpret_cast<uint32_t *>(s_a + 2 * N * W);  // [2][pol][N][W] half2
+    for (int i = tid; i < TW::TOTAL; i += kBlock) {
+        const float2 w = a.twp[i];
+        s_tw[i] = make_float4(w.x, w.x, -w.y, -w.y);
+    }
+    const float sc = a.row_inv[0] * a.inv_sw / a.sy[c];             // as cols_acc
+    constexpr int RL2 = kBlock / HB * RL;
+    float2 pw[RL2];                                                 // second half: XX, YY of its two slots
+    float xr[RL2], xi[RL2];                                         // Re, Im XY
 #pragma unroll
-            for (int q = 0; q < NPROD; ++q)
+    for (int r = 0; r < RL2; ++r) {
+        pw[r] = make_float2(0.f, 0.f);
+        xr[r] = xi[r] = 0.f;
+    }
+    // copies: piece (p, row, part) of 16 bytes; rows no kernel reaches are cleared once and never read
+    constexpr int ROWCH = W / 4, ITER = 2 * N * ROWCH / HB;
+    static_assert(2 * N * ROWCH % HB == 0 && ITER <= 32, "pieces per thread");
+    uint32_t act = 0;
+    if (!second) {
 #pragma unroll
-                for (int r = 0; r < RL; ++r) part[(q * RL + r) * kBlock + tid] = acc[q][r];
-        }
-        cl_g.sync();
-        if (rank == 0) {
-            for (int z = 1; z < nz; ++z) {
-                const float *o = cl_g.map_shared_rank(part, z);
-#pragma unroll
-                for (int q = 0; q < NPROD; ++q)
-#pragma unroll
-                    for (int r = 0; r < RL; ++r) acc[q][r] += o[(q * RL + r) * kBlock + tid];
+        for (int k = 0; k < ITER; ++k) {
+            const int q = u + k * HB, ry = (q / ROWCH) % N;
+            if (!a.row_nz || ((a.row_nz[ry >> 5] >> (ry & 31)) & 1u)) {
+                act |= 1u << k;
+            } else {
+                *reinterpret_cast<uint4 *>(s_in + 4 * q) = make_uint4(0u, 0u, 0u, 0u);
+                *reinterpret_cast<uint4 *>(s_in + DS::STRIP + 4 * q) = make_uint4(0u, 0u, 0u, 0u);
             }
         }
-        cl_g.sync();                                     // the partial sums have been read
+    }
+    const uint32_t *src0 = reinterpret_cast<const uint32_t *>(a.H) + (long long)cl * a.slab_c * 2 * N * N + kx0 +
+                           (u / ROWCH) * N + (u % ROWCH) * 4;
+    auto copy = [&](int tt) {
+        const uint32_t *src = src0 + (long long)tt * a.slab_t * 2 * N * N;
+        const uint32_t dst = tc::smem_u32(s_in + (tt & 1) * DS::STRIP + 4 * u);
+        static_assert(HB % ROWCH == 0, "whole rows per round");
+#pragma unroll
+        for (int k = 0; k < ITER; ++k) cp_async16_if((act >> k) & 1u, dst + k * HB * 16, src + k * (HB / ROWCH) * N);
+        cp_async_commit();
+    };
+    if (!second && tlo < thi) {
+        copy(tlo);
+        cp_async_wait<0>();
+    }
+    __syncthreads();
+    for (int t = tlo; t <= thi; ++t) {                              // first pass of t, last pass of t - 1
+        if (!second) {
+            if (t + 1 < thi) copy(t + 1);
+            if (t < thi) {
+                const uint32_t *in = s_in + (t & 1) * DS::STRIP;
+                float4 *out = s_a + (t & 1) * N * W;
+#pragma unroll 1
+                for (int sl = u; sl < W * NSL; sl += HB) {
+                    const int col = sl % W, j = sl / W;
+                    Pol2 v[R0];
+#pragma unroll
+                    for (int r = 0; r < R0; ++r) {
+                        const int e = (j + r * NSL) * W + col;
+                        const float2 x = __half22float2(*reinterpret_cast<const __half2 *>(in + e));
+                        const float2 y = __half22float2(*reinterpret_cast<const __half2 *>(in + N * W + e));
+                        v[r] = {make_float2(x.x, y.x), make_float2(x.y, y.y)};
+                    }
+                    pdft<R0>(v);
+#pragma unroll
+                    for (int r = 0; r < R0; ++r) out[stockham_out<R0, 1>(j, r) * W + col] = pol_pack(v[r]);
+                }
+            }
+            cp_async_wait<0>();
+        } else if (t > tlo) {
+            const int tt = t - 1;
+            const float4 *src = s_a + (tt & 1) * N * W;
+#pragma unroll
+            for (int k = 0; k < kBlock / HB; ++k) {
+                const int colL = (u + k * HB) % W, jL = (u + k * HB) / W;
+                Pol2 v[RL];
+#pragma unroll
+                for (int r = 0; r < RL; ++r) v[r] = pol_unpack(src[(jL + r * NS) * W + colL]);
+                ptwiddle<RL, NS>(v, jL, s_tw + TW::OFF1);
+                pdft<RL>(v);
+                if constexpr (TAPS) pol_taps<RL, NS>(a, v, tt, cl, c, kx0 + colL, jL, sc);
+#pragma unroll
+                for (int r = 0; r < RL; ++r) {
+                    const int i = k * RL + r;
+                    pw[i] = dftc::fma2(v[r].re, v[r].re, dftc::fma2(v[r].im, v[r].im, pw[i]));
+                    xr[i] = fmaf(v[r].re.x, v[r].re.y, fmaf(v[r].im.x, v[r].im.y, xr[i]));
+                    xi[i] = fmaf(v[r].im.x, v[r].re.y, fmaf(-v[r].re.x, v[r].im.y, xi[i]));
+                }
+            }
+        }
+        __syncthreads();
+    }
+    auto value = [&](int q, int i) -> float { return q == 0 ? pw[i].x : (q == 1 ? pw[i].y : (q == 2 ? xr[i] : xi[i])); };
+    if constexpr (MODE == 1) {   // the cluster's parts in rank order (cols_finish)
+        namespace cg = cooperative_groups;
+        cg::cluster_group cl_g = cg::this_cluster();
+        float *part = reinterpret_cast<float *>(s_a);
+        const int rank = (int)cl_g.block_rank(), nz = gridDim.z;
+        if (rank > 0 && second) {
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+#pragma unroll
+                for (int i = 0; i < RL2; ++i) part[(q * RL2 + i) * HB + u] = value(q, i);
+        }
+        cl_g.sync();
+        if (rank == 0 && second) {
+            for (int z = 1; z < nz; ++z) {
+                const float *o = cl_g.map_shared_rank(part, z) + u;
+#pragma unroll
+                for (int i = 0; i < RL2; ++i) {
+                    pw[i].x += o[i * HB];
+                    pw[i].y += o[(RL2 + i) * HB];
+                    xr[i] += o[(2 * RL2 + i) * HB];
+                    xi[i] += o[(3 * RL2 + i) * HB];
+                }
+            }
+        }
+        cl_g.sync();
         if (rank > 0) return;
     }
-    // Fold this chunk's FP32 sums into the FP64 accumulators (one owner per pixel).
-    // The additions happen in L2 (in a persistent launch another SM folded the previous chunk): on the FP64 pipe the
-    // conversion and the sum were 4 to 7 % of a 128-sample chunk.
-    const double sc2 = H16 ? (double)sc * (double)sc : 1.0;
-    const int se = H16 ? pow2_exp(sc2) : 0;
-    const int kx = kx0 + colL;
+    if (!second) return;
+    const double sc2 = (double)sc * (double)sc;
+    const int se = pow2_exp(sc2);
 #pragma unroll
-    for (int q = 0; q < NPROD; ++q) {
-        double *d = a.acc + ((long long)c * NPROD + q) * N * N + (long long)jL * N + kx;
+    for (int q = 0; q < 4; ++q)
 #pragma unroll
-        for (int r = 0; r < RL; ++r) red_scaled(d + r * CS::NS * N, acc[q][r], se, sc2);
-    }
+        for (int i = 0; i < RL2; ++i) {
+            const int k = i / RL, r = i % RL, colL = (u + k * HB) % W, jL = (u + k * HB) / W;
+            red_scaled(a.acc + ((long long)c * 4 + q) * N * N + (long long)(jL + r * NS) * N + kx0 + colL, value(q, i), se, sc2);
+        }
+}
+
+// The shape's column kernel in a persistent launch (launch_cols_t's choice).
+template <int N, int P, bool H16, bool TAPS, int MODE>
+__device__ __forceinline__ void cols_any(const ColArgs &a, const int sx, const int cl, const int nz = 1) {
+    if constexpr (cols_use_pol<N, P, H16>()) cols_pol<N, H16, TAPS, MODE>(a, sx, cl, nz);
+    else cols_acc<N, P, H16, TAPS, MODE>(a, sx, cl, nz);
 }
 
 template <int N, int P, bool H16, bool TAPS, bool SPLIT>
 __global__ void __launch_bounds__(kBlock) k_cols_acc(const ColArgs a) {
     cols_acc<N, P, H16, TAPS, SPLIT ? 1 : 0>(a, blockIdx.x, blockIdx.y);
+}
+template <int N, bool H16, bool TAPS, bool SPLIT>
+__global__ void __launch_bounds__(kBlock, N == 256 ? 1 : 2) k_cols_pol(const ColArgs a) {
+    cols_pol<N, H16, TAPS, SPLIT ? 1 : 0>(a, blockIdx.x, blockIdx.y);
+}
+template <int N, bool TAPS, bool SPLIT>
+__global__ void __launch_bounds__(kBlock, 2) k_cols_duo(const ColArgs a) {
+    cols_duo<N, TAPS, SPLIT ? 1 : 0>(a, blockIdx.x, blockIdx.y);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -839,7 +1258,7 @@ __global__ void __launch_bounds__(kBlock) k_image_persist(const __grid_constant_
             ca.nt = ch.y;
             ca.c0 = ch.z;
             ca.nc = ch.w;
-            cols_acc<N, P, false, false, 2>(ca, w.z, w.w, cols_parts<N, P, false>(ca.nt, ca.nc));
+            cols_any<N, P, false, false, 2>(ca, w.z, w.w, cols_parts<N, P, false>(ca.nt, ca.nc));
         }
         __threadfence();
         __syncthreads();
@@ -944,11 +1363,23 @@ cudaError_t launch_grid_p(int TB, bool staged, bool go, const GridArgs &a, int n
 
 template <int N, int P, bool H16>
 cudaError_t launch_cols_t(const ColArgs &a, cudaStream_t st) {
+    // Two pols: the FP16 field of N <= 128 takes cols_duo (us, cols_acc -> cols_duo: 64 grid, 256 channels x 256 samples
+    // 688 -> 647; 128 grid, 128 x 256 1242 -> 1186), N >= 256 cols_pol (FP32, 256 grid, 32 x 256 2396 -> 1680; FP32, 512
+    // grid, 8 x 128 1585 -> 991; FP16, 256 grid, 64 x 256 3224 -> 2864).  The FP32 field of N <= 128 stays with cols_acc:
+    // its columns run at 0.84 of the copy bandwidth.
     const int nz = cols_parts<N, P, H16>(a.nt, a.nc);
     // pixel taps (feedback calibration, beams) compiled in only where asked for
     const bool taps = a.etap || a.n_beam;
-    auto k = nz > 1 ? (taps ? k_cols_acc<N, P, H16, true, true> : k_cols_acc<N, P, H16, false, true>)
-                    : (taps ? k_cols_acc<N, P, H16, true, false> : k_cols_acc<N, P, H16, false, false>);
+    void (*k)(ColArgs);
+    if constexpr (cols_use_duo<N, P, H16>())
+        k = nz > 1 ? (taps ? k_cols_duo<N, true, true> : k_cols_duo<N, false, true>)
+                   : (taps ? k_cols_duo<N, true, false> : k_cols_duo<N, false, false>);
+    else if constexpr (cols_use_pol<N, P, H16>())
+        k = nz > 1 ? (taps ? k_cols_pol<N, H16, true, true> : k_cols_pol<N, H16, false, true>)
+                   : (taps ? k_cols_pol<N, H16, true, false> : k_cols_pol<N, H16, false, false>);
+    else
+        k = nz > 1 ? (taps ? k_cols_acc<N, P, H16, true, true> : k_cols_acc<N, P, H16, false, true>)
+                   : (taps ? k_cols_acc<N, P, H16, true, false> : k_cols_acc<N, P, H16, false, false>);
     const size_t smem = col_smem_bytes_t<N>(P, H16);
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;

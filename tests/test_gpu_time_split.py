@@ -47,15 +47,25 @@ def test_short_blocks(N, P, T):
                                atol=1e-5 * img[0, :P].max(), rtol=0)
 
 
-@pytest.mark.parametrize("fp16", [False, True])
-def test_short_blocks_of_the_fp16_field(fp16):
-    pos, taps, codes, gains = case(9, 40, 64, 2, 2, 100)
-    with moff.Plan(pos, taps, 64, 2, 2, fp16tc=fp16) as pl:
+@pytest.mark.parametrize("N", [32, 64, 128, 256, 512])
+@pytest.mark.parametrize("C,T", [(1, 1), (2, 100), (80, 5), (80, 130)])
+def test_fp16_field(N, C, T):
+    """The FP16 field's column kernels, split and whole, at odd sample counts (3e-3, the reduced-precision bar)."""
+    if N == 512 and C == 80:
+        C = 20
+    pos, taps, codes, gains = case(N + T, 12, N, 2, C, T)
+    with moff.Plan(pos, taps, N, C, 2, fp16tc=True) as pl:
+        assert pl.route() == "fp16_rowspec"
         pl.set_gains(gains)
+        pl.set_beams([N // 3], [N // 5])
         pl.submit(codes)
+        beams = pl.read_beams()
         img, _ = pl.read_image()
-    err = oracle.max_norm_err(img, oracle.moff_image(codes, gains, pos, taps, 64, 2)).max()
-    assert err <= (3e-3 if fp16 else 1e-5)
+    pick = [0, C - 1]
+    ref = oracle.moff_image(np.ascontiguousarray(codes[:, pick]), gains[pick], pos, taps, N, 2)
+    assert oracle.max_norm_err(img[pick], ref).max() <= 3e-3
+    power = (np.abs(beams[:, :, 0].astype(np.complex128)) ** 2).sum(axis=0)
+    np.testing.assert_allclose(power, img[:, :2, N // 5, N // 3], atol=1e-5 * img[:, :2].max(), rtol=0)
 
 
 @pytest.mark.parametrize("A,N,P,K", [(64, 32, 1, 5), (300, 128, 2, 5), (700, 128, 2, 9), (700, 256, 2, 5), (3000, 256, 2, 9),
