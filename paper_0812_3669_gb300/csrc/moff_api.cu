@@ -122,26 +122,22 @@ std::vector<float2> pass_twiddles_n(int n) {
 
 bool is_pow2(long long v) { return v > 0 && (v & (v - 1)) == 0; }
 
-// FP64 sums -> FP32 image; RESET also starts the next integration (one pass instead of a memset behind it).  Nothing is
-// read or reset once a kernel of the plan has recorded a failed wait (err).
-template <bool RESET>
-__global__ void __launch_bounds__(256) k_to_f32(double *__restrict__ a, float *__restrict__ o, long long n4,
+// FP64 sums -> FP32 image; nothing is written once a kernel of the plan has recorded a failed wait (err).  (Zeroing the
+// sums in the same pass took 612 us for 67 M values; this 143 and a memset behind it 80.)
+__global__ void __launch_bounds__(256) k_to_f32(const double *__restrict__ a, float *__restrict__ o, long long n4,
                                                 const int *__restrict__ err) {
     if (err && *err) return;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n4; i += (long long)gridDim.x * blockDim.x) {
-        double2 *p = reinterpret_cast<double2 *>(a) + 2 * i;
+        const double2 *p = reinterpret_cast<const double2 *>(a) + 2 * i;
         const double2 u = p[0], v = p[1];
-        if (RESET) p[0] = p[1] = make_double2(0.0, 0.0);
         reinterpret_cast<float4 *>(o)[i] = make_float4((float)u.x, (float)u.y, (float)v.x, (float)v.y);
     }
 }
-__global__ void __launch_bounds__(256) k_to_f32_any(double *__restrict__ a, float *__restrict__ o, long long n,
-                                                    const int *__restrict__ err, int reset) {
+__global__ void __launch_bounds__(256) k_to_f32_any(const double *__restrict__ a, float *__restrict__ o, long long n,
+                                                    const int *__restrict__ err) {
     if (err && *err) return;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
         o[i] = (float)a[i];
-        if (reset) a[i] = 0.0;
-    }
 }
 
 }  // namespace
@@ -218,14 +214,13 @@ cudaError_t launch_persist(int N, int P, int cpl, bool wide, const PersistArgs &
     return cudaErrorInvalidValue;
 }
 
-cudaError_t launch_to_f32(double *acc, float *out, long long n, cudaStream_t st, const int *err, bool reset) {
+cudaError_t launch_to_f32(const double *acc, float *out, long long n, cudaStream_t st, const int *err) {
     // images are whole multiples of 1024 values; an output that is no 16-byte aligned buffer goes value by value
     const bool vec = n % 4 == 0 && (((uintptr_t)acc | (uintptr_t)out) & 15) == 0;
     const long long m = vec ? n / 4 : n;
     const unsigned blocks = (unsigned)std::max(1LL, std::min<long long>((m + 255) / 256, 152LL * 16));
-    if (!vec) k_to_f32_any<<<blocks, 256, 0, st>>>(acc, out, n, err, reset ? 1 : 0);
-    else if (reset) k_to_f32<true><<<blocks, 256, 0, st>>>(acc, out, m, err);
-    else k_to_f32<false><<<blocks, 256, 0, st>>>(acc, out, m, err);
+    if (vec) k_to_f32<<<blocks, 256, 0, st>>>(acc, out, m, err);
+    else k_to_f32_any<<<blocks, 256, 0, st>>>(acc, out, n, err);
     return cudaGetLastError();
 }
 
@@ -2856,32 +2851,29 @@ moff_status moff_read_image(moff_plan *pl, float *out, long long *n_samples, int
     if (s != MOFF_OK) return s;
     if (!out) return fail(MOFF_EINVAL, "out is NULL");
     const long long n = (long long)pl->C * pl->nprod * pl->N * pl->N;
-    auto done = [&]() -> moff_status {
-        if (n_samples) *n_samples = pl->n_samples;
-        if (reset) {
-            pl->n_samples = 0;
-            if (pl->auto_on) {   // the autocorrelation sums follow the integration
-                MOFF_CK(cudaMemsetAsync(pl->d_auto_pw, 0, (size_t)pl->C * pl->A * 3 * 16, pl->st));
-                pl->auto_samples = 0;
-            }
-        }
-        return MOFF_OK;
-    };
-    if (out_on_device) {   // conversion, reset and status word behind the plan's work, one wait for all of it
+    if (out_on_device) {   // conversion and status word behind the plan's work, one wait for all of it
         if (timeout_ms >= 0 && (s = sync_plan(pl, timeout_ms)) != MOFF_OK) return s;
-        MOFF_CK(launch_to_f32(pl->d_acc, out, n, pl->st, pl->d_err, reset != 0));
+        MOFF_CK(launch_to_f32(pl->d_acc, out, n, pl->st, pl->d_err));
         if (pl->d_err) MOFF_CK(cudaMemcpyAsync(pl->h_err, pl->d_err, sizeof(int), cudaMemcpyDeviceToHost, pl->st));
         if ((s = sync_plan(pl, -1)) != MOFF_OK) return s;
         if (pl->d_err && *pl->h_err) return check_device_err(pl);
-        return done();
+    } else {
+        if ((s = sync_plan(pl, timeout_ms)) != MOFF_OK) return s;
+        if ((s = check_device_err(pl)) != MOFF_OK) return s;
+        MOFF_CK(launch_to_f32(pl->d_acc, pl->d_img, n, pl->st));
+        MOFF_CK(cudaMemcpyAsync(out, pl->d_img, (size_t)n * 4, cudaMemcpyDeviceToHost, pl->st));
+        if ((s = sync_plan(pl, -1)) != MOFF_OK) return s;
     }
-    if ((s = sync_plan(pl, timeout_ms)) != MOFF_OK) return s;
-    if ((s = check_device_err(pl)) != MOFF_OK) return s;
-    MOFF_CK(launch_to_f32(pl->d_acc, pl->d_img, n, pl->st));
-    MOFF_CK(cudaMemcpyAsync(out, pl->d_img, (size_t)n * 4, cudaMemcpyDeviceToHost, pl->st));
-    if ((s = sync_plan(pl, -1)) != MOFF_OK) return s;
-    if (reset) MOFF_CK(cudaMemsetAsync(pl->d_acc, 0, (size_t)n * 8, pl->st));
-    return done();
+    if (n_samples) *n_samples = pl->n_samples;
+    if (reset) {
+        MOFF_CK(cudaMemsetAsync(pl->d_acc, 0, (size_t)n * 8, pl->st));
+        pl->n_samples = 0;
+        if (pl->auto_on) {   // the autocorrelation sums follow the integration
+            MOFF_CK(cudaMemsetAsync(pl->d_auto_pw, 0, (size_t)pl->C * pl->A * 3 * 16, pl->st));
+            pl->auto_samples = 0;
+        }
+    }
+    return MOFF_OK;
 }
 
 moff_status moff_sync(moff_plan *pl, int timeout_ms) {

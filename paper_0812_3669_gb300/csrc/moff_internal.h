@@ -375,8 +375,7 @@ cudaError_t launch_pfb(int CN, const PfbArgs &a, cudaStream_t st);
 // spec_sm ([AP][F][C]), then the reorder to codes / spec ([F][C][AP]).
 cudaError_t launch_pfb1024(const PfbArgs &a, cudaStream_t st);
 cudaError_t launch_pfb_reorder(const PfbArgs &a, cudaStream_t st);
-cudaError_t launch_to_f32(double *acc, float *out, long long n, cudaStream_t st, const int *err = nullptr,
-                          bool reset = false);
+cudaError_t launch_to_f32(const double *acc, float *out, long long n, cudaStream_t st, const int *err = nullptr);
 
 // Tensor-core path (moff_tc_kernels.cu).
 constexpr int kRowSpecMaxK = 256;   // largest contraction length (64 per 32-voltage chunk) held on chip
