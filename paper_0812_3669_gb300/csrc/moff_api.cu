@@ -21,6 +21,7 @@
 #include <mutex>
 #include <string>
 #include <thread>
+#include <tuple>
 #include <vector>
 
 #include "../../include/moff.h"
@@ -1260,11 +1261,23 @@ moff_status build_bins(int A, int K, int N, int P, bool jones, const double *pos
         return 2 * (u / (N / 2)) * N + 2 * (u % (N / 2));
     };
     std::vector<std::vector<Ent>> lists(nunit);
-    std::vector<int> order(nunit);
+    std::vector<int> order(nunit), by_pos, slot;
     const float2 zero = make_float2(0.f, 0.f);
     for (int s = 0; s < ns; ++s) {
         b->ant_off[s + 1] = b->ant_off[s] + (int)sant[s].size();
-        b->ant_list.insert(b->ant_list.end(), sant[s].begin(), sant[s].end());
+        // Voltage slots in raster order of the anchors: neighbouring lanes gather from neighbouring antennas, whose slots
+        // lie in different banks (volt_at).  The entries keep the antennas' order, and so every sum its own.
+        by_pos.resize(sant[s].size());
+        for (size_t i = 0; i < by_pos.size(); ++i) by_pos[i] = (int)i;
+        std::sort(by_pos.begin(), by_pos.end(), [&](int x, int y) {
+            const int u = sant[s][x], v = sant[s][y];
+            return std::tie(ay[u], ax[u], u) < std::tie(ay[v], ax[v], v);
+        });
+        slot.assign(std::max<size_t>(by_pos.size(), 1), 0);
+        for (size_t i = 0; i < by_pos.size(); ++i) {
+            slot[by_pos[i]] = (int)i;
+            b->ant_list.push_back(sant[s][by_pos[i]]);
+        }
         auto &v = scon[s];
         std::stable_sort(v.begin(), v.end(), [](const Contrib &x, const Contrib &y) { return x.cell < y.cell; });
         for (auto &l : lists) l.clear();
@@ -1313,7 +1326,7 @@ moff_status build_bins(int A, int K, int N, int P, bool jones, const double *pos
                     const auto &L = lists[order[k * 32 + l]];
                     const Ent en = e < L.size() ? L[e] : Ent{0, {zero, zero, zero, zero}};
                     for (int c2 = 0; c2 < cpl; ++c2) b->con_tap.push_back(en.t[c2]);
-                    b->con_y.push_back((uint16_t)en.y);
+                    b->con_y.push_back((uint16_t)volt_at(P, b->tb, slot[en.y / P], en.y % P));
                 }
             for (int l = 0; l < 32; ++l)
                 b->lane_cell[si * 32 + l] = (uint16_t)first_cell(order[k * 32 + l]);

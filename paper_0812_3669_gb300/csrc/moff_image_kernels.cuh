@@ -197,7 +197,7 @@ __device__ __forceinline__ void grid_rows(const GridArgs &a, const int s, const 
     float2 *s_tw = reinterpret_cast<float2 *>(smem + DREG);
     float2 *s_buf = s_tw + (DFT ? 0 : TW::TOTAL);      // gridded rows
     float2 *s_alt = ONEBUF ? s_buf : s_buf + F * LDR;  // second buffer of the row passes (none in place)
-    float2 *s_y = s_alt + ((F * LDR + 1) & ~1);        // [nloc*P][YS]: TB samples, padded row (16-byte aligned)
+    float2 *s_y = s_alt + ((F * LDR + 1) & ~1);        // voltages of TB samples (volt_at; 16-byte aligned), at most YS per antenna-pol
     float2 *s_g = s_y + YS * a.max_nloc * P;
     // staged kernel values (CPL per entry, read as 16-byte vectors when CPL >= 2: 16-byte aligned)
     float2 *s_tap = reinterpret_cast<float2 *>((reinterpret_cast<uintptr_t>(s_g + a.max_nloc * P) + 15) & ~uintptr_t(15));
@@ -270,7 +270,7 @@ __device__ __forceinline__ void grid_rows(const GridArgs &a, const int s, const 
                 const int yi = tid + m * kBlock;
                 if (yi < nyi) {
                     const float2 g = s_g[yi];
-                    float2 *yrow = s_y + yi * YS;
+                    float2 *yrow = s_y + volt_at(P, TB, yi / P, yi % P);
 #pragma unroll
                     for (int t = 0; t < TB; ++t) yrow[t] = t < nb ? cmul(g, decode4(vb[m][t])) : make_float2(0.f, 0.f);
                 }
@@ -281,7 +281,7 @@ __device__ __forceinline__ void grid_rows(const GridArgs &a, const int s, const 
                 const int la = yi / P, q = yi - la * P;
                 const float2 g = s_g[yi];
                 const uint8_t *src = vchan + (long long)(a.t0 + tb0) * a.volt_tstride + (long long)s_ant[la] * P + q;
-                float2 *yrow = s_y + yi * YS;
+                float2 *yrow = s_y + volt_at(P, TB, yi / P, yi % P);
                 for (int t = 0; t < TB; ++t)
                     yrow[t] = t < nb ? cmul(g, decode4(src[t * a.volt_tstride])) : make_float2(0.f, 0.f);
             }
@@ -346,7 +346,7 @@ __device__ __forceinline__ void grid_rows(const GridArgs &a, const int s, const 
                 load_ent(i0 + U, tn, yn);
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
-                    const float2 *yy = s_y + yv[u] * YS;
+                    const float2 *yy = s_y + yv[u];
                     if constexpr (TB >= 2) {
 #pragma unroll
                         for (int t = 0; t < TB; t += 2) {
