@@ -116,19 +116,32 @@ __global__ void __launch_bounds__(256) k_auto_acc(const FbArgs a) {
 // Q[c][q][u] = sum_a pw[c][a][q] X[a][q][u]: the antennas' kernel cross-correlation
 // patches weighted by their autocorrelation sums (FP64).  One thread per (q, u) of a channel.
 // With channel-dependent kernels, X holds one [A][NQ][U] block per set and chan_group[c] picks it.
-__global__ void k_auto_patch(const double2 *__restrict__ pw, const double2 *__restrict__ X,
-                             const int *__restrict__ chan_group, int A, int NQ, int U, double2 *__restrict__ Q) {
-    const int c = blockIdx.y;
+// The sum is over all antennas in FP64, whose pipe does two operations a cycle and SM: eight threads share a (q, u), their
+// partial sums added in order, so that all SMs take part (one thread each used 64 blocks of a 32-channel plan).
+constexpr int kPatchK = 32;                                 // (q, u) per block
+__global__ void __launch_bounds__(256) k_auto_patch(const double2 *__restrict__ pw, const double2 *__restrict__ X,
+                                                    const int *__restrict__ chan_group, int A, int NQ, int U,
+                                                    double2 *__restrict__ Q) {
+    __shared__ double2 s_part[8][kPatchK];
+    const int c = blockIdx.y, kl = threadIdx.x % kPatchK, g = threadIdx.x / kPatchK;
     if (chan_group) X += (long long)chan_group[c] * A * NQ * U;
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;    // q * U + u
-    if (k >= NQ * U) return;
-    const int q = k / U;
+    const int k = blockIdx.x * kPatchK + kl;                // q * U + u
     double re = 0.0, im = 0.0;
-    for (int an = 0; an < A; ++an) {
-        const double2 w = pw[((long long)c * A + an) * 3 + q];
-        const double2 x = X[((long long)an * NQ + q) * U + (k - q * U)];
-        re += w.x * x.x - w.y * x.y;
-        im += w.x * x.y + w.y * x.x;
+    if (k < NQ * U) {
+        const int q = k / U;
+        for (int an = g; an < A; an += 8) {
+            const double2 w = pw[((long long)c * A + an) * 3 + q];
+            const double2 x = X[((long long)an * NQ + q) * U + (k - q * U)];
+            re += w.x * x.x - w.y * x.y;
+            im += w.x * x.y + w.y * x.x;
+        }
+    }
+    s_part[g][kl] = make_double2(re, im);
+    __syncthreads();
+    if (g || k >= NQ * U) return;
+    for (int i = 1; i < 8; ++i) {
+        re += s_part[i][kl].x;
+        im += s_part[i][kl].y;
     }
     Q[(long long)c * NQ * U + k] = make_double2(re, im);
 }
@@ -154,7 +167,7 @@ __global__ void __launch_bounds__(256) k_auto_image(const double2 *__restrict__ 
         if (kx < N)
             for (int ux = 0; ux < L; ++ux) {
                 const double2 v = s_q[uy * L + ux];
-                const double2 w = s_w[(((long long)kx * (ux - h)) % N + N) % N];
+                const double2 w = s_w[(kx * (ux - h)) & (N - 1)];
                 re += v.x * w.x - v.y * w.y;
                 im += v.x * w.y + v.y * w.x;
             }
@@ -167,9 +180,9 @@ __global__ void __launch_bounds__(256) k_auto_image(const double2 *__restrict__ 
         double re = 0.0, im = 0.0;
         for (int uy = 0; uy < L; ++uy) {
             const double2 v = s_t[uy * 64 + kl];
-            const double2 w = s_w[(((long long)ky * (uy - h)) % N + N) % N];
+            const double2 w = s_w[(ky * (uy - h)) & (N - 1)];    // N is a power of two
             re += v.x * w.x - v.y * w.y;
-            im += v.x * w.y + v.y * w.x;
+            if (q == 2) im += v.x * w.y + v.y * w.x;              // XX and YY are real
         }
         const long long pix = (long long)ky * N + kx;
         if (q < 2) {
@@ -197,7 +210,7 @@ cudaError_t launch_auto_acc(const FbArgs &a, cudaStream_t st) {
 cudaError_t launch_auto_image(const double2 *pw, const double2 *X, const int *chan_group, int C, int A, int P, int K,
                               int N, const double2 *wN, double2 *Q, double *img, cudaStream_t st) {
     const int NQ = P == 1 ? 1 : 3, L = 2 * K - 1, U = L * L;
-    k_auto_patch<<<dim3((NQ * U + 255) / 256, C), 256, 0, st>>>(pw, X, chan_group, A, NQ, U, Q);
+    k_auto_patch<<<dim3((NQ * U + kPatchK - 1) / kPatchK, C), 256, 0, st>>>(pw, X, chan_group, A, NQ, U, Q);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     const size_t smem = ((size_t)N + U + (size_t)L * 64) * sizeof(double2);
