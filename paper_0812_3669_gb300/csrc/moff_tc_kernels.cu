@@ -20,7 +20,10 @@
 //                  A = 128 samples of the row's segment voltages (TMA tiles of 32 plane rows,
 //                  128-byte swizzled, MN-major),
 //                  D = TMEM (double buffered), epilogue writes the row-transformed field in
-//                  FP16 under an exact power-of-two scale (undone by the column kernel).
+//                  FP16 under an exact power-of-two scale (undone by the column kernel).  B arrives by one bulk
+//                  copy while the first chunks of A are under way: with all threads copying it before the roles began
+//                  the kernel took 6693 us for 256 channels x 1000 samples of 1024 antennas, now 5765 (the field
+//                  written and the planes read take 4.5 ms at the copy bandwidth).
 #include <cuda_fp16.h>
 
 #include "moff_fft.cuh"
@@ -411,21 +414,16 @@ __global__ void __launch_bounds__(kTcRoleThreads, 1)
     unsigned char *sE = sA + (size_t)kAStages * kAChunkBytes;  // [kEpiWarps][kEpiBufs] boxes, 1024-aligned
     uint64_t *bars = reinterpret_cast<uint64_t *>(sE + kEpiWarps * kEpiBufs * kBoxBytes);
     uint64_t *a_full = bars, *a_empty = bars + kAStages, *d_full = bars + 2 * kAStages,
-             *d_empty = bars + 2 * kAStages + 2;
-    uint32_t *tslot = reinterpret_cast<uint32_t *>(bars + 2 * kAStages + 4);
+             *d_empty = bars + 2 * kAStages + 2, *b_full = bars + 2 * kAStages + 4;
+    uint32_t *tslot = reinterpret_cast<uint32_t *>(bars + 2 * kAStages + 5);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(tslot + 1);
 
-    {
-        const uint4 *src = reinterpret_cast<const uint4 *>(a.bimg + a.bimg_off[item]);
-        uint4 *dst = reinterpret_cast<uint4 *>(sB);
-        const int n16 = NT * kp * 2 / 16;
-        for (int i = tid; i < n16; i += blockDim.x) dst[i] = src[i];
-    }
     if (tid == 0) {
         for (int b = 0; b < kAStages; ++b) {
             tc::mbar_init(&a_full[b], 1);        // the producer's arrive + the chunk's TMA bytes
             tc::mbar_init(&a_empty[b], 1);
         }
+        tc::mbar_init(b_full, 1);
         for (int b = 0; b < 2; ++b) {
             tc::mbar_init(&d_full[b], 1);
             tc::mbar_init(&d_empty[b], kEpiWarps * 32);
@@ -436,17 +434,21 @@ __global__ void __launch_bounds__(kTcRoleThreads, 1)
         tc::tmem_alloc(tslot, S::TCOLS);
         tc::tmem_relinquish();
     }
-    tc::fence_async_smem();   // resident B written by generic stores, read by the tensor core
+    tc::fence_async_smem();
     tc::fence_before_sync();
     __syncthreads();
     tc::fence_after_sync();
     const uint32_t tbase = *tslot;
 
     if (warp == kEpiWarps) {
-        // ---------------- producer (the whole warp runs it, one elected lane issues): chunk after chunk into the
-        // ring, one box of both planes per 64-sample half completing on a_full; the chunks' plane rows (at most
-        // four) stay in the lanes' registers.
+        // ---------------- producer (the whole warp runs it, one elected lane issues): B by one bulk copy (completing on
+        // b_full), then chunk after chunk into the ring, one box of both planes per 64-sample half completing on
+        // a_full; the chunks' plane rows (at most four) stay in the lanes' registers.
         const uint32_t one = tc::elect_one();
+        if (one) {
+            tc::mbar_arrive_expect_tx(b_full, (uint32_t)(NT * kp * 2));
+            tc::bulk_load(tc::smem_u32(sB), a.bimg + a.bimg_off[item], (uint32_t)(NT * kp * 2), b_full);
+        }
         const int row_l = lane < nchunk ? a.chunk_row[ch0 + lane] : 0;
         int g = 0, st = 0;
         uint32_t ph = 1;
@@ -467,6 +469,7 @@ __global__ void __launch_bounds__(kTcRoleThreads, 1)
         // tiles still landing (the MMA warp stopped early): let them finish before the shared memory is released
         for (int gg = g - kAStages > 0 ? g - kAStages : 0; gg < g; ++gg)
             tc::mbar_wait_bounded(&a_full[gg % kAStages], (uint32_t)((gg / kAStages) & 1), kWaitCycles);
+        tc::mbar_wait_bounded(b_full, 0, kWaitCycles);
     } else if (warp == kEpiWarps + 1) {
         // ---------------- MMA issuer (one elected lane of the warp issues)
         const uint32_t one = tc::elect_one();
@@ -475,7 +478,7 @@ __global__ void __launch_bounds__(kTcRoleThreads, 1)
         const uint32_t sbb = tc::smem_u32(sB);
         int st = 0;
         uint32_t ph = 0;
-        bool ok = true;
+        bool ok = tc::mbar_wait_warp(b_full, 0, kWaitCycles, abort_flag);
         for (int i = 0; i < nitems && ok; ++i) {
             const int b = i & 1;
             if (!(ok = tc::mbar_wait_warp(&d_empty[b], (uint32_t)(((i >> 1) & 1) ^ 1), kWaitCycles, abort_flag))) break;
@@ -569,7 +572,7 @@ __global__ void __launch_bounds__(kTcRoleThreads, 1)
 size_t rowspec_smem_bytes(int N, int kp_max) {
     const int KX = N < 128 ? N : 128, NT = 2 * KX;
     size_t b = 1024 + (size_t)NT * kp_max * 2 + (size_t)kAStages * kAChunkBytes +
-               (size_t)kEpiWarps * kEpiBufs * kBoxBytes + (size_t)(2 * kAStages + 4) * 8 + 8;
+               (size_t)kEpiWarps * kEpiBufs * kBoxBytes + (size_t)(2 * kAStages + 5) * 8 + 8;
     b = (b + 127) & ~(size_t)127;
     // one CTA per SM: two CTAs must never wait on each other's TMEM columns
     return b < 120 * 1024 ? 120 * 1024 : b;
