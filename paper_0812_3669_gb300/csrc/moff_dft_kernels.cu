@@ -1,17 +1,19 @@
-// moff_dft_kernels.cu -- the column half of Eq. m6 step 3 (Morales, arXiv
-// 0812.3669) as factored DFT contractions on the tensor cores, fused with step 4
+// moff_dft_kernels.cu -- the row and column transforms of Eq. m6 step 3 (Morales, arXiv
+// 0812.3669) as factored DFT contractions on the tensor cores, the columns fused with step 4
 // (|E|^2 and the cross-pol products summed over a chunk, then added to the FP64
-// accumulators), for the dense FP16 path.  The row half runs inside the
-// gridding kernel (k_grid_rows_dft, moff_dft.cuh).
+// accumulators), for the dense FP16 path.  (The FP32 gather's row transform runs inside the
+// gridding kernel: k_grid_rows_dft, moff_dft.cuh.)
 //
-//   k_cols_dft  one CTA = 16 columns of one channel walking a chunk of samples.
-//               Per sample: the FP16 field's 16-column strip (cp.async, 32-byte
-//               pieces of the reached rows) lands as the stage-1 A operand
-//               (rows (b, x), k = (a, re/im)); stage 1 on the tensor cores; the
-//               twiddled FP32 result is written back as the stage-2 A operand
-//               (128-byte swizzled, rows (c, x)); stage 2 leaves E in TMEM,
-//               where the epilogue squares and sums it.  Loads of sample t + 1 and
-//               stage 1 of sample t run while the epilogue of sample t - 1 works.
+//   k_rows_dft8  one CTA = a stripe of grid rows of one channel walking a chunk of samples.
+//   k_cols_pipe  one CTA = 8 (or 16) columns of one channel walking a chunk of samples, each
+//                step on warps of its own.
+//   k_cols_dft   the same work with block barriers between the steps: 16 columns on the 512
+//                grid, whose accumulators leave no TMEM for a second buffer.  Per sample: the FP16
+//                field's strip (cp.async) lands as the stage-1 A operand (rows (b, x), k = (a,
+//                re/im)); stage 1 on the tensor cores; the twiddled FP32 result is written back as
+//                the stage-2 A operand (128-byte swizzled, rows (c, x)); stage 2 leaves E in TMEM,
+//                where the epilogue squares and sums it.  Loads of sample t + 1 and stage 1 of
+//                sample t run while the epilogue of sample t - 1 works.
 #include <cuda_fp16.h>
 
 #include <cmath>
@@ -1046,21 +1048,9 @@ cudaError_t launch_rows_dft8(int N, int P, const RowDftArgs &a, cudaStream_t st)
     return cudaErrorInvalidValue;
 }
 
-// Columns per CTA by default: 8 (two CTAs per SM, so one CTA's epilogue runs while the other
-// waits on its MMAs) unless MOFF_COLS_W=16 (one CTA per SM); MOFF_AUTOTUNE times both.
+// Columns per CTA by default: 8 (k_cols_pipe) unless MOFF_COLS_W=16; MOFF_AUTOTUNE times both.
 int cols_dft_width() { return (getenv("MOFF_COLS_W") && atoi(getenv("MOFF_COLS_W")) == 16) ? 16 : 8; }
 bool cols_dft_width_forced() { return getenv("MOFF_COLS_W") != nullptr; }
-
-size_t cols_dft_smem_bytes(int N, int P, int W) {
-    if (W == 16) {
-        if (N == 512) return P == 1 ? ColDftShape<512, 1, 16>::SMEM : ColDftShape<512, 2, 16>::SMEM;
-        if (N == 256) return P == 1 ? ColDftShape<256, 1, 16>::SMEM : ColDftShape<256, 2, 16>::SMEM;
-    } else {
-        if (N == 512) return P == 1 ? ColDftShape<512, 1, 8>::SMEM : ColDftShape<512, 2, 8>::SMEM;
-        if (N == 256) return P == 1 ? ColDftShape<256, 1, 8>::SMEM : ColDftShape<256, 2, 8>::SMEM;
-    }
-    return 0;
-}
 
 cudaError_t launch_cols_dft(int N, int P, int W, const ColDftArgs &a, cudaStream_t st) {
     if (W == 16) {

@@ -8,9 +8,9 @@
 //                 chunk of samples TB at a time: each kernel entry is read
 //                 once (coalesced, sliced-ELL order, from L2) per TB samples,
 //                 and the TB x P x rows rows are transformed in place.
-//   k_cols_acc  : second axis of step 3 (column transforms) fused with step 4
-//                 (|E|^2 and the cross-pol products summed over the chunk in
-//                 registers, then added to FP64 accumulators).
+//   k_cols_acc, k_cols_pol, k_cols_duo : second axis of step 3 (column transforms)
+//                 fused with step 4 (|E|^2 and the cross-pol products summed over the
+//                 chunk in registers, then added to FP64 accumulators).
 // The row-transformed field goes through global memory between the two.
 #pragma once
 #include <cooperative_groups.h>

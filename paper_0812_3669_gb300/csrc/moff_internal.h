@@ -365,7 +365,6 @@ size_t pfb_smem_bytes(int CN);
 std::vector<unsigned char> build_dft_table(int N, bool cols = false);
 float dft_kernel_scale(int A, int K, int N, int P, bool jones, const double *pos, const float *taps);
 // W = columns per CTA of the column kernel (8 or 16).
-size_t cols_dft_smem_bytes(int N, int P, int W);
 cudaError_t launch_cols_dft(int N, int P, int W, const ColDftArgs &a, cudaStream_t st);
 int cols_dft_width();            // the default W (MOFF_COLS_W=16 selects 16)
 bool cols_dft_width_forced();    // MOFF_COLS_W set: the autotuner keeps it
