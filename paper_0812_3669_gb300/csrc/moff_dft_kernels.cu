@@ -346,6 +346,11 @@ struct ColPipeShape {
     static constexpr int A1 = P * CS::A1P, A2 = P * CS::A2P;                  // operand bytes of one sample
     static constexpr int TAB = S::B1_BYTES + S::B2_BYTES;                     // twiddles go to registers
     static constexpr int NBAR = 2 * kCpStages + 12;
+    // Groups of four twiddle warps with rows to twiddle: two tiles, or two pols of one tile; one pol of one tile leaves
+    // the second group without any.  That group keeps out of the hand-overs: only a warp that waits for the
+    // operand buffer's release (a2_empty) may arrive on a2_full, or two arrivals of its own could complete a phase that
+    // the other group, still writing, has not arrived for.
+    static constexpr int TGROUPS = CS::T1 * P >= 2 ? 2 : 1;
     static constexpr size_t SMEM = 1024 + (size_t)kCpStages * A1 + 2 * (size_t)A2 + TAB + NBAR * 8 + 16;
     static_assert(TC_ <= 512 && SMEM <= 227 * 1024 && CS::T1 <= 2, "column pipeline shape");
 };
@@ -380,8 +385,8 @@ __global__ void __launch_bounds__(kCpThreads, 1) k_cols_pipe(const ColDftArgs a)
         }
         for (int b = 0; b < 2; ++b) {
             tc::mbar_init(&d1_full[b], 1);
-            tc::mbar_init(&d1_empty[b], 8);
-            tc::mbar_init(&a2_full[b], 8);
+            tc::mbar_init(&d1_empty[b], 4 * CP::TGROUPS);
+            tc::mbar_init(&a2_full[b], 4 * CP::TGROUPS);
             tc::mbar_init(&a2_empty[b], 1);
             tc::mbar_init(&d2_full[b], 1);
             tc::mbar_init(&d2_empty[b], 8);
@@ -411,7 +416,7 @@ __global__ void __launch_bounds__(kCpThreads, 1) k_cols_pipe(const ColDftArgs a)
         // piece (c group ch, k) at a2_t + ch * (8 W / 64) * K2 * 128 + k * 128, k = b and N2 + b (same k mod 8)
         const int cgx = W == 8 ? x : (x & 7);
         const uint32_t a2_t = (uint32_t)((W == 16 ? (x >> 3) * K2 * 128 : 0) + b * 128 + ((cgx ^ (b & 7)) << 4));
-        for (int t = 0; t < a.nt; ++t) {
+        for (int t = 0; t < a.nt && g < CP::TGROUPS; ++t) {
             const int buf = t & 1;
             const uint32_t ph = (uint32_t)((t >> 1) & 1);
             if (!tc::mbar_wait_abortable(&d1_full[buf], ph, dftc::kWaitCycles, abort_flag)) break;
@@ -451,11 +456,6 @@ __global__ void __launch_bounds__(kCpThreads, 1) k_cols_pipe(const ColDftArgs a)
                 }
             }
             if (!ok) break;
-            if (P == 1 && PW == 2 && p0 == 1) {                  // one pol, one tile: this group has no rows
-                tc::fence_before_sync();
-                __syncwarp();
-                if (lane == 0) tc::mbar_arrive(&d1_empty[buf]);
-            }
             tc::fence_async_smem();
             __syncwarp();
             if (lane == 0) tc::mbar_arrive(&a2_full[buf]);

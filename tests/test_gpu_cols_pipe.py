@@ -63,3 +63,31 @@ def test_power_of_two_gains_scale_exactly(monkeypatch, shift):
     a = image(pos, taps, 256, codes, gains)
     b = image(pos, taps, 256, codes, gains * 2.0 ** shift)
     assert np.array_equal(b, np.ldexp(a, 2 * shift))
+
+
+@pytest.mark.parametrize("P", [1, 2])
+def test_hand_overs_hold_over_full_waves(monkeypatch, P):
+    """One pol of one stage-1 tile (the 256 grid at 8 columns per CTA) leaves four of the twiddle warps without
+    rows; they must not stand in for the four that write the operand.  Thirteen or more waves of CTAs, blocks of
+    four launches of 128 samples, repeated: the images equal each other bit for bit, and those of 16 columns per CTA,
+    whose twiddle warps all have rows and whose arithmetic and order of sums are the same."""
+    monkeypatch.setenv("MOFF_TC_DFT", "1")
+    N, C, T = 256, 64, 512
+    pos, taps, codes, gains = case(5 + P, 90, N, P, C, T)
+    dev = torch.from_numpy(codes).cuda()
+    images = {}
+    for width in (8, 16):
+        monkeypatch.setenv("MOFF_COLS_W", str(width))
+        with moff.Plan(pos, taps, N, C, P, fp16tc=True) as pl:
+            assert pl.route() == "fp16_tcgrid" and pl.dft_tuning()["cols_width"] == width
+            pl.set_gains(gains)
+            images[width] = []
+            for _ in range(6):
+                pl.submit(dev)
+                images[width].append(pl.read_image(reset=True)[0])
+    for width in (8, 16):
+        for img in images[width]:
+            assert np.array_equal(img, images[16][0])
+    pick = [0, C - 1]
+    ref = oracle.moff_image(np.ascontiguousarray(codes[:, pick]), gains[pick], pos, taps, N, P)
+    assert oracle.max_norm_err(images[8][0][pick], ref).max() <= 3e-3
