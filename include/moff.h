@@ -108,7 +108,8 @@ enum {
                                  MOFF_ETIMEDOUT.  FP32 path of an unserved plan only (MOFF_EINVAL
                                  with MOFF_PREC_FP16TC or MOFF_SERVED); the gridding shape is 4
                                  samples per pass with entries through L2 (MOFF_AUTOTUNE picks among
-                                 those).  Blocks with feedback calibration, beams or autocorrelation
+                                 those); sets of moff_set_channel_groups too dense for it run the
+                                 direct launches.  Blocks with feedback calibration, beams or autocorrelation
                                  subtraction on run the direct launches.  With MOFF_GRAPH the
                                  persistent launch is what the graph replays. */
 };

@@ -969,7 +969,10 @@ moff_status run_image(moff_plan *pl, const uint8_t *volt, int n_time, long long 
     if (pl->gtc) return run_image_gtc(pl, volt, n_time, tstride);
     if (pl->dft) return run_image_dft(pl, volt, n_time, tstride);
     if (pl->tc) return run_image_tc(pl, volt, n_time, tstride);
-    if (pl->persist && !pl->fb_on && !pl->auto_on && pl->n_beam == 0) return run_image_persist(pl, volt, n_time, tstride);
+    // the persistent kernel runs 4 samples per pass with entries through L2; sets of positions and kernels that fit
+    // only another shape (moff_set_channel_groups) take the direct launches
+    if (pl->persist && pl->tb == 4 && !pl->staged && !pl->fb_on && !pl->auto_on && pl->n_beam == 0)
+        return run_image_persist(pl, volt, n_time, tstride);
     for (int c0 = 0; c0 < pl->C; c0 += pl->Cb) {
         if (moff_status w = chunk_ready(pl, c0); w != MOFF_OK) return w;
         const int nc = std::min(pl->Cb, pl->C - c0);
@@ -1670,6 +1673,7 @@ moff_status upload_bins(moff_plan *pl, const Bins &b) {
     pl->max_nloc = b.max_nloc;
     pl->n_slices = b.n_slices;
     pl->grid_smem = b.grid_smem;
+    if (pl->persist) pl->persist_smem = std::max(b.grid_smem, col_smem_bytes(pl->N, pl->P));
     pl->grid_smem_fft = pl->dft ? grid_smem_bytes(pl->N, pl->P, b.tb, b.rows, b.max_nloc, fft_tw_total(pl->N), 0, b.pairs)
                                 : b.grid_smem;
     return MOFF_OK;
@@ -2405,7 +2409,6 @@ moff_status moff_plan_create(moff_plan **out, int n_ant, const double *pos, int 
         if ((flags & MOFF_AUTOTUNE) && (s = tune_cols_width(pl)) != MOFF_OK) return bail(s);
     }
     if (pl->persist) {
-        pl->persist_smem = std::max(pl->grid_smem, col_smem_bytes(grid_n, n_pol));
         if (pl->persist_smem > 227 * 1024)
             return bail(fail(MOFF_EINVAL, "MOFF_PERSIST: the persistent kernel needs %zu bytes of shared memory",
                              pl->persist_smem));

@@ -137,3 +137,56 @@ def test_dependency_wait_runs_out_and_returns_timeout(monkeypatch):
     img, n, _ = run(pos, taps, gains, 64, 4, 2, blocks, persist=True)
     ref = oracle.moff_image(blocks[0], gains, pos, taps, 64, 2)
     assert n == 30 and oracle.max_norm_err(img, ref).max() <= TOL32
+
+
+def squeezed(seed, A, N, K, P, rows):
+    """Positions over the whole grid, and the same antennas on `rows` grid rows, with kernels for each."""
+    rng = np.random.default_rng(seed)
+    pos = rng.uniform(0, N, size=(2, A, 2))
+    pos[1, :, 1] = N // 3 + rng.integers(0, rows, size=A)
+    return pos, c64(rng.normal(size=(2, A, P, K, K)) + 1j * rng.normal(size=(2, A, P, K, K)))
+
+
+@pytest.mark.parametrize("groups", [[1, 1, 1], [0, 1, 1]])
+def test_denser_sets_after_creation(groups):
+    """Replacing the positions by denser ones needs more shared memory per stripe than the plan was created with: the
+    persistent launch takes it from the sets in force, and gives the direct launches' image."""
+    N, P, K, A, C, T = 128, 1, 5, 2000, 3, 33
+    pos, taps = squeezed(970, A, N, K, P, 20)
+    rng = np.random.default_rng(971)
+    codes = synth.pack_4bit(rng.integers(-7, 8, size=(T, C, A, P)), rng.integers(-7, 8, size=(T, C, A, P)))
+    sets = (pos[1:], taps[1:], None) if min(groups) == 1 else (pos, taps, groups)
+    out = []
+    for persist in (False, True):
+        with moff.Plan(pos[0], taps[0], N, C, P, persist=persist) as pl:
+            before = pl.tuning()["time_batch"]
+            pl.set_channel_groups(*sets)
+            pl.set_timing(True)
+            pl.submit(codes)
+            assert pl.timing(8)[1] == (1 if persist else 0)
+            out.append(pl.read_image()[0])
+            assert not persist or before == 4
+    assert np.array_equal(out[0], out[1])
+    err = oracle.max_norm_err(out[1], oracle.moff_image_sets(codes, np.ones((C, A, P), complex), pos, taps, groups, N, P))
+    assert err.max() <= TOL32
+
+
+def test_sets_that_no_persistent_shape_fits_run_the_direct_launches():
+    """A set that fits one sample per pass but not four: the persistent kernel is built for four, so the plan's blocks
+    take the direct launches."""
+    N, P, K, A, C, T = 256, 2, 9, 2600, 2, 10
+    pos, taps = squeezed(980, A, N, K, P, 1)
+    rng = np.random.default_rng(981)
+    codes = synth.pack_4bit(rng.integers(-7, 8, size=(T, C, A, P)), rng.integers(-7, 8, size=(T, C, A, P)))
+    out = []
+    for persist in (False, True):
+        with moff.Plan(pos[0], taps[0], N, C, P, persist=persist) as pl:
+            pl.set_channel_groups(pos, taps, [0, 1])
+            assert pl.tuning()["time_batch"] == 1
+            pl.set_timing(True)
+            pl.submit(codes)
+            assert pl.timing(8)[1] == 0 and pl.timing(1)[1] > 0
+            out.append(pl.read_image()[0])
+    assert np.array_equal(out[0], out[1])
+    err = oracle.max_norm_err(out[1], oracle.moff_image_sets(codes, np.ones((C, A, P), complex), pos, taps, [0, 1], N, P))
+    assert err.max() <= TOL32
