@@ -1032,7 +1032,7 @@ moff_status fail_msg(moff_status s, const char *msg) { return fail(s, "%s", msg)
 // lists (host only).  The stripe height is the largest power of two <= 16
 // whose lists fit the gridding kernel's shared-memory budget.
 moff_status build_bins(int A, int K, int N, int P, bool jones, const double *pos, const float *taps, Bins *b,
-                       const GridChoice *force, bool dft, bool narrow) {
+                       const GridChoice *force, bool dft, GridRule rule) {
     const int h = K / 2;
     std::vector<int> ax(A), ay(A);
     for (int a = 0; a < A; ++a) {
@@ -1117,7 +1117,7 @@ moff_status build_bins(int A, int K, int N, int P, bool jones, const double *pos
     // Entries are read through L2 by default (more CTAs per SM measured faster
     // than shared-memory staging); MOFF_GRID_STAGE=1 prefers staging.
     const char *stage_env = getenv("MOFF_GRID_STAGE");
-    const bool prefer_staged = !dft && stage_env && atoi(stage_env) != 0;
+    const bool prefer_staged = !dft && rule != GridRule::persist && stage_env && atoi(stage_env) != 0;
     const Cand *pick = nullptr;
     bool staged = false;
     // The rule's first choice: cell pairs on stripes of twice the rows with 8 or 4 samples per pass, on one CTA per SM
@@ -1130,7 +1130,10 @@ moff_status build_bins(int A, int K, int N, int P, bool jones, const double *pos
     //              rho 2.9  0.69 / -    / 0.72              rho 12   1.57 / 1.77 / 1.82
     //              rho 6.0  does not fit / 2.56 / 2.87 (one sample, which the rule took before: 3.06)
     // Each cell's sum keeps its order in every shape.
-    if (!force && !dft && !narrow && !wide_env && pairs && !prefer_staged) {
+    // A persistent launch (GridRule::persist) has 4 samples per pass; there the wide stripes pay where the rule takes them (us
+    // per block, wide / narrow: 128 grid 3977 / 4900, 256 grid 1650 / 2042 with one pol and 3924 / 5147 with two, 512 grid
+    // 2761 / 3047 with two) but for one pol on the 512 grid (1450 / 1229).
+    if (!force && !dft && rule != GridRule::narrow && !wide_env && pairs && !prefer_staged) {
         long long total = 0;
         int reached = 0;
         for (int y = 0; y < N; ++y) {
@@ -1145,6 +1148,7 @@ moff_status build_bins(int A, int K, int N, int P, bool jones, const double *pos
         if (N <= 64) wants = {8};
         else if (N <= 256) wants = rho >= 3.3 ? std::vector<int>{8, 4} : std::vector<int>{4};
         else if (rho >= 2.3) wants = {8, 4};
+        if (rule == GridRule::persist && !wants.empty()) wants = N == 512 && P == 1 ? std::vector<int>{} : std::vector<int>{4};
         for (int want : wants) {
             const std::vector<Cand> w = shapes(2 * F, {want});
             if (w.empty() || w[0].sm_plain > big) continue;
@@ -1155,7 +1159,7 @@ moff_status build_bins(int A, int K, int N, int P, bool jones, const double *pos
             break;
         }
     }
-    if (!pick) cands = shapes(F, {8, 4, 2, 1});
+    if (!pick) cands = rule == GridRule::persist && !force ? shapes(F, {4}) : shapes(F, {8, 4, 2, 1});
     if (force) {
         for (const Cand &cd : cands)
             if (cd.tb == force->tb) {
@@ -1558,7 +1562,8 @@ namespace {
 moff_status build_bin_sets(const moff_plan *pl, int n_sets, const double *pos, const float *taps,
                            const GridChoice *force, Bins *out) {
     const int A = pl->A, K = pl->K, N = pl->N, P = pl->P;
-    if (n_sets == 1) return build_bins(A, K, N, P, pl->jones, pos, taps, out, force, pl->dft);
+    if (n_sets == 1)
+        return build_bins(A, K, N, P, pl->jones, pos, taps, out, force, pl->dft, pl->persist ? GridRule::persist : GridRule::any);
     const size_t pos_set = (size_t)A * 2;
     const size_t tap_set = (size_t)A * P * (pl->jones ? 2 : 1) * K * K * 2;
     std::vector<GridChoice> cands;
@@ -2395,14 +2400,6 @@ moff_status moff_plan_create(moff_plan **out, int n_ant, const double *pos, int 
             if ((s = tune_grid(pl, pos, taps, &tuned)) != MOFF_OK) return bail(s);
         }
         if ((s = bin_plan(pl, pos, taps, pl->tune_source ? &tuned : nullptr)) != MOFF_OK) return bail(s);
-        if (pl->persist && (pl->tb != 4 || pl->staged)) {
-            GridChoice ch{4, false, pl->pairs, pl->wide, pl->quads};
-            if ((s = bin_plan(pl, pos, taps, &ch)) != MOFF_OK && ch.wide) {   // half the rows need less shared memory
-                ch.wide = false;
-                s = bin_plan(pl, pos, taps, &ch);
-            }
-            if (s != MOFF_OK) return bail(s);
-        }
     }
     if (pl->dft) {   // the column kernel's width: the default, or timed (needs the plan's reached-row mask)
         pl->cols_w = cols_dft_width();

@@ -332,10 +332,13 @@ struct GridChoice {
     bool wide = false;    // twice grid_fft_rows(N) rows per pass (more gather work per barrier)
     bool quads = false;   // each lane sums a 2 x 2 block of cells (pairs ignored; entries through L2)
 };
+// Which shapes the built-in rule considers: any, those with the smaller lists (narrow stripes), or what the persistent
+// kernel is built for (4 samples per pass, entries through L2).
+enum class GridRule { any, narrow, persist };
 // force = nullptr: the built-in rule; else exactly that shape (MOFF_EINVAL if infeasible).
 // dft: shapes of the gridding kernel with the tensor-core row transform (k_grid_rows_dft).
 moff_status build_bins(int A, int K, int N, int P, bool jones, const double *pos, const float *taps, Bins *b,
-                       const GridChoice *force = nullptr, bool dft = false, bool narrow = false);
+                       const GridChoice *force = nullptr, bool dft = false, GridRule rule = GridRule::any);
 std::vector<float2> pass_twiddles_for(int n);   // pass-twiddle table of the n-point transform (FP64-built)
 
 // Row spectra of the kernel rows for the tensor-core path (host side).

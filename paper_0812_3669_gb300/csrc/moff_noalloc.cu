@@ -99,7 +99,7 @@ extern "C" moff_status moff_image_noalloc(int n_ant, const double *pos, int ksiz
     }
 
     Bins b;
-    moff_status s = build_bins(n_ant, ksize, N, P, jones, pos, taps, &b, nullptr, false, true);   // the smaller lists
+    moff_status s = build_bins(n_ant, ksize, N, P, jones, pos, taps, &b, nullptr, false, GridRule::narrow);
     if (s != MOFF_OK) return s;
     const std::vector<float2> tw = pass_twiddles_for(N);
 

@@ -190,3 +190,21 @@ def test_sets_that_no_persistent_shape_fits_run_the_direct_launches():
     assert np.array_equal(out[0], out[1])
     err = oracle.max_norm_err(out[1], oracle.moff_image_sets(codes, np.ones((C, A, P), complex), pos, taps, [0, 1], N, P))
     assert err.max() <= TOL32
+
+
+@pytest.mark.parametrize("N,P,A,wide", [(64, 1, 300, 1), (128, 2, 300, 1), (512, 1, 6000, 0), (512, 2, 6000, 1)])
+def test_built_in_shape(N, P, A, wide):
+    """The rule picks among the persistent kernel's shapes (4 samples per pass) and takes wide stripes where they pay: not
+    for one pol on the 512 grid.  The image is the direct launches'."""
+    K, C, T = 7, 1, 9
+    pos, taps, gains, blocks = case(990, A, N, K, P, C, [T])
+    if N == 512:
+        pos = 100 + (pos - pos.min()) * 0.45        # dense enough for wide stripes in a direct plan
+    with moff.Plan(pos, taps, N, C, P) as pl:
+        assert pl.tuning()["wide_rows"] == 1
+    with moff.Plan(pos, taps, N, C, P, persist=True) as pl:
+        t = pl.tuning()
+        assert (t["time_batch"], t["wide_rows"], t["staged"]) == (4, wide, 0)
+    d, _, _ = run(pos, taps, gains, N, C, P, blocks)
+    p, _, _ = run(pos, taps, gains, N, C, P, blocks, persist=True)
+    assert np.array_equal(d, p)
