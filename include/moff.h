@@ -161,8 +161,10 @@ moff_status moff_set_gains(moff_plan *plan, const float *gains, int on_device);
  *   chan_group  host int [C]: the set of each channel (may be NULL when
  *               n_groups = 1, which replaces the creation-time set)
  * All copied.  Channels of one set are imaged exactly as a plan created with
- * that set.  The gridding shape stays the plan's where every set fits it, else
- * the first of the built-in rule's shapes that all sets fit.  Waits for the
+ * that set.  The gridding shape stays the plan's where every set fits it.
+ * Else one set takes the shape that the built-in rule picks for it, and several
+ * the first that all fit of cell pairs, then single cells, on stripes of the
+ * smaller height with 4, 8, 2 and 1 samples per pass.  Waits for the
  * plan's work in flight; applies to blocks submitted afterwards (the running
  * integration is kept: reset first to start a new one).  Calibrator beams and
  * autocorrelation patches follow the new sets.  FP32 path only.

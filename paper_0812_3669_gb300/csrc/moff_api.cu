@@ -2564,8 +2564,16 @@ moff_status moff_set_channel_groups(moff_plan *pl, int n_groups, const double *p
                 return fail(MOFF_EINVAL, "chan_group[%d] = %d outside [0, %d)", c, chan_group[c], n_groups);
     if ((s = sync_plan(pl, -1)) != MOFF_OK) return s;
     const GridChoice cur{pl->tb, pl->staged, pl->pairs, pl->wide, pl->quads};
+    const bool keep = !pl->persist || (pl->tb == 4 && !pl->staged);
     Bins b;
-    if ((s = build_bin_sets(pl, n_groups, pos, taps, &cur, &b)) != MOFF_OK) return s;
+    // The plan's shape where the sets fit it.  One set that does not takes the built-in rule's (for a persistent plan the
+    // rule's with 4 samples per pass, else any: the direct launches); several take the first of build_bin_sets' list.
+    s = build_bin_sets(pl, n_groups, pos, taps, keep ? &cur : nullptr, &b);
+    if (n_groups == 1 && s == MOFF_EINVAL && keep) s = build_bin_sets(pl, 1, pos, taps, nullptr, &(b = Bins{}));
+    if (n_groups == 1 && s == MOFF_EINVAL && pl->persist)
+        s = build_bins(pl->A, pl->K, pl->N, pl->P, pl->jones, pos, taps, &(b = Bins{}));
+    if (s != MOFF_OK) return s;
+    g_err.clear();
     int *d_grp = nullptr;
     if (n_groups > 1) {
         if ((s = palloc(pl, &d_grp, (size_t)pl->C * 4)) != MOFF_OK) return s;

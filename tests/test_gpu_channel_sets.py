@@ -204,3 +204,37 @@ def test_edge_padding_samples_the_same_image():
     err = oracle.max_norm_err(big[:, :, ::2, ::2], small)
     assert err.max() <= 2 * TOL32
     assert oracle.max_norm_err(big, oracle.moff_image(codes, gains, pos, taps, 2 * N, P)).max() <= TOL32
+
+
+@pytest.mark.parametrize("side,K,jones,persist,scale", [(128, 7, False, False, 0.7), (128, 7, False, False, 0.5),
+                                                      (180, 7, False, False, 0.98), (100, 9, True, False, 0.7),
+                                                      (128, 7, False, True, 0.5)])
+def test_one_denser_set_takes_the_rules_shape(side, K, jones, persist, scale):
+    """The filled lattices' plans use nearly all shared memory of a stripe on the 512 grid.  The same array at another
+    frequency lies denser and does not fit that shape: it is imaged in the shape of a plan created with it."""
+    N, P, C, T = 512, 2, 1, 5
+    rng = np.random.default_rng(880 + side)
+    base = synth.positions_lattice(rng, side, side, 1.0, 0.05, (N / 2 - side, N / 2 - side))
+    A = base.shape[0]
+    pos = np.stack([base, N / 2 + scale * (base - N / 2)])
+    shape = (A, 2, 2, K, K) if jones else (A, P, K, K)
+    taps = (rng.normal(size=shape) + 1j * rng.normal(size=shape)).astype(np.complex64)
+    codes = synth.pack_4bit(rng.integers(-7, 8, size=(T, C, A, P)), rng.integers(-7, 8, size=(T, C, A, P)))
+    with moff.Plan(pos[0], taps, N, C, P, jones=jones, persist=persist) as pl:
+        first = pl.tuning()
+        pl.set_channel_groups(pos[1:], taps[None])
+        second = pl.tuning()
+        pl.submit(codes)
+        img, _ = pl.read_image(reset=True)
+        pl.set_channel_groups(pos[:1], taps[None])
+        pl.submit(codes)
+        back, _ = pl.read_image()
+    assert persist or first != second
+    ref = []
+    for k in (1, 0):
+        with moff.Plan(pos[k], taps, N, C, P, jones=jones) as pl:
+            pl.submit(codes)
+            ref.append(pl.read_image()[0])
+    assert np.array_equal(img, ref[0]) and np.array_equal(back, ref[1])
+    want = oracle.moff_image(codes, np.ones((C, A, P), complex), pos[1], taps.astype(complex), N, P, jones=jones)
+    assert oracle.max_norm_err(img, want).max() <= TOL32
