@@ -18,6 +18,7 @@
 // read consecutive entries.
 #pragma once
 #include <cuda_runtime.h>
+#include <limits.h>
 #include <stdint.h>
 
 namespace moff {
@@ -196,20 +197,26 @@ __device__ __forceinline__ int pad_store(int j, int r) {
     }
 }
 
-// Exponent of a power of two.
-__device__ __forceinline__ int pow2_exp(double s) { return (int)((__double2hiint(s) >> 20) & 2047) - 1023; }
+// Exponent of a power of two for red_scaled; kNoExp for a scale so small, large, zero, infinite or NaN that an FP32 value
+// times it could leave FP64's normal range.
+constexpr int kNoExp = INT_MIN, kMaxExp = 895;
+__device__ __forceinline__ int pow2_exp(double s) {
+    const int e = (int)((__double2hiint(s) >> 20) & 2047) - 1023;
+    return e < -kMaxExp || e > kMaxExp ? kNoExp : e;
+}
 
 // *a += s v, with s a power of two, without the FP64 pipe (two operations a cycle and SM): the product's bits are put
 // together from v's and the addition is left to L2 (a reduction without return; one owner per element, so the sum
-// is that of a load, add and store).  Values whose product is subnormal, infinite or NaN take the plain path.
+// is that of a load, add and store).  v subnormal, infinite or NaN, and scales without an exponent (pow2_exp), take the
+// plain path: a normal v has an exponent field of 1 to 254, so the product's, e + 896 + scale_exp, lies in 2 to 2045.
 __device__ __forceinline__ void red_scaled(double *a, float v, int scale_exp, double s) {
     const uint32_t u = __float_as_uint(v);
     const int e = (int)((u >> 23) & 255u);
     double d;
-    if (e != 0 && e != 255) {
+    if (e != 0 && e != 255 && scale_exp != kNoExp) {
         const uint32_t m = u & 0x7FFFFFu;
         d = __hiloint2double((int)((u & 0x80000000u) | ((uint32_t)(e + 896 + scale_exp) << 20) | (m >> 3)), (int)(m << 29));
-    } else if ((u << 1) == 0u) {
+    } else if ((u << 1) == 0u && scale_exp != kNoExp) {
         return;                                                  // adding zero
     } else {
         d = (double)v * s;

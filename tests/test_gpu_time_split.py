@@ -85,3 +85,29 @@ def test_wide_and_narrow_stripes_agree(monkeypatch, A, N, P, K):
     narrow, b = image()
     assert narrow["wide_rows"] == 0 and wide["wide_rows"] == 1
     np.testing.assert_array_equal(a, b)
+
+
+@pytest.mark.parametrize("N,P", [(64, 1), (128, 2), (256, 2)])
+@pytest.mark.parametrize("large", [False, True])
+def test_scales_outside_fp32(N, P, large):
+    """Gains and kernels so small (or large) together that the row-spectrum route's FP32 scale of a channel is 0 (or
+    infinite): a fold that puts the product's bits together must not wrap its exponent.  The image is 0 (the true one lies
+    below FP32's range), or nowhere finite."""
+    A, C, T = 12, 2, 40
+    pos, taps, codes, gains = case(N + 3, A, N, P, C, T)
+    gains /= np.abs(gains)
+    if large:
+        gains, taps = gains * 1e30, taps * 1e15
+    else:   # one antenna without signal sets the channel's scale, so that the others' sums are far below 1
+        codes[:, :, 0] = 0
+        gains, taps = gains * 2e-38, taps * 1e-12
+        gains[:, 0] *= 5e5
+    with moff.Plan(pos, taps.astype(np.complex64), N, C, P, fp16tc=True) as pl:
+        assert pl.route() == "fp16_rowspec"
+        pl.set_gains(gains.astype(np.complex64))
+        pl.submit(codes)
+        img, _ = pl.read_image()
+    if large:
+        assert not np.isfinite(img).any()
+    else:
+        assert np.array_equal(img, np.zeros_like(img))
