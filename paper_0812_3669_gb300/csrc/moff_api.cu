@@ -434,21 +434,20 @@ void destroy_plan(moff_plan *pl) {
     delete pl;
 }
 
-// Without a limit the runtime waits; with one, polling without pause for the first 0.2 ms (a pause of 50 us takes
-// about 100, which a short block's two waits felt: 200 of the 362 us of a tiny array's block), then with pauses.
+// Polls without pause for the first 0.2 ms and then lets any other thread that is ready have the core between two polls; a
+// wait longer than 20 ms goes on with pauses, so it does not occupy a core.  A pause of 50 us ends about 100 us later, and
+// even finer ones (timer slack of 1 ns) or the event's interrupt (cudaEventBlockingSync) end a wait 35 to 75 us late: half
+// of a tiny array's block, 1 to 6 % of blocks of 2 to 4 ms, and 0.5 % of the shortest wait that sees them here.
 moff_status wait_event(cudaEvent_t ev, int timeout_ms) {
-    if (timeout_ms < 0) {
-        const cudaError_t e = cudaEventSynchronize(ev);
-        return e == cudaSuccess ? MOFF_OK : fail(MOFF_ECUDA, "waiting for the GPU: %s", cudaGetErrorString(e));
-    }
     const auto t0 = std::chrono::steady_clock::now();
     for (;;) {
         cudaError_t e = cudaEventQuery(ev);
         if (e == cudaSuccess) return MOFF_OK;
         if (e != cudaErrorNotReady) return fail(MOFF_ECUDA, "waiting for the GPU: %s", cudaGetErrorString(e));
         const auto us = std::chrono::duration_cast<std::chrono::microseconds>(std::chrono::steady_clock::now() - t0).count();
-        if (us >= 1000LL * timeout_ms) return fail(MOFF_ETIMEDOUT, "GPU work not finished after %d ms", timeout_ms);
-        if (us > 200) std::this_thread::sleep_for(std::chrono::microseconds(50));
+        if (timeout_ms >= 0 && us >= 1000LL * timeout_ms) return fail(MOFF_ETIMEDOUT, "GPU work not finished after %d ms", timeout_ms);
+        if (us > 20000) std::this_thread::sleep_for(std::chrono::microseconds(50));
+        else if (us > 200) std::this_thread::yield();
     }
 }
 
