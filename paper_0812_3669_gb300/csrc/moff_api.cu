@@ -1839,7 +1839,7 @@ std::string tune_key(const moff_plan *pl, const double *pos, const float *taps) 
     char buf[128];
     // the prefix changes with the gridding kernels, so picks timed on an older build are not reused
     snprintf(buf, sizeof buf, "%s-A%d-K%d-N%d-P%d-J%d-T%d-C%d-sm%d-%016llx",
-             pl->dft ? "gdft1" : (pl->persist ? "gpst1" : "grid6"), pl->A, pl->K,
+             pl->dft ? "gdft2" : (pl->persist ? "gpst2" : "grid7"), pl->A, pl->K,
              pl->N, pl->P, (int)pl->jones, pl->Tb, std::min(pl->Cb, pl->C), prop.multiProcessorCount,
              (unsigned long long)h);
     return buf;

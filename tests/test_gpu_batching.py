@@ -156,3 +156,28 @@ def test_tuning_cache_file_is_shared_between_processes(tmp_path):
     assert outs[0][1] == "1" and outs[1][1] == "2"
     assert outs[0][2:] == outs[1][2:]
     assert open(path).read().count("\n") == 1
+
+
+@pytest.mark.parametrize("flags,earlier", [("", "grid6"), (", persist=True", "gpst1")])
+def test_picks_of_earlier_gridding_kernels_are_not_reused(tmp_path, flags, earlier):
+    """The pick's key names the kernels that it was timed on: a file written before the voltages of a stripe were laid out
+    by antenna and the short launches' samples were split is measured anew."""
+    path = str(tmp_path / "tune.txt")
+    code = ("import sys; sys.path.insert(0, %r)\n"
+            "import numpy as np, paper_0812_3669_gb300 as moff\n"
+            "rng = np.random.default_rng(9)\n"
+            "pos = rng.uniform(10, 50, size=(150, 2)); taps = np.ones((150, 1, 5, 5), complex)\n"
+            "pl = moff.Plan(pos, taps, 64, 2, 1, autotune=True%s)\n"
+            "print('SRC', pl.tuning()['source'])\n" % (ROOT, flags))
+    env = dict(os.environ, MOFF_TUNE_CACHE=path)
+
+    def source():
+        r = subprocess.run([sys.executable, "-c", code], env=env, capture_output=True, text=True, timeout=300)
+        assert r.returncode == 0, r.stderr[-2000:]
+        return int([ln for ln in r.stdout.splitlines() if ln.startswith("SRC")][0].split()[1])
+
+    assert source() == 1
+    line = open(path).read()
+    with open(path, "w") as f:
+        f.write(earlier + line[line.index("-"):])
+    assert source() == 1
