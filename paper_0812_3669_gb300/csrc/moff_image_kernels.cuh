@@ -1287,9 +1287,11 @@ cudaError_t launch_persist_t(const PersistArgs &pa, size_t smem, int sms, cudaSt
 // through L2; CPL and wide stripes as the plan chose them.
 template <int N, int P>
 cudaError_t launch_persist_p(int cpl, bool wide, const PersistArgs &pa, size_t smem, int sms, cudaStream_t st) {
-    if (cpl == 4) {
-        if constexpr (GridShape<N, P, 4, true>::ROWS % 2 == 0 && GridShape<N, P, 4, false>::ROWS % 2 == 0)
-            return wide ? launch_persist_t<N, P, 4, true>(pa, smem, sms, st) : launch_persist_t<N, P, 4, false>(pa, smem, sms, st);
+    if (cpl == 4) {   // 2 x 2 blocks need an even stripe height
+        if constexpr (GridShape<N, P, 4, true>::ROWS % 2 == 0)
+            if (wide) return launch_persist_t<N, P, 4, true>(pa, smem, sms, st);
+        if constexpr (GridShape<N, P, 4, false>::ROWS % 2 == 0)
+            if (!wide) return launch_persist_t<N, P, 4, false>(pa, smem, sms, st);
         return cudaErrorInvalidValue;
     }
     if (cpl == 2)

@@ -208,3 +208,22 @@ def test_built_in_shape(N, P, A, wide):
     d, _, _ = run(pos, taps, gains, N, C, P, blocks)
     p, _, _ = run(pos, taps, gains, N, C, P, blocks, persist=True)
     assert np.array_equal(d, p)
+
+
+@pytest.mark.parametrize("N", [256, 512])
+def test_block_lanes_on_wide_stripes(monkeypatch, N):
+    """2 x 2 blocks per lane with two pols on the large grids: only the wide stripes have two rows (the autotuner may
+    pick them)."""
+    monkeypatch.setenv("MOFF_GRID_QUADS", "1")
+    monkeypatch.setenv("MOFF_GRID_WIDE", "1")
+    pos, taps, gains, blocks = case(995, 150, N, 5, 2, 2, [21])
+    out = []
+    for persist in (False, True):
+        with moff.Plan(pos, taps, N, 2, 2, persist=persist) as pl:
+            t = pl.tuning()
+            assert (t["cells_per_lane"], t["wide_rows"], t["time_batch"]) == (4, 1, 4)
+            pl.set_gains(gains)
+            pl.submit(blocks[0])
+            out.append(pl.read_image()[0])
+    assert np.array_equal(out[0], out[1])
+    assert oracle.max_norm_err(out[1], oracle.moff_image(blocks[0], gains, pos, taps, N, 2)).max() <= TOL32
