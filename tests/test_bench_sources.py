@@ -100,3 +100,32 @@ def test_tcgrid_work_model():
     assert w["grid_rows"]["tensor"] == 8 * 9
     assert w["row_transform"]["tensor"] == 6 * fac and w["cols_integrate"]["tensor"] == 256 * fac
     assert w["row_transform"]["bytes"] == 3 * 64 * 4 + 6 * 256 * 4
+
+
+def test_the_line_on_stdout_stays_short():
+    """One line with every key a reader of the benchmark needs and the legs' rates; long details (here megabytes of
+    them) do not enter it."""
+    import argparse
+
+    pad = {"x" * 10: "y" * 100000}
+    leg = {"value": 123456.789012345678, **pad}
+    sat = {"throughput": 123456.789012345678, **pad}
+    head = {"value": 896037.214680385, "ms_per_step": 585.1185546875, "channels": 4096, "samples_per_step": 128,
+            "route": "fp16_tcgrid", "gpu_launches": 123456, "plan_create_s": 1.42, "kernels": pad, **pad,
+            "clocks": {"sm_mhz": 2070.0, "sm_max_mhz": 2070.0, "power_w_max": 1322.0, "reasons": ["sw_power_cap"], **pad},
+            "e2e": {"value": 824295.257489882, "unit": bench.UNIT, "h2d_bytes_per_step": 34359738368,
+                    "d2h_bytes_per_step": 5726623061, **pad}}
+    roof = {"bound": "hbm", "kernel": "cols_dft", "achieved": 2893.733091120192, "peak": 6788.3, "unit": "GB/s",
+            "frac": 0.42628244054036973, "traffic_over_algorithmic": 1.0123456789, **pad}
+    legs = {"fp32_same_workload": leg, "precision_filled_aperture": {"fp16tc": leg, "fp32": leg}, "dualpol_fstage": leg,
+            "serving": {"saturation": sat, "fp16tc_stream": {"saturation": sat}}, "batching": pad}
+    cpu = {"value": 46.2123456789, "unit": bench.UNIT, "cores": 1, "kind": "oracle", "nproc": 16, "all_core": pad}
+    args = argparse.Namespace(steps=20, warmup=5)
+    d = bench.contract_line(args, 8, bench.DENSE["widefield"], head, roof, cpu, legs)
+    assert len(json.dumps(d)) < 1500
+    for k in ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+              "vs_baseline", "dtype", "data", "config", "e2e", "gpu_launches", "clocks", "roofline", "cpu_baseline"):
+        assert k in d, k
+    assert d["value"] == head["value"] and d["legs"]["serving_fp16"] == 123500.0
+    none = bench.contract_line(args, 1, bench.DENSE["widefield"], head, roof, None, dict.fromkeys(legs))
+    assert none["cpu_baseline"] is None and none["legs"] == {}
