@@ -298,7 +298,7 @@ struct moff_plan {
     // (power of two: the gridded field times sy[c] * dft_s_t stays within FP16), and the
     // gridding kernel's shared memory for a grid-only (FP32 transform) launch
     bool dft = false;
-    unsigned char *d_dft_tab = nullptr;     // rows (gridding kernel, row transform)
+    unsigned char *d_dft_tab = nullptr;     // rows inside the gridding kernel (the gather)
     unsigned char *d_dft_tab_r8 = nullptr;  // tables of the row transform (tensor-core gridding)
     unsigned char *d_dft_tab_c = nullptr;   // the column kernel's image
     int cols_w = 8;                         // columns per CTA of k_cols_dft
@@ -2344,19 +2344,18 @@ moff_status moff_plan_create(moff_plan **out, int n_ant, const double *pos, int 
     if (pl->dft) {
         // factored-DFT tables, and the kernel scale: every cell's sum of |tap| over its contributions
         // (all output pols) times dft_s_t is at most 1, so |G| sy[c] dft_s_t <= 2^14
-        std::vector<unsigned char> tab = build_dft_table(grid_n), tabc = build_dft_table(grid_n, true);
-        if ((s = palloc(pl, &pl->d_dft_tab, tab.size())) != MOFF_OK) return bail(s);
-        if ((s = palloc(pl, &pl->d_dft_tab_c, tabc.size())) != MOFF_OK) return bail(s);
-        if (cudaMemcpy(pl->d_dft_tab, tab.data(), tab.size(), cudaMemcpyHostToDevice) != cudaSuccess ||
-            cudaMemcpy(pl->d_dft_tab_c, tabc.data(), tabc.size(), cudaMemcpyHostToDevice) != cudaSuccess)
-            return bail(fail(MOFF_ECUDA, "tensor-core DFT table upload failed"));
+        auto table = [&](unsigned char **dst, const std::vector<unsigned char> &v) -> moff_status {
+            moff_status st = palloc(pl, dst, v.size());
+            if (st == MOFF_OK && cudaMemcpy(*dst, v.data(), v.size(), cudaMemcpyHostToDevice) != cudaSuccess)
+                st = fail(MOFF_ECUDA, "tensor-core DFT table upload failed");
+            return st;
+        };
+        if ((s = table(&pl->d_dft_tab_c, build_dft_table(grid_n, true))) != MOFF_OK) return bail(s);
+        // rows: the row transform's own table, or the gather's
+        if ((s = pl->gtc ? table(&pl->d_dft_tab_r8, build_rows8_table(grid_n))
+                         : table(&pl->d_dft_tab, build_dft_table(grid_n))) != MOFF_OK)
+            return bail(s);
         if (!pl->gtc) pl->dft_s_t = dft_kernel_scale(n_ant, ksize, grid_n, n_pol, pl->jones, pos, taps);
-        if (pl->gtc) {
-            std::vector<unsigned char> t8 = build_rows8_table(grid_n);
-            if ((s = palloc(pl, &pl->d_dft_tab_r8, t8.size())) != MOFF_OK) return bail(s);
-            if (cudaMemcpy(pl->d_dft_tab_r8, t8.data(), t8.size(), cudaMemcpyHostToDevice) != cudaSuccess)
-                return bail(fail(MOFF_ECUDA, "row-transform table upload failed"));
-        }
         if ((s = palloc(pl, &pl->d_sy, (size_t)n_chan * 4)) != MOFF_OK) return bail(s);
         if (pl->gtc) {
             pl->gt_tiles = (int)gtab.tile_cell.size();

@@ -66,15 +66,15 @@ struct ColDftShape {
     // warp groups per stage-2 tile: with one tile (W = 8) the two groups split the d range
     static constexpr int DSPLIT = 2 / T2;
     static constexpr int ND = N2 / DSPLIT;             // d values per thread
-    static constexpr int MINB = W == 8 ? 2 : 1;        // CTAs per SM
     static constexpr size_t SMEM = 1024 + (size_t)P * A2P + 2 * (size_t)P * A1P + S::TAB_BYTES + 32;
-    static_assert(T2 >= 1 && T2 <= 2 && T1 >= 1 && TC_ * MINB <= 512 && NPIECE % kBlock == 0 && ITER <= 32 &&
-                      ND % 8 == 0 && (2 * H * N) % kBlock == 0 && ROWS_K % N2 == 0 && SMEM * MINB <= 225 * 1024,
+    static_assert(T2 >= 1 && T2 <= 2 && T1 >= 1 && TC_ <= 512 && NPIECE % kBlock == 0 && ITER <= 32 && ND % 8 == 0 &&
+                      (2 * H * N) % kBlock == 0 && ROWS_K % N2 == 0 && SMEM <= 225 * 1024,
                   "column-kernel shape");
 };
 
-template <int N, int P, int W>
-__global__ void __launch_bounds__(kBlock, ColDftShape<N, P, W>::MINB) k_cols_dft(const ColDftArgs a) {
+template <int P>
+__global__ void __launch_bounds__(kBlock, 1) k_cols_dft(const ColDftArgs a) {
+    constexpr int N = 512, W = 16;
     using S = DftShape<N>;
     using CS = ColDftShape<N, P, W>;
     constexpr int N2 = S::N2, K2 = S::K2, C2 = S::C2, H = CS::H, ND = CS::ND;
@@ -115,7 +115,7 @@ __global__ void __launch_bounds__(kBlock, ColDftShape<N, P, W>::MINB) k_cols_dft
     const int src_t = field_offset(N, r0, ri0, blockIdx.x * H + h0);
     auto piece_dst = [&](int k) -> uint32_t {      // k compile-time after unrolling
         const int PK = (k * kBlock) / (2 * H * N), RYK = ((k * kBlock) % (2 * H * N)) / (2 * H), AK = RYK / N2;
-        // 2 AK is a multiple of 8 but for 16 columns at N = 512, where it flips bit 2 of the swizzle (kt < 4 there)
+        // 2 AK is a multiple of 4: its bit 2 flips that of the swizzle (kt < 4)
         return (uint32_t)(PK * CS::A1P + 2 * AK * 128) + (dst_t ^ (uint32_t)(((2 * AK) & 4) << 4));
     };
     auto piece_src = [&](int k) -> long long {
@@ -213,11 +213,9 @@ __global__ void __launch_bounds__(kBlock, ColDftShape<N, P, W>::MINB) k_cols_dft
             }
         }
     };
-    // Square and sum: warp group g = warp / 4 takes stage-2 tile j2 (two tiles) or half the d range
-    // (one tile); lane quarter q's row l = 32 q + lane of the tile is m2 = 128 j2 + l = 8 W c_hi + 8 x
-    // + c_lo: pixels (ky = 8 c_hi + c_lo + 16 d, kx = x0 + x) for the group's d.
-    const int g = warp >> 2;
-    const int j2 = CS::T2 == 2 ? g : 0, dbase = CS::T2 == 2 ? 0 : g * ND;
+    // Square and sum: warp group j2 = warp / 4 takes stage-2 tile j2; lane quarter q's row l = 32 q + lane of the tile is
+    // m2 = 128 j2 + l = 8 W c_hi + 8 x + c_lo: pixels (ky = 8 c_hi + c_lo + 16 d, kx = x0 + x) for every d.
+    const int j2 = warp >> 2;
     // sums of d and d + 1 side by side (packed FP32)
     float2 acc[NPROD][ND / 2];
 #pragma unroll
@@ -227,7 +225,7 @@ __global__ void __launch_bounds__(kBlock, ColDftShape<N, P, W>::MINB) k_cols_dft
     auto epi2 = [&]() {
 #pragma unroll
         for (int db = 0; db < ND / 8; ++db) {         // 8 d per TMEM load of each pol: real parts, then imaginary
-            const uint32_t col = (uint32_t)(CS::D1 + j2 * C2 + 2 * dbase + 16 * db);
+            const uint32_t col = (uint32_t)(CS::D1 + j2 * C2 + 16 * db);
             float ex[16];
             tc::tmem_ld16(tbase + ((uint32_t)(32 * q) << 16) + col, ex);
             if constexpr (P == 1) {
@@ -299,7 +297,7 @@ __global__ void __launch_bounds__(kBlock, ColDftShape<N, P, W>::MINB) k_cols_dft
             double *dst = a.acc + ((long long)c * NPROD + pq) * N * N + x0 + x;
 #pragma unroll
             for (int d = 0; d < ND; ++d)
-                dst[(long long)(cy + 16 * (dbase + d)) * N] += (double)((d & 1) ? acc[pq][d >> 1].y : acc[pq][d >> 1].x) * sc2;
+                dst[(long long)(cy + 16 * d) * N] += (double)((d & 1) ? acc[pq][d >> 1].y : acc[pq][d >> 1].x) * sc2;
         }
     } else if (tid == 0) {
         atomicExch(a.err, tc::kErrWaitTimeout);
@@ -648,16 +646,16 @@ cudaError_t launch_cols_pipe_t(const ColDftArgs &a, cudaStream_t st) {
     return cudaGetLastError();
 }
 
-template <int N, int P, int W>
+template <int P>
 cudaError_t launch_cols_dft_t(const ColDftArgs &a, cudaStream_t st) {
-    auto k = k_cols_dft<N, P, W>;
-    const size_t smem = ColDftShape<N, P, W>::SMEM;
+    using CS = ColDftShape<512, P, 16>;
+    auto k = k_cols_dft<P>;
+    const size_t smem = CS::SMEM;
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    k<<<dim3(N / W, a.nc), kBlock, smem, st>>>(a);
+    k<<<dim3(512 / 16, a.nc), kBlock, smem, st>>>(a);
     return cudaGetLastError();
 }
-
 
 // ---------------------------------------------------------------------------------------------
 // Row transform of the tensor-core gridding's tile-major field as N1 x N2 (8 x 64 on the 512 grid,
@@ -1054,7 +1052,7 @@ bool cols_dft_width_forced() { return getenv("MOFF_COLS_W") != nullptr; }
 
 cudaError_t launch_cols_dft(int N, int P, int W, const ColDftArgs &a, cudaStream_t st) {
     if (W == 16) {
-        if (N == 512) return P == 1 ? launch_cols_dft_t<512, 1, 16>(a, st) : launch_cols_dft_t<512, 2, 16>(a, st);
+        if (N == 512) return P == 1 ? launch_cols_dft_t<1>(a, st) : launch_cols_dft_t<2>(a, st);
         if (N == 256) return P == 1 ? launch_cols_pipe_t<256, 1, 16>(a, st) : launch_cols_pipe_t<256, 2, 16>(a, st);
     } else {
         if (N == 512) return P == 1 ? launch_cols_pipe_t<512, 1, 8>(a, st) : launch_cols_pipe_t<512, 2, 8>(a, st);

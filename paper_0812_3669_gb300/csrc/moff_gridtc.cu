@@ -105,8 +105,8 @@ __global__ void __launch_bounds__(kGtThreads, 1)
     if (warp == kGtEpiWarps) {
         // ---------------- producer (the whole warp runs it, one elected lane issues): the tile's kernel matrix B by
         // one bulk copy (completing on b_full), then chunk after chunk into the ring, one box of both planes
-        // per 64-sample half completing on a_full.  The chunks' plane rows stay in the lanes' registers (a tile has
-        // at most kp_max / 32 <= 20 chunks) and ring slot and phase are counted, not divided out.
+        // per 64-sample half completing on a_full.  The chunks' plane rows stay in the lanes' registers (B fits
+        // shared memory beside the ring, so a tile has at most 28 chunks) and ring slot and phase are counted, not divided out.
         const uint32_t one = tc::elect_one();
         if (one) {
             tc::mbar_arrive_expect_tx(b_full, bbytes_item);
@@ -122,7 +122,7 @@ __global__ void __launch_bounds__(kGtThreads, 1)
             for (int ch = 0; ch < nchunk; ++ch, ++g) {
                 if (!(ok = tc::mbar_wait_warp(&a_empty[st], ph, kGtWaitCycles, abort_flag))) break;
                 const uint32_t sa = tc::smem_u32(sA) + (uint32_t)(st * kGtStageBytes);
-                const int y = y0 + (ch < 32 ? __shfl_sync(0xffffffffu, row_l, ch) : a.chunk_row[ch0 + ch]);
+                const int y = y0 + __shfl_sync(0xffffffffu, row_l, ch);
                 tc::mbar_expect_tx_warp(one, &a_full[st], kGtStageBytes);
                 tc::tma_load_3d_warp(one, sa, &amap, t0b, y, 0, &a_full[st]);
                 tc::tma_load_3d_warp(one, sa + kGtHalfBytes, &amap, t0b + 64, y, 0, &a_full[st]);

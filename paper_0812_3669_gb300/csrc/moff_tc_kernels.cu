@@ -458,7 +458,7 @@ __global__ void __launch_bounds__(kTcRoleThreads, 1)
             for (int ch = 0; ch < nchunk; ++ch, ++g) {
                 if (!(ok = tc::mbar_wait_warp(&a_empty[st], ph, kWaitCycles, abort_flag))) break;
                 const uint32_t sa = tc::smem_u32(sA) + (uint32_t)(st * kAChunkBytes);
-                const int y = y0 + (ch < 32 ? __shfl_sync(0xffffffffu, row_l, ch) : a.chunk_row[ch0 + ch]);
+                const int y = y0 + __shfl_sync(0xffffffffu, row_l, ch);
                 tc::mbar_expect_tx_warp(one, &a_full[st], kAChunkBytes);
                 tc::tma_load_3d_warp(one, sa, &amap, t0b, y, 0, &a_full[st]);
                 tc::tma_load_3d_warp(one, sa + kAHalfBytes, &amap, t0b + 64, y, 0, &a_full[st]);
