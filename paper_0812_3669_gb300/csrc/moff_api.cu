@@ -434,10 +434,10 @@ void destroy_plan(moff_plan *pl) {
     delete pl;
 }
 
-// Polls without pause for the first 0.2 ms and then lets any other thread that is ready have the core between two polls; a
-// wait longer than 20 ms goes on with pauses, so it does not occupy a core.  A pause of 50 us ends about 100 us later, and
-// even finer ones (timer slack of 1 ns) or the event's interrupt (cudaEventBlockingSync) end a wait 35 to 75 us late: half
-// of a tiny array's block, 1 to 6 % of blocks of 2 to 4 ms, and 0.5 % of the shortest wait that sees them here.
+// Polls without pause for the first 20 ms; a longer wait goes on with pauses, so it does not occupy a core.  A pause of 50 us
+// ends about 100 us later, and even finer ones (timer slack of 1 ns) or the event's interrupt (cudaEventBlockingSync) end a
+// wait 35 to 75 us late: half of a tiny array's block, 1 to 6 % of blocks of 2 to 4 ms, and 0.5 % of the shortest wait that
+// sees them here.  (Yielding the core between polls made blocks of 2 ms take 8 on a machine with all cores busy.)
 moff_status wait_event(cudaEvent_t ev, int timeout_ms) {
     const auto t0 = std::chrono::steady_clock::now();
     for (;;) {
@@ -447,7 +447,6 @@ moff_status wait_event(cudaEvent_t ev, int timeout_ms) {
         const auto us = std::chrono::duration_cast<std::chrono::microseconds>(std::chrono::steady_clock::now() - t0).count();
         if (timeout_ms >= 0 && us >= 1000LL * timeout_ms) return fail(MOFF_ETIMEDOUT, "GPU work not finished after %d ms", timeout_ms);
         if (us > 20000) std::this_thread::sleep_for(std::chrono::microseconds(50));
-        else if (us > 200) std::this_thread::yield();
     }
 }
 
