@@ -242,6 +242,10 @@ moff_status moff_grid_snapshot(moff_plan *plan, const uint8_t *volt, int on_devi
  *   reset      1: zero the accumulators after reading.
  *   timeout_ms bounded wait for outstanding work (< 0: wait without limit);
  *              on expiry MOFF_ETIMEDOUT and nothing is read or reset.
+ * A pixel's power is summed in FP32 over a chunk of at most 128 samples and in
+ * FP64 across chunks.  Plans of few channels share a chunk's FP32 sum among
+ * several CTAs, added in a fixed order: a plan's image is reproducible, but the
+ * same channel in plans of different channel counts can differ in FP32 rounding.
  */
 moff_status moff_read_image(moff_plan *plan, float *out, long long *n_samples, int reset,
                             int timeout_ms, int out_on_device);

@@ -1064,7 +1064,7 @@ moff_status build_bins(int A, int K, int N, int P, bool jones, const double *pos
                     }
                 }
             }
-    // Stripe shape: F = TB * P * rows rows are transformed together.  Prefer
+    // Stripe shapes of fr = TB * P * rows rows transformed together.  Prefer
     // kernel entries staged in shared memory, then more samples per pass.
     // The built-in rule takes cell pairs unless MOFF_GRID_PAIRS=0.
     const char *pairs_env = getenv("MOFF_GRID_PAIRS");
@@ -1073,43 +1073,43 @@ moff_status build_bins(int A, int K, int N, int P, bool jones, const double *pos
     const bool quads = force ? force->quads : (quads_env && atoi(quads_env) != 0);
     const bool pairs = !quads && (force ? force->pairs : !(pairs_env && atoi(pairs_env) == 0));
     struct Cand { int tb, rows, nloc; long long entries; size_t sm_staged, sm_plain; };
-    auto shapes = [&](int F, std::initializer_list<int> tbs) {
-    std::vector<Cand> cands;
-    for (int tb : tbs) {
-        int rows = F / (tb * P);
-        if (rows < 1) continue;
-        rows = std::min(rows, N);
-        const int ns = N / rows;
-        std::vector<int> nloc(ns, 0), seen(ns, -1);
-        for (int a = 0; a < A; ++a)
-            for (int iy = 0; iy < K; ++iy) {
-                const int s = ((ay[a] + iy - h + N) % N) / rows;
-                if (seen[s] != a) { seen[s] = a; nloc[s]++; }
+    auto shapes = [&](int fr, std::initializer_list<int> tbs) {
+        std::vector<Cand> cands;
+        for (int tb : tbs) {
+            int rows = fr / (tb * P);
+            if (rows < 1) continue;
+            rows = std::min(rows, N);
+            const int ns = N / rows;
+            std::vector<int> nloc(ns, 0), seen(ns, -1);
+            for (int a = 0; a < A; ++a)
+                for (int iy = 0; iy < K; ++iy) {
+                    const int s = ((ay[a] + iy - h + N) % N) / rows;
+                    if (seen[s] != a) { seen[s] = a; nloc[s]++; }
+                }
+            const int mnl = std::max(1, *std::max_element(nloc.begin(), nloc.end()));
+            if ((long long)mnl * P >= 65536) continue;
+            long long ment = 0;
+            std::vector<int> c((size_t)P * rows * N);
+            for (int s = 0; s < ns; ++s) {
+                size_t n = 0;
+                for (int po = 0; po < P; ++po)
+                    for (int rl = 0; rl < rows; ++rl)
+                        for (int x = 0; x < N; ++x) c[n++] = cnt_all[((size_t)po * N + s * rows + rl) * N + x];
+                if (pairs)   // a pair's joint list is at most the sum of its two cells' lists
+                    for (size_t k = 0; k < c.size() / 2; ++k) c[k] = c[2 * k] + c[2 * k + 1];
+                const size_t nu = pairs ? c.size() / 2 : c.size();
+                std::sort(c.begin(), c.begin() + nu, [](int x, int y) { return x > y; });
+                long long e = 0;
+                for (size_t k = 0; k < nu; k += 32) e += 32LL * c[k];
+                ment = std::max(ment, e);
             }
-        const int mnl = std::max(1, *std::max_element(nloc.begin(), nloc.end()));
-        if ((long long)mnl * P >= 65536) continue;
-        long long ment = 0;
-        std::vector<int> c((size_t)P * rows * N);
-        for (int s = 0; s < ns; ++s) {
-            size_t n = 0;
-            for (int po = 0; po < P; ++po)
-                for (int rl = 0; rl < rows; ++rl)
-                    for (int x = 0; x < N; ++x) c[n++] = cnt_all[((size_t)po * N + s * rows + rl) * N + x];
-            if (pairs)   // a pair's joint list is at most the sum of its two cells' lists
-                for (size_t k = 0; k < c.size() / 2; ++k) c[k] = c[2 * k] + c[2 * k + 1];
-            const size_t nu = pairs ? c.size() / 2 : c.size();
-            std::sort(c.begin(), c.begin() + nu, [](int x, int y) { return x > y; });
-            long long e = 0;
-            for (size_t k = 0; k < nu; k += 32) e += 32LL * c[k];
-            ment = std::max(ment, e);
+            Cand cd{tb, rows, mnl, ment,
+                    dft ? (size_t)1 << 40
+                        : grid_smem_bytes(N, P, tb, rows, mnl, tw_total, (int)std::min<long long>(ment, 1 << 28), pairs),
+                    dft ? grid_smem_bytes_dft(N, P, tb, rows, mnl) : grid_smem_bytes(N, P, tb, rows, mnl, tw_total, 0, pairs)};
+            cands.push_back(cd);
         }
-        Cand cd{tb, rows, mnl, ment,
-                dft ? (size_t)1 << 40
-                    : grid_smem_bytes(N, P, tb, rows, mnl, tw_total, (int)std::min<long long>(ment, 1 << 28), pairs),
-                dft ? grid_smem_bytes_dft(N, P, tb, rows, mnl) : grid_smem_bytes(N, P, tb, rows, mnl, tw_total, 0, pairs)};
-        cands.push_back(cd);
-    }
-    return cands;
+        return cands;
     };
     std::vector<Cand> cands;
     // Entries are read through L2 by default (more CTAs per SM measured faster

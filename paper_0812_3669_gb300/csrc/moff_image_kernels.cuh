@@ -502,8 +502,9 @@ __host__ __device__ constexpr size_t col_smem_bytes_t(int P, bool h16 = false) {
     return (size_t)((FftTw<N>::TOTAL + 1) & ~1) * 8 + tile * (h16 ? 4 : 8) * 2 + tile * 8 * (FP::NP == 3 ? 2 : 1);
 }
 // Bytes of one CTA's sums, and the parts that a launch's samples are split into: short of CTAs, a cluster of up to eight
-// shares a strip's samples (at least eight each), up to four CTAs per SM.  FP32 fields split only where a persistent
-// launch, which gives the same image, has room for the sums of the parts before beside its tiles.
+// shares a strip's samples (at least eight each), up to four CTAs per SM (of 152).  FP32 fields split only where a persistent
+// launch, which gives the same image, has room for the sums of the parts before beside its tiles.  The parts, and so the
+// grouping of a pixel's FP32 sums, follow the launch's channels and samples: always the same for one plan and block length.
 template <int N>
 __host__ __device__ constexpr size_t col_sums_bytes_t(int P) { return (size_t)(P == 1 ? 1 : 4) * ColShape<N>::RL * kBlock * 4; }
 template <int N, int P, bool H16>
@@ -783,7 +784,8 @@ __device__ __forceinline__ void cols_acc(const ColArgs &a, const int sx, const i
 // instruction for both pols; scalar rotations and products were a third of the instructions before), the passes
 // exchange 16-byte elements, and XX, YY are one packed sum.  The field's elements go straight from global memory into
 // the registers of the first pass, S samples a round so that all threads have a slot, loaded one round ahead -- no
-// staging tiles, so two or three CTAs share an SM where the 512 grid had one.
+// staging tiles, so two CTAs share an SM on the 512 grid where there was one (118 to 128 registers); on the 256 grid the
+// two 16-point passes take 202 to 240 registers and one CTA of eight warps has the SM.
 struct Pol2 {
     float2 re, im;   // (x, y)
 };
@@ -1003,7 +1005,8 @@ __device__ __forceinline__ void cols_pol(const ColArgs &a, const int sx, const i
 // The FP16 field's two-pass columns (N = 32, 64, 128; two pols in step) with the passes on different warps: threads
 // 0-127 copy sample t + 1's strip (cp.async) and run the first pass of sample t, threads 128-255 the last pass and
 // the products of sample t - 1, one barrier a sample.  Each half needs only its own registers (16 values, or the sums),
-// so two CTAs fit an SM without spills, and one half's arithmetic covers the other's waits.  Bound by FP32 arithmetic.
+// so two CTAs fit an SM at 128 registers (spilling at most 16 bytes a thread on the 64 grid, 92 to 144 on the 128 grid), and
+// one half's arithmetic covers the other's waits.  Bound by FP32 arithmetic.
 template <int N, bool TAPS, int MODE>
 __device__ __forceinline__ void cols_duo(const ColArgs &a, const int sx, const int cl) {
     using FP = FftPlan<N>;

@@ -65,14 +65,14 @@ def test_power_of_two_gains_scale_exactly(monkeypatch, shift):
     assert np.array_equal(b, np.ldexp(a, 2 * shift))
 
 
-@pytest.mark.parametrize("P", [1, 2])
-def test_hand_overs_hold_over_full_waves(monkeypatch, P):
+@pytest.mark.parametrize("N,P,C", [(256, 1, 64), (256, 2, 64), (512, 1, 16), (512, 2, 16)])
+def test_hand_overs_hold_over_full_waves(monkeypatch, N, P, C):
     """One pol of one stage-1 tile (the 256 grid at 8 columns per CTA) leaves four of the twiddle warps without
-    rows; they must not stand in for the four that write the operand.  Thirteen or more waves of CTAs, blocks of
-    four launches of 128 samples, repeated: the images equal each other bit for bit, and those of 16 columns per CTA,
-    whose twiddle warps all have rows and whose arithmetic and order of sums are the same."""
+    rows; they must not stand in for the four that write the operand.  Several waves of CTAs, blocks of
+    four launches of 128 samples, repeated: the images equal each other bit for bit, and those of 16 columns per CTA (on
+    the 512 grid a kernel of its own, without roles), whose arithmetic and order of sums are the same."""
     monkeypatch.setenv("MOFF_TC_DFT", "1")
-    N, C, T = 256, 64, 512
+    T = 512
     pos, taps, codes, gains = case(5 + P, 90, N, P, C, T)
     dev = torch.from_numpy(codes).cuda()
     images = {}
