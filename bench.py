@@ -7,8 +7,7 @@ jitter; 512 x 256 cells, so x wraps the 512 grid), full pol with per-antenna
 9x9 kernels whose taps are 2x2 Jones matrices (seeded smooth beam, leakage and
 a non-coplanar w-phase), 4096 channels, 512 x 512 grid, integrations of 4000
 samples accumulated in FP64 across blocks.  It runs on the FP16 tensor-core
-path (the factored-DFT route: FP32 gridding, both transform axes as tcgen05
-contractions).  One step = one block of 128 samples of every channel =
+path (gridding and both transform axes as tcgen05 contractions).  One step = one block of 128 samples of every channel =
 524,288 channel-snapshots; its 34 GB of voltages are far larger than L2, so
 no flush is needed between steps.
 
