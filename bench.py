@@ -7,9 +7,9 @@ jitter; 512 x 256 cells, so x wraps the 512 grid), full pol with per-antenna
 9x9 kernels whose taps are 2x2 Jones matrices (seeded smooth beam, leakage and
 a non-coplanar w-phase), 4096 channels, 512 x 512 grid, integrations of 4000
 samples accumulated in FP64 across blocks.  It runs on the FP16 tensor-core
-path (gridding and both transform axes as tcgen05 contractions).  One step = one block of 128 samples of every channel =
-524,288 channel-snapshots; its 34 GB of voltages are far larger than L2, so
-no flush is needed between steps.
+path (gridding and both transform axes as tcgen05 contractions).  One step =
+one block of 128 samples of every channel = 524,288 channel-snapshots; its 34
+GB of voltages are far larger than L2, so no flush is needed between steps.
 
 Named legs: the same array on the FP32 path; the 16384-antenna filled-aperture
 precision workload (512 grid, 7x7 kernels, FP16 tensor-core and FP32); the
@@ -18,8 +18,8 @@ the FP16 row-spectrum route, feedback calibration, beams, channel sets,
 oversampling); serving and batching.
 
 Prints one JSON line (rank 0); the details of the legs and kernels are a JSON
-line on stderr.  ``--impl reference`` times the FP64 CPU
-oracle on a bounded sample of the headline workload instead.
+line on stderr.  ``--impl reference`` times the FP64 CPU oracle on a bounded
+sample of the headline workload instead.
 """
 from __future__ import annotations
 
